@@ -181,7 +181,9 @@ struct gsr_saved {
     int64_t rec_cap = 0, inst_cap = 0, row_cap = 0;   // visible records, kept instances, kept tile rows
     int64_t lb_pre_words = 0, lb_dup_words = 0;
     DevMem rec, vis_key, sorted_k, vis_aux, kstart, tile_key, tile_val, ranges, tfinal, ncontrib, wmask, ctrl;
-    DevMem open_tiles, depthpos;         // two-round lists: open-tile bits, record depth positions
+    // two-round lists: open-tile bits with the open blocks' behind them, record
+    // depth positions, per-tile statistics scratch
+    DevMem open_tiles, depthpos, tile_need;
     // Two-round lists.  prefix: the first round's record fraction of the
     // last forward (1: one round); region2: where its second list region
     // starts (-1: one region).
@@ -465,6 +467,9 @@ static float choose_prefix(const unsigned long long* H, const unsigned long long
     return best_b < kSatBuckets && best <= kTake * one ? (float)sat_edge(best_b) : 1.0f;
 }
 
+// Words of a bit array over n tiles (or blocks).
+static size_t open_words(int64_t n) { return (size_t)((std::max<int64_t>(n, 1) + 31) / 32); }
+
 static gsr_status size_saved(gsr_ctx* ctx, gsr_saved* s, const Table& T)
 {
     cudaError_t e;
@@ -492,14 +497,16 @@ static gsr_status size_saved(gsr_ctx* ctx, gsr_saved* s, const Table& T)
     if ((e = s->tile_key.ensure((size_t)span * 4)) != cudaSuccess) return cuda_fail(ctx, e, "alloc tile keys");
     if ((e = s->tile_val.ensure((size_t)span * 4)) != cudaSuccess) return cuda_fail(ctx, e, "alloc tile vals");
     if (two) {
-        if ((e = s->open_tiles.ensure((size_t)((std::max<int64_t>(T.n_tiles, 1) + 31) / 32) * 4)) != cudaSuccess)
+        if ((e = s->open_tiles.ensure(4 * (open_words(T.n_tiles) + open_words(4 * T.n_tiles)))) != cudaSuccess)
             return cuda_fail(ctx, e, "alloc open tiles");
+        if ((e = s->tile_need.ensure((size_t)std::max<int64_t>(T.n_tiles, 1) * 8)) != cudaSuccess)
+            return cuda_fail(ctx, e, "alloc tile statistics");
         if ((e = s->depthpos.ensure((size_t)rc * 4)) != cudaSuccess) return cuda_fail(ctx, e, "alloc depth positions");
     }
     if ((e = s->ranges.ensure((size_t)std::max<int64_t>(T.n_tiles, 1) * 8)) != cudaSuccess) return cuda_fail(ctx, e, "alloc ranges");
     if ((e = s->tfinal.ensure((size_t)T.n_pixels * 4)) != cudaSuccess) return cuda_fail(ctx, e, "alloc tfinal");
     if ((e = s->ncontrib.ensure((size_t)T.n_pixels * 4)) != cudaSuccess) return cuda_fail(ctx, e, "alloc ncontrib");
-    if ((e = s->wmask.ensure((size_t)span)) != cudaSuccess) return cuda_fail(ctx, e, "alloc warp masks");
+    if ((e = s->wmask.ensure(blend_mask_bytes(span, T.n_tiles))) != cudaSuccess) return cuda_fail(ctx, e, "alloc warp masks");
     s->lb_pre_words = std::max<int64_t>(preprocess_blocks(T), 1);
     s->lb_dup_words = std::max<int64_t>(duplicate_blocks(rc), 1);
     const size_t ctrl = kCtrlHead + 8 * (size_t)(s->lb_pre_words + 2 * s->lb_dup_words);
@@ -564,7 +571,7 @@ static void enqueue_forward(gsr_ctx* ctx, gsr_saved* s, const gsr_gaussians* g, 
     const bool two = prefix < 1.0f;
     s->prefix = prefix;
     s->region2 = two ? region2_start(s->inst_cap) : -1;
-    if (two) cudaMemsetAsync(s->open_tiles.p, 0, (size_t)((std::max<int64_t>(T.n_tiles, 1) + 31) / 32) * 4, st);
+    if (two) cudaMemsetAsync(s->open_tiles.p, 0, 4 * (open_words(T.n_tiles) + open_words(4 * T.n_tiles)), st);
     // the automatic fraction's statistics (depth positions, the two
     // histograms): taken by forwards that synchronise, the only ones whose
     // statistics are read back
@@ -580,13 +587,16 @@ static void enqueue_forward(gsr_ctx* ctx, gsr_saved* s, const gsr_gaussians* g, 
     ba.alpha = out->alpha;
     ba.tfinal = s->tfinal.as<float>();
     ba.ncontrib = s->ncontrib.as<uint32_t>();
-    ba.wmask = s->wmask.as<uint8_t>();
+    ba.wmask = s->wmask.as<uint32_t>();
+    ba.region2 = two ? (uint32_t)s->region2 : 0xffffffffu;
     ba.status = status;
     ba.counters = counters;
-    ba.wait_ns = ctx->wait_ns;
     ba.count_pairs = !(ctx->cfg.flags & GSR_FLAG_NO_PAIR_COUNTS);
     ba.prefix = prefix;
     ba.open_tiles = two ? s->open_tiles.as<uint32_t>() : nullptr;
+    ba.open_blocks = two ? ba.open_tiles + open_words(T.n_tiles) : nullptr;
+    ba.tile_need = hist ? s->tile_need.as<uint2>() : nullptr;
+    if (hist) cudaMemsetAsync(s->tile_need.p, 0, (size_t)std::max<int64_t>(T.n_tiles, 1) * 8, st);
     ba.depthpos = hist ? s->depthpos.as<uint32_t>() : nullptr;
     ba.hist = hist ? reinterpret_cast<unsigned long long*>(ctrl + kCtrlSatHist) : nullptr;
     // each list round (r = 0 alone, or r = 1 then r = 2): emission into the
@@ -637,7 +647,7 @@ static void enqueue_forward(gsr_ctx* ctx, gsr_saved* s, const gsr_gaussians* g, 
         ba.round = r;
         ba.work = reinterpret_cast<unsigned int*>(ctrl + (second ? kCtrlWorkFwd2 : kCtrlWorkFwd));
         prof_mark(pr, m0 + 3, st);
-        launch_blend_fwd(T, s->batch, ba, ctx->num_sms, st);
+        launch_blend_fwd(T, ba, ctx->num_sms, st);
         prof_mark(pr, m0 + 4, st);
     }
 }
@@ -880,7 +890,8 @@ gsr_status gsr_backward(gsr_ctx* ctx, const gsr_gaussians* g, const gsr_view* vi
     bb.ranges = s->ranges.as<uint2>();
     bb.tfinal = s->tfinal.as<float>();
     bb.ncontrib = s->ncontrib.as<uint32_t>();
-    bb.wmask = s->wmask.as<uint8_t>();
+    bb.wmask = s->wmask.as<uint32_t>();
+    bb.region2 = s->region2 >= 0 ? (uint32_t)s->region2 : 0xffffffffu;
     bb.dl_rgb = dl_drgb;
     bb.dl_depth = dl_ddepth;
     bb.dl_alpha = dl_dalpha;
@@ -1575,7 +1586,7 @@ gsr_status gsr_forward_noalloc(const gsr_config* cfg, const gsr_gaussians* g, co
     ba.status = status;
     ba.counters = counters;
     ba.count_pairs = !(cfg->flags & GSR_FLAG_NO_PAIR_COUNTS);
-    launch_blend_fwd(T, cfg->blend_batch, ba, num_sms, st);
+    launch_blend_fwd(T, ba, num_sms, st);
     if (cudaGetLastError() != cudaSuccess) return GSR_ERR_CUDA;
 
     // the instance count is only known on the device: read the status word

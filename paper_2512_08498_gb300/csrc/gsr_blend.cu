@@ -1,22 +1,22 @@
 // gsr_blend.cu -- per-pixel compositing (forward) and its adjoint (backward).
 //
-// One persistent launch covers every (view, tile) of the batch: each CTA
-// takes the next global tile from an atomic counter, so views of uneven size
-// and tiles of uneven list length share one grid of (SMs x resident CTAs).
-// A CTA has one thread per pixel (256 = tile_w x tile_h, warps laid out as
-// 8x4 pixel blocks).  The tile's sorted list is walked in batches of BATCH
-// records; each batch is gathered into shared memory with one bulk async copy
-// (cp.async.bulk, the TMA engine) per record (64 bytes; the backward stages
-// only the 48 it reads), completing on an mbarrier, double-buffered so the
-// gather of batch b+1 overlaps the arithmetic of batch b.
+// One persistent launch per direction covers every (view, tile) of the batch:
+// work comes from an atomic tile counter, so views of uneven size and tiles of
+// uneven list length share one grid of (SMs x resident blocks).  A tile has
+// 256 pixels.  The forward gives an 8x8 pixel block to a warp that waits for
+// no other (see below); the backward gives the tile to a block of eight warps
+// over 8x4 pixels each and walks the list in batches of BATCH records, each
+// gathered into shared memory with one bulk async copy (cp.async.bulk, the TMA
+// engine) per record (the 48 bytes it reads), completing on an mbarrier,
+// double-buffered so the gather of batch b+1 overlaps the arithmetic of batch b.
 //
-// Warp culling: every record carries a conservative box outside which its
+// Culling: every record carries a conservative box outside which its
 // binary32 alpha is certainly below 1/255 (see alpha_box in
-// gsr_preprocess.cu).  After a batch lands, each record's box is tested
-// against the eight warps' 8x4 pixel blocks, and each warp walks only the
-// entries that can touch its pixels, in list order.  Skipped pairs would
-// have been skipped by the 1/255 rule anyway, so every decision (blend, skip,
-// stop, contributor count) is unchanged.
+// gsr_preprocess.cu) and a threshold of its exponent.  A forward warp walks only
+// the entries that can touch its block, in list order, and records which 8x4
+// halves composited each entry; the backward walks exactly those.  Skipped
+// pairs would have been skipped by the 1/255 rule anyway, so every decision
+// (blend, skip, stop, contributor count) is unchanged.
 //
 // Forward, front to back (binary32 decisions per the contract):
 //   P2 = dx (qa dx + qb dy) + qc dy^2           (= log2 of the Gaussian)
@@ -85,77 +85,400 @@ __device__ __forceinline__ float rect_max_form(float x0, float x1, float y0, flo
     return fmaxf(p1, p2);
 }
 
-// Bit w of mask[t]: record t can reach alpha >= 1/255 at a pixel centre of
-// warp w.  Two conservative tests: the record's alpha box against the warp's
+// ---------------------------------------------------------------------------
+// forward
+// ---------------------------------------------------------------------------
+// One warp renders one 8x8 pixel block of a tile, two horizontally adjacent
+// pixels per lane, and nothing in it waits for another warp.  The tile's list
+// is walked in chunks of 32 entries.  Per chunk: the records (64 bytes each)
+// arrive by asynchronous copies issued one chunk ahead; each lane tests one
+// entry against the block (alpha box, then the maximum of the exponent over the
+// block); the survivors' walk values are written densely to shared memory; the
+// walk evaluates each survivor at the lane's two pixels.
+//
+// Bound by instruction issue (about 90 % of the slots; DRAM idle).  Against one
+// pixel per lane with the tile's eight 8x4 warps in step (a barrier per 256
+// staged entries, 82 % of the slots): a record's loads, dy and the row's products
+// serve two pixels, the barriers and the batch bookkeeping are gone, and a block
+// stops fetching as soon as its own pixels have stopped; it walks more idle
+// lanes (8x8 blocks composite 69 % of the walked lanes on the 1M-Gaussian
+// six-camera rig, 8x4 blocks 77 %).  Rig 2.04 -> 1.63 ms, 30-view window (with
+// pair counters) 9.8 -> 7.35 ms, 60-view road 29.1 -> 21.6 ms.  Packed pairs
+// (fma.rn.f32x2 over the two pixels) take the issue slots of the two scalar
+// operations on this part and need their operands twice: 1.69 ms on the rig.
+constexpr int kFwdWarps = 4;            // warps per block (they share nothing)
+constexpr int kFwdThreads = 32 * kFwdWarps;
+constexpr int kChunk = 32;              // list entries per step: one per lane
+constexpr int kBlk = 8;                 // the pixel block's side
+constexpr int kBlocksPerTile = kBlendThreads / (kBlk * kBlk);
+
+// A surviving record as the walk reads it.
+struct DenseRec {
+    float4 q[3];   // {u, v, qa, qb}, {qc, sigma, r, g}, {b, z, -, -}
+};
+
+struct FwdSmem {
+    float4 raw[2][kChunk][4];        // staged records, 16-byte pieces swizzled (see raw_piece)
+    DenseRec dense[kChunk];          // the chunk's survivors
+    uint8_t entry[kChunk];           // a survivor's position in the chunk
+    uint2 own;                       // see next_block
+    unsigned long long stat[3];      // the warp's walked entries, examined and composited pairs
+};
+
+// Piece q of lane l's record: lanes l and l + 2 would otherwise meet in a bank.
+__device__ __forceinline__ int raw_piece(int l, int q) { return q ^ ((l >> 1) & 3); }
+
+__device__ __forceinline__ void stage_record(float4* dst, const float4* src, int lane)
+{
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst + raw_piece(lane, q))), "l"(src + q)
+                     : "memory");
+}
+
+// Whether a record can reach alpha >= 1/255 at a pixel centre of the block at
+// (X0, Y0).  Two conservative tests: the record's alpha box against the
 // block, then the maximum of the record's exponent over the block against
 // its culling threshold (record slot 11).  The corner offsets are rounded
 // exactly as the blend rounds each pixel's offset, so every pixel's rounded
 // offset lies in the tested rectangle.
-template <int BX, int BY>
-__device__ __forceinline__ void warp_masks(const float4* B, int cnt, int tx0, int ty0, uint8_t* s_mask)
+__device__ __forceinline__ bool block_hit(const float4& r0, float qc, float thr_cull, const float4& bb, float X0, float Y0)
 {
-    using TS = TileShape<BX, BY>;
-    for (int t = threadIdx.x; t < cnt; t += kBlendThreads) {
-        const float4 r0 = B[4 * t];
-        const float qc = B[4 * t + 1].x;
-        const float thr_cull = B[4 * t + 2].w;
-        const float4 bb = B[4 * t + 3];
+    bool hit = bb.x <= X0 + (kBlk - 0.5f) && bb.y >= X0 + 0.5f && bb.z <= Y0 + (kBlk - 0.5f) && bb.w >= Y0 + 0.5f;
+    if (hit && thr_cull > -3.0e38f) {
         const float kx = -r0.w / (2.0f * r0.z), ky = -r0.w / (2.0f * qc);
-        uint32_t m = 0;
-#pragma unroll 1
-        for (int w = 0; w < kWarps; ++w) {
-            const float X0 = (float)(tx0 + (w % TS::WPR) * TS::WX);
-            const float Y0 = (float)(ty0 + (w / TS::WPR) * TS::WY);
-            bool hit = bb.x <= X0 + (TS::WX - 0.5f) && bb.y >= X0 + 0.5f && bb.z <= Y0 + (TS::WY - 0.5f) &&
-                       bb.w >= Y0 + 0.5f;
-            if (hit && thr_cull > -3.0e38f) {
-                const float x0 = __fsub_rn(__fadd_rn(X0, 0.5f), r0.x);
-                const float x1 = __fsub_rn(__fadd_rn(X0, TS::WX - 0.5f), r0.x);
-                const float y0 = __fsub_rn(__fadd_rn(Y0, 0.5f), r0.y);
-                const float y1 = __fsub_rn(__fadd_rn(Y0, TS::WY - 0.5f), r0.y);
-                hit = rect_max_form(x0, x1, y0, y1, r0.z, r0.w, qc, kx, ky) >= thr_cull;
-            }
-            m |= (uint32_t)hit << w;
-        }
-        s_mask[t] = (uint8_t)m;
+        const float x0 = __fsub_rn(__fadd_rn(X0, 0.5f), r0.x);
+        const float x1 = __fsub_rn(__fadd_rn(X0, kBlk - 0.5f), r0.x);
+        const float y0 = __fsub_rn(__fadd_rn(Y0, 0.5f), r0.y);
+        const float y1 = __fsub_rn(__fadd_rn(Y0, kBlk - 0.5f), r0.y);
+        hit = rect_max_form(x0, x1, y0, y1, r0.z, r0.w, qc, kx, ky) >= thr_cull;
     }
+    return hit;
 }
 
-// This warp's entries of the batch, in list order; returns their number.
-__device__ __forceinline__ int warp_list(const uint8_t* s_mask, int cnt, int w, int lane, uint16_t* list)
-{
-    int nl = 0;
-    const uint32_t lt = (1u << lane) - 1u;
-    for (int base = 0; base < cnt; base += 32) {
-        const int t = base + lane;
-        const bool bit = t < cnt && ((s_mask[t] >> w) & 1u);
-        const uint32_t bal = __ballot_sync(0xffffffffu, bit);
-        if (bit) list[nl + __popc(bal & lt)] = (uint16_t)t;
-        nl += __popc(bal);
-    }
-    __syncwarp();
-    return nl;
-}
-
-// One (pixel, entry) pair of the forward up to alpha (independent of T).
+// One entry at a lane's two pixels (same row, so dy and its products are
+// equal) up to alpha (independent of T).  2^P2 is the contract's exp2_nonpos
+// bit for bit wherever a pixel can composite: the upper clamp (P2 <= 0) is
+// left out because the entry is refused there anyway, and the final scaling by
+// 2^n adds n to the exponent field, which differs from the product only below
+// 2^-126, far under the 1/255 threshold.
 struct FwdPair {
-    int k;
-    float P2, al;
-    float4 c;      // colour, depth
+    float P0, P1;      // P2 at the two pixels
+    float al0, al1;
+    float r, g, b, z;  // colour, depth
 };
 
-__device__ __forceinline__ FwdPair fwd_pair(const float4* B, int k, float pxf, float pyf)
+__device__ __forceinline__ float exp2_walk(float P)
+{
+    const float y = fmaxf(P, -126.0f);
+    const float j = __fadd_rn(y, 0x1.8p23f);
+    const float f = __fsub_rn(y, __fsub_rn(j, 0x1.8p23f));
+    return __int_as_float(__float_as_int(exp2_poly(f)) + (__float_as_int(j) << 23));
+}
+
+__device__ __forceinline__ FwdPair fwd_pair(const DenseRec& d, float px0, float px1, float py)
 {
     FwdPair e;
-    e.k = k;
-    const float4 r0 = B[4 * k];
-    const float4 r1 = B[4 * k + 1];
-    const float4 r2 = B[4 * k + 2];
-    const float dx = __fsub_rn(pxf, r0.x), dy = __fsub_rn(pyf, r0.y);
-    e.P2 = __fmaf_rn(dx, __fmaf_rn(r0.z, dx, __fmul_rn(r0.w, dy)), __fmul_rn(__fmul_rn(r1.x, dy), dy));
-    e.al = fminf(GSR_ALPHA_MAX, __fmul_rn(r1.y, exp2_nonpos(fminf(e.P2, 0.0f))));
-    e.c = make_float4(r2.x, r2.y, r2.z, r1.z);
+    const float4 q0 = d.q[0], q1 = d.q[1];
+    const float2 q2 = *reinterpret_cast<const float2*>(&d.q[2]);
+    const float dx0 = __fsub_rn(px0, q0.x), dx1 = __fsub_rn(px1, q0.x), dy = __fsub_rn(py, q0.y);
+    const float t = __fmul_rn(q0.w, dy), s = __fmul_rn(__fmul_rn(q1.x, dy), dy);
+    e.P0 = __fmaf_rn(dx0, __fmaf_rn(q0.z, dx0, t), s);
+    e.P1 = __fmaf_rn(dx1, __fmaf_rn(q0.z, dx1, t), s);
+    e.al0 = fminf(GSR_ALPHA_MAX, __fmul_rn(q1.y, exp2_walk(e.P0)));
+    e.al1 = fminf(GSR_ALPHA_MAX, __fmul_rn(q1.y, exp2_walk(e.P1)));
+    e.r = q1.z; e.g = q1.w; e.b = q2.x; e.z = q2.y;
     return e;
+}
+
+// The next pixel block of a warp.  The warps of a block of threads share one
+// tile's blocks (state: tile << 32 | next block), so the records a warp
+// stages are mostly in L1 for the other three (the 65M-record road gathers from
+// 4 GB: with independent warps its forward took 37 ms, 22 ms with the sharing).  A warp that finds the tile
+// exhausted takes a new one from the global queue and installs it; if another
+// warp installed one meanwhile, it renders its own tile alone.  No warp waits.
+__device__ __forceinline__ uint2 next_block(unsigned long long* shared, uint2* own, unsigned int* work)
+{
+    const uint2 o = *own;   // a tile held alone: {tile, next block}
+    if (o.y < kBlocksPerTile) {
+        own->y = o.y + 1u;
+        return o;
+    }
+    for (;;) {
+        const unsigned long long old = *reinterpret_cast<volatile unsigned long long*>(shared);
+        const unsigned int b = (unsigned int)old;
+        if (b < kBlocksPerTile) {
+            if (atomicCAS(shared, old, old + 1ull) == old) return make_uint2((unsigned int)(old >> 32), b);
+            continue;
+        }
+        const unsigned int t = atomicAdd(work, 1u);
+        if (atomicCAS(shared, old, ((unsigned long long)t << 32) | 1ull) != old) *own = make_uint2(t, 1u);
+        return make_uint2(t, 0u);
+    }
+}
+
+// First 32-bit word of a tile's composited-entry masks: kMaskWords words per
+// chunk of 32 list positions, word 2 blk + h the entries that some pixel of
+// the upper (h = 0) or lower 8x4 half of block blk composited.  A tile's
+// chunks start at its range's first position / 32 plus the tile id (plus the
+// tile count in the second list region), so no two tiles' words overlap:
+// floor((x + n) / 32) - floor(x / 32) + 1 >= ceil(n / 32).
+constexpr int kMaskWords = 2 * kBlocksPerTile;
+__device__ __forceinline__ size_t mask_base(uint32_t first, uint32_t tile, uint32_t region2, int64_t n_tiles)
+{
+    return (size_t)kMaskWords * ((size_t)(first / kChunk) + tile + (first >= region2 ? (size_t)n_tiles : (size_t)0));
+}
+
+// COUNT: keep the per-pixel examined and composited counts (statistics only;
+// a separate instantiation because the running counts lengthen the walk).
+// 80 registers, six blocks per SM (at 72 the walk spills: 6 % slower).
+template <int BX, bool COUNT>
+__global__ void __launch_bounds__(kFwdThreads, 6)
+blend_fwd_kernel(const __grid_constant__ Table Tb, BlendFwdArgs a)
+{
+    if (earlier_wait_timed_out(a.status)) return;
+    constexpr int BY = kBlendThreads / BX, BPR = BX / kBlk;   // blocks per tile row
+    __shared__ __align__(128) FwdSmem s_warp[kFwdWarps];
+    __shared__ unsigned long long s_queue;
+    if (threadIdx.x == 0) s_queue = (unsigned long long)kBlocksPerTile;   // no tile
+    const int lane = threadIdx.x & 31;
+    FwdSmem& S = s_warp[threadIdx.x >> 5];
+    if (lane == 0) {
+        S.own = make_uint2(0u, kBlocksPerTile);
+        S.stat[0] = S.stat[1] = S.stat[2] = 0ull;
+    }
+    __syncthreads();
+    if (a.round == 2 && a.counters[kCntOpenTiles] == 0ull) return;
+    bool prefix_all = false;   // the first round's lists are the full ones
+    if (a.round == 1) {
+        const int64_t n_vis = (int64_t)a.counters[kCntVisible];
+        prefix_all = prefix_records(n_vis, a.prefix) == n_vis;
+    }
+    const uint32_t lt_mask = (1u << lane) - 1u;
+
+    for (;;) {
+        uint2 next = make_uint2(0u, 0u);
+        if (lane == 0) next = next_block(&s_queue, &S.own, a.work);
+        const unsigned int tile = __shfl_sync(0xffffffffu, next.x, 0), blk = __shfl_sync(0xffffffffu, next.y, 0);
+        if ((int64_t)tile >= Tb.n_tiles) break;
+        if (a.round == 2 && !((a.open_tiles[tile >> 5] >> (tile & 31u)) & 1u)) continue;
+        const int view = find_view_of_tile(Tb, tile);
+        const DevView& V = Tb.v[view];
+        const int lt = (int)(tile - V.tile_base);
+        const int bx0 = (lt % V.TX) * BX + (int)(blk % BPR) * kBlk, by0 = (lt / V.TX) * BY + (int)(blk / BPR) * kBlk;
+        const int px = bx0 + 2 * (lane & 3), py = by0 + (lane >> 2);
+        const uint2 rg = a.ranges[tile];
+        const int n = (int)(rg.y - rg.x);
+        const float fx = __fadd_rn((float)px, 0.5f), fy = __fadd_rn((float)py, 0.5f);
+        const float fx1 = __fadd_rn(fx, 1.0f);
+        float Cr0 = 0.0f, Cr1 = 0.0f, Cg0 = 0.0f, Cg1 = 0.0f, Cb0 = 0.0f, Cb1 = 0.0f, D0 = 0.0f, D1 = 0.0f;
+        // transmittance, negated once the pixel has stopped (or if it lies
+        // outside the image): a negative T passes no stop test, so nothing more
+        // is composited
+        float T0 = py < V.H && px < V.W ? 1.0f : -1.0f, T1 = py < V.H && px + 1 < V.W ? 1.0f : -1.0f;
+        uint32_t last0 = 0, last1 = 0, exam0 = (uint32_t)n, exam1 = (uint32_t)n, nblend = 0;
+        auto all_stopped = [&]() { return __all_sync(0xffffffffu, T0 < 0.0f && T1 < 0.0f); };
+        // list positions up to the end of the chunk in which every pixel had
+        // stopped (0: they did not)
+        int satpos = 0;
+        unsigned int walked = 0;
+        uint2* words = a.wmask ? reinterpret_cast<uint2*>(a.wmask + mask_base(rg.x, tile, a.region2, Tb.n_tiles)) + blk
+                               : nullptr;
+        const uint32_t* vals = a.vals + rg.x;
+        bool all = all_stopped();   // a block outside the image
+
+        uint32_t kn = 0;   // record of this lane's entry of the next chunk
+        if (lane < n) stage_record(S.raw[0][lane], a.rec + 4 * (size_t)vals[lane], lane);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        if (kChunk + lane < n) kn = vals[kChunk + lane];
+        for (int c0 = 0; c0 < n && !all; c0 += kChunk) {
+            const int s = (c0 / kChunk) & 1;
+            if (c0 + kChunk + lane < n) stage_record(S.raw[s ^ 1][lane], a.rec + 4 * (size_t)kn, lane);
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            if (c0 + 2 * kChunk + lane < n) kn = vals[c0 + 2 * kChunk + lane];
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            // each lane reads the record it staged itself
+            const float4* R = S.raw[s][lane];
+            bool hit = false, indefinite = false;
+            float4 r0, r1, r2;
+            if (c0 + lane < n) {
+                r0 = R[raw_piece(lane, 0)];
+                r1 = R[raw_piece(lane, 1)];
+                r2 = R[raw_piece(lane, 2)];
+                hit = block_hit(r0, r1.x, r2.w, R[raw_piece(lane, 3)], (float)bx0, (float)by0);
+                indefinite = hit && !(r2.w > -3.0e38f);
+            }
+            const uint32_t hits = __ballot_sync(0xffffffffu, hit);
+            const int m = __popc(hits), rank = __popc(hits & lt_mask);
+            if (hit) {
+                DenseRec& d = S.dense[rank];
+                float4* q = reinterpret_cast<float4*>(&d);
+                q[0] = r0;
+                q[1] = make_float4(r1.x, r1.y, r2.x, r2.y);
+                q[2] = make_float4(r2.z, r1.z, 0.0f, 0.0f);
+                S.entry[rank] = (uint8_t)lane;
+            } else if ((m & 1) && lane == 31 - __clz(~hits)) {
+                // an odd survivor count is padded with a record that composites
+                // nowhere (sigma = 0); m is odd, so some lane is no hit
+                float4* q = reinterpret_cast<float4*>(&S.dense[m]);
+#pragma unroll
+                for (int i = 0; i < 3; ++i) q[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            }
+            __syncwarp();
+            // Branch-free: after exact culling nearly every walked entry
+            // composites somewhere in the block, so every lane evaluates it and
+            // the decisions select the updates (a zero weight leaves C and D
+            // bit-identical).  Entries are taken two at a time: the second's
+            // alpha does not depend on T, so it overlaps the first's update.
+            // Bit p of w0 / w1: the pixel composited the chunk's survivor p.
+            uint32_t w0 = 0, w1 = 0, x0 = 0, x1 = 0, bit = 1u;
+            const bool live0 = T0 > 0.0f, live1 = T1 > 0.0f;
+            // TEST_P: whether P2 > 0 has to be tested.  A record with a culling
+            // threshold has a negative definite form of condition below 1e5,
+            // whose binary32 value is within 8 2^-24 cond < 5 % of the exact one
+            // and so never positive.
+            auto step = [&](const FwdPair& e, uint32_t b, auto TEST_P) {
+                const float n0 = __fmul_rn(T0, __fsub_rn(1.0f, e.al0)), n1 = __fmul_rn(T1, __fsub_rn(1.0f, e.al1));
+                const bool pass0 = (!TEST_P.value || e.P0 <= 0.0f) && e.al0 >= GSR_ALPHA_MIN;
+                const bool pass1 = (!TEST_P.value || e.P1 <= 0.0f) && e.al1 >= GSR_ALPHA_MIN;
+                const bool bl0 = pass0 && n0 >= GSR_T_STOP, bl1 = pass1 && n1 >= GSR_T_STOP;
+                const float g0 = bl0 ? e.al0 * T0 : 0.0f, g1 = bl1 ? e.al1 * T1 : 0.0f;
+                Cr0 = fmaf(e.r, g0, Cr0); Cr1 = fmaf(e.r, g1, Cr1);
+                Cg0 = fmaf(e.g, g0, Cg0); Cg1 = fmaf(e.g, g1, Cg1);
+                Cb0 = fmaf(e.b, g0, Cb0); Cb1 = fmaf(e.b, g1, Cb1);
+                D0 = fmaf(e.z, g0, D0); D1 = fmaf(e.z, g1, D1);
+                if constexpr (COUNT) {
+                    if (pass0 && !bl0) x0 |= b;
+                    if (pass1 && !bl1) x1 |= b;
+                }
+                if (pass0) T0 = bl0 ? n0 : -fabsf(T0);
+                if (pass1) T1 = bl1 ? n1 : -fabsf(T1);
+                if (bl0) w0 |= b;
+                if (bl1) w1 |= b;
+            };
+            int i = 0;
+            auto walk = [&](auto TEST_P) {
+                while (i < m && !all) {
+                    // the warp vote that ends the walk once every pixel has
+                    // stopped is taken after every fourth pair (a stopped pixel
+                    // passes nothing, so the extra entries change no result)
+                    const int e = min(i + 8, m);
+                    for (; i < e; i += 2) {
+                        const FwdPair e0 = fwd_pair(S.dense[i], fx, fx1, fy);
+                        const FwdPair e1 = fwd_pair(S.dense[i + 1], fx, fx1, fy);
+                        step(e0, bit, TEST_P);
+                        step(e1, bit << 1, TEST_P);
+                        bit <<= 2;
+                    }
+                    all = all_stopped();
+                }
+            };
+            if (__any_sync(0xffffffffu, indefinite)) walk(std::true_type{});
+            else walk(std::false_type{});
+            walked += (unsigned)min(i, m);
+            // a pixel's last composited entry is the highest set bit; one OR
+            // over each half of the warp says which survivors some pixel of its
+            // 8x4 half composited, spread back to the chunk's positions
+            if (w0) last0 = (uint32_t)(c0 + S.entry[31 - __clz(w0)] + 1);
+            if (w1) last1 = (uint32_t)(c0 + S.entry[31 - __clz(w1)] + 1);
+            if constexpr (COUNT) {
+                // the lowest bit of x0 / x1: the entry that stopped the pixel
+                if (live0 && x0) exam0 = (uint32_t)(c0 + S.entry[__ffs(x0) - 1] + 1);
+                if (live1 && x1) exam1 = (uint32_t)(c0 + S.entry[__ffs(x1) - 1] + 1);
+                nblend += __popc(w0) + __popc(w1);
+            }
+            if (words) {
+                const uint32_t own = w0 | w1;
+                const uint32_t up = __reduce_or_sync(0xffffffffu, lane < 16 ? own : 0u);
+                const uint32_t lo = __reduce_or_sync(0xffffffffu, lane < 16 ? 0u : own);
+                const uint32_t mu = __ballot_sync(0xffffffffu, hit && ((up >> rank) & 1u));
+                const uint32_t ml = __ballot_sync(0xffffffffu, hit && ((lo >> rank) & 1u));
+                if (lane == 0) words[(size_t)(c0 / kChunk) * kBlocksPerTile] = make_uint2(mu, ml);
+            }
+            __syncwarp();   // the dense records are rewritten by the next chunk
+            if (all) satpos = min(c0 + kChunk, n);
+        }
+        // no copy is left in flight into the buffers the next block stages
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        // A first round's tile is final when its pixels all stopped within
+        // the prefix lists (or those were the full lists); otherwise the
+        // second round renders it again over its full list.
+        const bool saturated = all;
+        const bool final_block = a.round != 1 || saturated || prefix_all;
+        if (lane == 0) {
+            if (!final_block) {
+                const size_t item = (size_t)tile * kBlocksPerTile + blk;
+                atomicOr(a.open_blocks + (item >> 5), 1u << (item & 31u));
+                const uint32_t bit = 1u << (tile & 31u);
+                if (!(atomicOr(a.open_tiles + (tile >> 5), bit) & bit)) atomicAdd(a.counters + kCntOpenTiles, 1ull);
+            }
+            if (a.hist) {
+                // the tile's last block records the share of the depth-ordered
+                // records the tile needed before every pixel stopped, weighted
+                // by its (estimated full) list length
+                uint2* need = a.tile_need + tile;   // {largest satpos, blocks that finished}
+                const uint32_t never = 0xffffffffu;
+                atomicMax(&need->x, saturated ? (uint32_t)satpos : never);
+                __threadfence();
+                if (atomicAdd(&need->y, 1u) == kBlocksPerTile - 1) {
+                    const uint32_t most = atomicMax(&need->x, 0u);
+                    const unsigned long long n_vis = a.counters[kCntVisible];
+                    int bucket = kSatBuckets;
+                    if (most != never && most > 0u && n_vis > 0ull) {
+                        const uint32_t k = vals[most - 1];
+                        bucket = sat_bucket((float)(a.depthpos[k] + 1u) / (float)n_vis);
+                    }
+                    unsigned long long len = (unsigned long long)n;
+                    if (a.round == 1) {
+                        const unsigned long long n_pre = (unsigned long long)prefix_records((int64_t)n_vis, a.prefix);
+                        if (n_pre > 0ull) len = len * n_vis / n_pre;
+                    }
+                    const bool open = a.round == 1 && most == never && !prefix_all;
+                    if (len && !open) atomicAdd(a.hist + bucket, len);
+                    *need = make_uint2(0u, 0u);   // for a second round
+                }
+            }
+        }
+        if (!final_block) continue;
+        // statistics are taken by the round that finishes the block
+        const size_t item = (size_t)tile * kBlocksPerTile + blk;
+        if (a.round != 2 || ((a.open_blocks[item >> 5] >> (item & 31u)) & 1u)) {
+            if (lane == 0) S.stat[0] += walked;
+            if constexpr (COUNT) {
+                unsigned long long exam = 0;
+                if (py < V.H && px < V.W) exam += exam0;
+                if (py < V.H && px + 1 < V.W) exam += exam1;
+                exam = warp_sum(exam);
+                nblend = __reduce_add_sync(0xffffffffu, nblend);
+                if (lane == 0) {
+                    S.stat[1] += exam;
+                    S.stat[2] += nblend;
+                }
+            }
+        }
+        if (py < V.H) {
+            const int64_t hw = (int64_t)V.W * V.H;
+            const int64_t off = (int64_t)py * V.W + px;
+            const int64_t pix = V.pix_base + off;
+            float* rgb = a.rgb + 3 * V.pix_base;
+            auto put = [&](int64_t o, float T, float C0, float C1, float C2, float Dz, uint32_t last) {
+                rgb[off + o] = C0 + T * Tb.bg[0];
+                rgb[hw + off + o] = C1 + T * Tb.bg[1];
+                rgb[2 * hw + off + o] = C2 + T * Tb.bg[2];
+                a.depth[pix + o] = Dz;
+                a.alpha[pix + o] = 1.0f - T;
+                a.tfinal[pix + o] = T;
+                a.ncontrib[pix + o] = last;
+            };
+            if (px < V.W) put(0, fabsf(T0), Cr0, Cg0, Cb0, D0, last0);
+            if (px + 1 < V.W) put(1, fabsf(T1), Cr1, Cg1, Cb1, D1, last1);
+        }
+    }
+    if (lane == 0) {
+        if (S.stat[0]) atomicAdd(a.counters + kCntWarpFwd, 2ull * S.stat[0]);   // in units of 32 pixels
+        if (S.stat[1]) atomicAdd(a.counters + kCntFwdPairs, S.stat[1]);
+        if (S.stat[2]) atomicAdd(a.counters + kCntBlended, S.stat[2]);
+    }
 }
 
 // Backward reduction over a warp's 32 pixels, transposed.  For each walked
@@ -259,246 +582,6 @@ __device__ __forceinline__ void slots_reduce(const float* __restrict__ sgp, cons
         atomicAdd(sg + 8, v[8]);
         atomicAdd(sg + 9, v[9]);
     }
-}
-
-// four blocks per SM: 64 registers (the two-entry walk would otherwise take
-// 72 and leave room for three).  COUNT: keep the per-pixel examined and
-// composited counts (statistics only; a separate instantiation because the
-// two running counts cost about 6 % of the walk).
-template <int BX, int BY, int BATCH, bool COUNT>
-__global__ void __launch_bounds__(kBlendThreads, 4)
-blend_fwd_kernel(const __grid_constant__ Table Tb, BlendFwdArgs a)
-{
-    if (earlier_wait_timed_out(a.status)) return;
-    using TS = TileShape<BX, BY>;
-    extern __shared__ __align__(128) float4 s_buf[];     // [2][BATCH][4]
-    __shared__ __align__(8) uint64_t s_bar[2];
-    __shared__ unsigned int s_item;
-    __shared__ uint8_t s_mask[BATCH];
-    __shared__ uint16_t s_list[kWarps][BATCH];
-    __shared__ __align__(16) uint8_t s_wb[kWarps][BATCH]; // per warp: composited each entry of the batch
-    // per tile (kept in shared memory, off the walk's registers): the warps'
-    // walked entries, and the list entries up to the end of the batch in
-    // which every pixel had stopped (0: they did not)
-    __shared__ unsigned int s_witer[kWarps];
-    __shared__ int s_satpos;
-    __shared__ int s_prefix_all;   // the first round's lists are the full ones
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    if (tid == 0) {
-        mbar_init(&s_bar[0], 1);
-        mbar_init(&s_bar[1], 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        const int64_t n_vis = (int64_t)a.counters[kCntVisible];
-        s_prefix_all = prefix_records(n_vis, a.prefix) == n_vis;
-    }
-    for (int t = tid; t < kWarps * BATCH / 4; t += kBlendThreads) reinterpret_cast<uint32_t*>(&s_wb[0][0])[t] = 0u;
-    __syncthreads();
-    uint32_t par0 = 0u, par1 = 0u;
-    const int lx = TS::lx(tid), ly = TS::ly(tid);
-    unsigned long long exam_total = 0, blended_total = 0;
-    unsigned int witer = 0;
-    bool failed = false;
-    uint16_t* L = s_list[w];
-    if (a.round == 2 && a.counters[kCntOpenTiles] == 0ull) return;
-
-    for (;;) {
-        if (tid == 0) s_item = atomicAdd(a.work, 1u);
-        __syncthreads();
-        const unsigned int item = s_item;
-        __syncthreads();
-        if ((int64_t)item >= Tb.n_tiles || failed) break;
-        if (a.round == 2 && !((a.open_tiles[item >> 5] >> (item & 31u)) & 1u)) continue;
-        if (lane == 0) s_witer[w] = 0u;
-        if (tid == 0) s_satpos = 0;
-        const int view = find_view_of_tile(Tb, item);
-        const DevView& V = Tb.v[view];
-        const int lt = (int)(item - V.tile_base);
-        const int tx0 = (lt % V.TX) * BX, ty0 = (lt / V.TX) * BY;
-        const int px = tx0 + lx, py = ty0 + ly;
-        const bool inside = px < V.W && py < V.H;
-        const uint2 rg = a.ranges[item];
-        const int n = (int)(rg.y - rg.x);
-        const int nb = (n + BATCH - 1) / BATCH;
-        const float pxf = __fadd_rn((float)px, 0.5f), pyf = __fadd_rn((float)py, 0.5f);
-        float T = 1.0f, C0 = 0.0f, C1 = 0.0f, C2 = 0.0f, D = 0.0f;
-        uint32_t last = 0, exam = (uint32_t)n, nblend = 0;
-        bool done = !inside;
-
-        if (nb > 0) issue_batch<4>(a.vals, a.rec, rg.x, min(BATCH, n), s_buf, &s_bar[0], nullptr);
-        for (int b = 0; b < nb; ++b) {
-            const int s = b & 1;
-            if (b + 1 < nb)
-                issue_batch<4>(a.vals, a.rec, rg.x + (b + 1) * BATCH, min(BATCH, n - (b + 1) * BATCH),
-                            s_buf + (size_t)(s ^ 1) * BATCH * 4, &s_bar[s ^ 1], nullptr);
-            const bool ok = mbar_wait_bounded(&s_bar[s], s ? par1 : par0, a.status, a.wait_ns);
-            if (s) par1 ^= 1u; else par0 ^= 1u;
-            if (__syncthreads_or(!ok)) {
-                failed = true;
-                if (b + 1 < nb) mbar_wait_bounded(&s_bar[s ^ 1], s ? par0 : par1, a.status, a.wait_ns);
-                break;
-            }
-            const int cnt = min(BATCH, n - b * BATCH);
-            const float4* B = s_buf + (size_t)s * BATCH * 4;
-            warp_masks<BX, BY>(B, cnt, tx0, ty0, s_mask);
-            __syncthreads();
-            const int nl = warp_list(s_mask, cnt, w, lane, L);
-            // Structured body and a warp vote per entry: the vote reconverges
-            // the warp every iteration (lanes would otherwise drift apart under
-            // independent thread scheduling) and ends the batch for the warp
-            // once all of its pixels are done.
-            if (!__all_sync(0xffffffffu, done)) {
-                // Branch-free: after exact culling nearly every walked entry
-                // composites somewhere in the warp, so every lane evaluates it
-                // and the decisions select the updates (a zero weight leaves C
-                // and D bit-identical).  Entries are taken two at a time: the
-                // second's alpha does not depend on T, so it overlaps the
-                // first's update; the warp vote that ends the walk once every
-                // pixel has stopped is taken after every second pair (a done
-                // pixel passes nothing, so the extra entries change no result).
-                // Returns whether this pixel composited the entry.
-                auto step = [&](const FwdPair& e) {
-                    const float Tn = __fmul_rn(T, __fsub_rn(1.0f, e.al));
-                    const bool pass = !done && e.P2 <= 0.0f && e.al >= GSR_ALPHA_MIN;
-                    const bool stop = pass && Tn < GSR_T_STOP;
-                    const bool blended_now = pass && !stop;
-                    const float wgt = blended_now ? e.al * T : 0.0f;
-                    C0 = fmaf(e.c.x, wgt, C0);
-                    C1 = fmaf(e.c.y, wgt, C1);
-                    C2 = fmaf(e.c.z, wgt, C2);
-                    D = fmaf(e.c.w, wgt, D);
-                    T = blended_now ? Tn : T;
-                    if constexpr (COUNT) {
-                        exam = stop ? (uint32_t)(b * BATCH + e.k + 1) : exam;
-                        nblend += blended_now ? 1u : 0u;
-                    }
-                    done = done || stop;
-                    return blended_now;
-                };
-                // Bit p of a lane's wb is its own decision for the p-th entry of
-                // a group of 32.  Per group: the pixel's last composited entry
-                // is the highest set bit, and one OR over the warp publishes
-                // which entries some pixel of the warp composited (entry
-                // L[i0 + l] by lane l).
-                auto publish = [&](uint32_t wb, int i0, int cnt) {
-                    if (wb) last = (uint32_t)(b * BATCH + L[i0 + 31 - __clz(wb)] + 1);
-                    const uint32_t any = __reduce_or_sync(0xffffffffu, wb);
-                    if (lane < cnt && ((any >> lane) & 1u)) s_wb[w][L[i0 + lane]] = 1;
-                };
-                int i = 0;
-                bool all = false;
-                // whole groups of 32 entries, bit positions fixed at compile time
-                for (; i + 32 <= nl; i += 32) {
-                    uint32_t wb = 0;
-                    int p = 0;
-#pragma unroll
-                    for (; p < 32; p += 2) {
-                        const FwdPair e0 = fwd_pair(B, L[i + p], pxf, pyf);
-                        const FwdPair e1 = fwd_pair(B, L[i + p + 1], pxf, pyf);
-                        if (step(e0)) wb |= 1u << p;
-                        if (step(e1)) wb |= 2u << p;
-                        if ((p & 2) && __all_sync(0xffffffffu, done)) { p += 2; all = true; break; }
-                    }
-                    publish(wb, i, p);
-                    if (all) { i += p; break; }
-                }
-                if (!all) {
-                    // the last (fewer than 32) entries
-                    uint32_t wb = 0;
-                    int p = 0;
-                    for (; i + p + 1 < nl; p += 2) {
-                        const FwdPair e0 = fwd_pair(B, L[i + p], pxf, pyf);
-                        const FwdPair e1 = fwd_pair(B, L[i + p + 1], pxf, pyf);
-                        if (step(e0)) wb |= 1u << p;
-                        if (step(e1)) wb |= 2u << p;
-                        if (__all_sync(0xffffffffu, done)) { p += 2; all = true; break; }
-                    }
-                    if (!all && i + p < nl) {
-                        if (step(fwd_pair(B, L[i + p], pxf, pyf))) wb |= 1u << p;
-                        ++p;
-                    }
-                    publish(wb, i, p);
-                    i += p;
-                }
-                if (lane == 0) s_witer[w] += (unsigned)i;
-            }
-            const bool all_done = __syncthreads_and(done);
-            // publish which warps composited each entry (the backward walks only those)
-            for (int t = tid; t < cnt; t += kBlendThreads) {
-                uint32_t m = 0;
-#pragma unroll
-                for (int ww = 0; ww < kWarps; ++ww) {
-                    m |= (uint32_t)s_wb[ww][t] << ww;
-                    s_wb[ww][t] = 0;
-                }
-                if (a.wmask) a.wmask[rg.x + (size_t)b * BATCH + t] = (uint8_t)m;
-            }
-            if (all_done) {
-                if (tid == 0) s_satpos = b * BATCH + cnt;
-                // drain the prefetched batch before leaving the tile
-                if (b + 1 < nb) {
-                    const bool ok2 = mbar_wait_bounded(&s_bar[s ^ 1], s ? par0 : par1, a.status, a.wait_ns);
-                    if (s) par0 ^= 1u; else par1 ^= 1u;
-                    if (__syncthreads_or(!ok2)) failed = true;
-                }
-                break;
-            }
-        }
-        // A first round's tile is final when its pixels all stopped within
-        // the prefix lists (or those were the full lists); otherwise the
-        // second round renders it again over its full list.
-        const bool saturated = __syncthreads_and(done);   // (also publishes s_witer and s_satpos)
-        const bool final_tile = a.round != 1 || saturated || s_prefix_all;
-        // (thread 0 re-reads the tile and its range: nothing of them stays
-        // live in registers across the walk)
-        if (!final_tile) {
-            if (tid == 0 && !failed) {
-                const unsigned int it = s_item;
-                atomicOr(a.open_tiles + (it >> 5), 1u << (it & 31u));
-                atomicAdd(a.counters + kCntOpenTiles, 1ull);
-            }
-            continue;
-        }
-        if (lane == 0) witer += s_witer[w];
-        if (tid == 0 && a.hist && !failed) {
-            // the share of the depth-ordered records the tile needed before
-            // every pixel stopped, weighted by its (estimated full) list length
-            const uint2 r = a.ranges[s_item];
-            const unsigned long long n_vis = a.counters[kCntVisible];
-            int bucket = kSatBuckets;
-            if (saturated && s_satpos > 0 && n_vis > 0ull) {
-                const uint32_t k = a.vals[r.x + s_satpos - 1];
-                bucket = sat_bucket((float)(a.depthpos[k] + 1u) / (float)n_vis);
-            }
-            unsigned long long len = r.y - r.x;
-            if (a.round == 1) {
-                const unsigned long long n_pre = (unsigned long long)prefix_records((int64_t)n_vis, a.prefix);
-                if (n_pre > 0ull) len = len * n_vis / n_pre;
-            }
-            if (len) atomicAdd(a.hist + bucket, len);
-        }
-        if (inside) {
-            const int64_t hw = (int64_t)V.W * V.H;
-            const int64_t off = (int64_t)py * V.W + px;
-            const int64_t pix = V.pix_base + off;
-            float* rgb = a.rgb + 3 * V.pix_base;
-            rgb[off] = C0 + T * Tb.bg[0];
-            rgb[hw + off] = C1 + T * Tb.bg[1];
-            rgb[2 * hw + off] = C2 + T * Tb.bg[2];
-            a.depth[pix] = D;
-            a.alpha[pix] = 1.0f - T;
-            a.tfinal[pix] = T;
-            a.ncontrib[pix] = last;
-            if constexpr (COUNT) {
-                exam_total += exam;
-                blended_total += nblend;
-            }
-        }
-    }
-    exam_total = warp_sum(exam_total);
-    blended_total = warp_sum(blended_total);
-    if (lane == 0 && exam_total) atomicAdd(a.counters + kCntFwdPairs, exam_total);
-    if (lane == 0 && blended_total) atomicAdd(a.counters + kCntBlended, blended_total);
-    if (lane == 0 && witer) atomicAdd(a.counters + kCntWarpFwd, (unsigned long long)witer);
 }
 
 // ---------------------------------------------------------------------------
@@ -639,12 +722,11 @@ blend_bwd_kernel(const __grid_constant__ Table Tb, BlendBwdArgs a)
         sdcd[lane] = make_float4(dC0, dC1, dC2, dD);   // read by the slot reduction (after __syncwarp)
         const float cxw = (float)(tx0 + (w % TS::WPR) * TS::WX + TS::WX / 2);
         const float cyw = (float)(ty0 + (w / TS::WPR) * TS::WY + TS::WY / 2);
-        {
-            uint32_t m = mylast;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-            if (lane == 0 && m) atomicMax(&s_maxlast, m);
-        }
+        const int warp_last = (int)__reduce_max_sync(0xffffffffu, mylast);
+        if (lane == 0 && warp_last) atomicMax(&s_maxlast, (uint32_t)warp_last);
+        // this warp's 8x4 block: half (w / WPR) & 1 of the forward's 8x8 block
+        const uint32_t* words = a.wmask + mask_base(rg.x, item, a.region2, Tb.n_tiles) +
+                                2 * ((w / TS::WPR / 2) * TS::WPR + w % TS::WPR) + ((w / TS::WPR) & 1);
         __syncthreads();
         const int maxlast = (int)s_maxlast;
         const int nb = (maxlast + BATCH - 1) / BATCH;
@@ -663,19 +745,12 @@ blend_bwd_kernel(const __grid_constant__ Table Tb, BlendBwdArgs a)
             const int s = q & 1;
             const int bb = nb - 1 - q;
             const int cnt = min(BATCH, maxlast - bb * BATCH);
-            // exactly the (warp, entry) pairs the forward composited: lane l
-            // holds the mask bytes of entries l + 32 j, read before the wait
-            uint32_t mw[(BATCH + 127) / 128];
-            {
-                const uint8_t* wm = a.wmask + rg.x + (size_t)bb * BATCH;
-#pragma unroll
-                for (int j = 0; j < (BATCH + 127) / 128; ++j) mw[j] = 0u;
-#pragma unroll
-                for (int j = 0; j < BATCH / 32; ++j) {
-                    const int t = lane + 32 * j;
-                    if (t < cnt) mw[j >> 2] |= (uint32_t)wm[t] << (8 * (j & 3));
-                }
-            }
+            // exactly the (warp, entry) pairs the forward composited: lane j
+            // holds the mask word of the batch's entries 32 j .., read before the
+            // wait (past the warp's last composited entry none was written)
+            uint32_t mword = 0u;
+            if (lane < BATCH / kChunk && bb * BATCH + kChunk * lane < warp_last)
+                mword = words[(size_t)(bb * (BATCH / kChunk) + lane) * kMaskWords];
             const bool ok = mbar_wait_bounded(&s_bar[s], s ? par1 : par0, a.status, a.wait_ns);
             if (s) par1 ^= 1u; else par0 ^= 1u;
             // (this barrier also orders the previous batch's flush before the
@@ -696,9 +771,8 @@ blend_bwd_kernel(const __grid_constant__ Table Tb, BlendBwdArgs a)
 #pragma unroll
                 for (int j = 0; j < BATCH / 32; ++j) {
                     if (32 * j < cnt) {
-                        const bool bit = (mw[j >> 2] >> (8 * (j & 3) + w)) & 1u;
-                        const uint32_t bal = __ballot_sync(0xffffffffu, bit);
-                        if (bit) L[nl + __popc(bal & lt)] = (ListT)(32 * j + lane);
+                        const uint32_t bal = __shfl_sync(0xffffffffu, mword, j);
+                        if ((bal >> lane) & 1u) L[nl + __popc(bal & lt)] = (ListT)(32 * j + lane);
                         nl += __popc(bal);
                     }
                 }
@@ -795,31 +869,30 @@ blend_bwd_kernel(const __grid_constant__ Table Tb, BlendBwdArgs a)
 // ---------------------------------------------------------------------------
 // dispatch
 // ---------------------------------------------------------------------------
-template <int BX, int BY, int BATCH, bool COUNT>
+template <int BX, bool COUNT>
 static void fwd_launch(const Table& T, const BlendFwdArgs& a, int num_sms, cudaStream_t s)
 {
-    auto kern = blend_fwd_kernel<BX, BY, BATCH, COUNT>;
-    const size_t smem = (size_t)2 * BATCH * kRecordBytes;
+    auto kern = blend_fwd_kernel<BX, COUNT>;
     // function attributes and occupancy are per device
     static std::atomic<int> per_sm_dev[kMaxDevices];
     const int per_sm = per_device_once(per_sm_dev, [&] {
         int n = 0;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kBlendThreads, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kFwdThreads, 0);
         return n < 1 ? 1 : n;
     });
     int64_t grid = (int64_t)num_sms * per_sm;
-    if (grid > T.n_tiles) grid = T.n_tiles;
+    const int64_t want = (T.n_tiles * kBlocksPerTile + kFwdWarps - 1) / kFwdWarps;
+    if (grid > want) grid = want;
     if (grid < 1) return;
     GSR_COUNT_LAUNCH();
-    kern<<<(unsigned)grid, kBlendThreads, smem, s>>>(T, a);
+    kern<<<(unsigned)grid, kFwdThreads, 0, s>>>(T, a);
 }
 
-template <int BX, int BY, int BATCH>
+template <int BX>
 static void fwd_one(const Table& T, const BlendFwdArgs& a, int num_sms, cudaStream_t s)
 {
-    if (a.count_pairs) fwd_launch<BX, BY, BATCH, true>(T, a, num_sms, s);
-    else fwd_launch<BX, BY, BATCH, false>(T, a, num_sms, s);
+    if (a.count_pairs) fwd_launch<BX, true>(T, a, num_sms, s);
+    else fwd_launch<BX, false>(T, a, num_sms, s);
 }
 
 template <int BX, int BY, int BATCH>
@@ -871,9 +944,17 @@ bool blend_supported(int tw, int th, int batch)
         }                                                                                        \
     } while (0)
 
-void launch_blend_fwd(const Table& T, int batch, const BlendFwdArgs& a, int num_sms, cudaStream_t s)
+// (the forward stages chunks of 32 entries per warp whatever the staging batch)
+void launch_blend_fwd(const Table& T, const BlendFwdArgs& a, int num_sms, cudaStream_t s)
 {
-    GSR_DISPATCH(fwd_one, T, batch, a, num_sms, s);
+    if (T.tile_w == 16) fwd_one<16>(T, a, num_sms, s);
+    else if (T.tile_w == 32) fwd_one<32>(T, a, num_sms, s);
+    else fwd_one<8>(T, a, num_sms, s);
+}
+
+size_t blend_mask_bytes(int64_t list_span, int64_t n_tiles)
+{
+    return ((size_t)(list_span / kChunk) + 2 * (size_t)n_tiles + 1) * kMaskWords * sizeof(uint32_t);
 }
 
 void launch_blend_bwd(const Table& T, int batch, const BlendBwdArgs& a, int num_sms, cudaStream_t s)

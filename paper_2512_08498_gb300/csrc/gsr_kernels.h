@@ -212,11 +212,11 @@ struct BlendFwdArgs {
     float* alpha;
     float* tfinal;
     uint32_t* ncontrib;
-    uint8_t* wmask;                // [inst_cap] bit w: warp w composited this list entry (may be nullptr)
-    unsigned int* work;            // zeroed tile counter
+    uint32_t* wmask;               // blend_mask_bytes: which 8x4 blocks composited each list entry (may be nullptr)
+    uint32_t region2 = 0xffffffffu;    // first list position of the second region (0xffffffff: one region)
+    unsigned int* work;            // zeroed block counter
     uint32_t* status;
     unsigned long long* counters;
-    uint64_t wait_ns = kWaitLimitNs;   // limit of each mbarrier wait
     bool count_pairs = true;       // examined and composited pair counters
     // Two-round lists.  round: 0 for a forward of one round; 1 for the
     // first of two, which renders the prefix lists (the first
@@ -228,6 +228,8 @@ struct BlendFwdArgs {
     int round = 0;
     float prefix = 1.0f;
     uint32_t* open_tiles = nullptr;
+    uint32_t* open_blocks = nullptr;        // the same per 8x8 pixel block (bit 4 tile + block)
+    uint2* tile_need = nullptr;             // with hist: [n_tiles] zeroed {largest position needed, blocks done}
     const uint32_t* depthpos = nullptr;     // with hist: record -> depth position
     unsigned long long* hist = nullptr;     // [kSatBuckets + 1] saturation histogram, or nullptr
 };
@@ -241,7 +243,8 @@ struct BlendBwdArgs {
     const float* dl_rgb;
     const float* dl_depth;         // may be nullptr
     const float* dl_alpha;         // may be nullptr
-    const uint8_t* wmask;          // written by the forward that filled the saved state
+    const uint32_t* wmask;         // written by the forward that filled the saved state
+    uint32_t region2 = 0xffffffffu;    // as in that forward
     float4* grad_rec;              // [n_vis][3], zeroed
     unsigned int* work;            // zeroed tile counter
     uint32_t* status;
@@ -250,7 +253,8 @@ struct BlendBwdArgs {
 };
 
 bool blend_supported(int tile_w, int tile_h, int batch);
-void launch_blend_fwd(const Table& T, int batch, const BlendFwdArgs& a, int num_sms, cudaStream_t s);
+void launch_blend_fwd(const Table& T, const BlendFwdArgs& a, int num_sms, cudaStream_t s);
+size_t blend_mask_bytes(int64_t list_span, int64_t n_tiles);   // composited-entry masks of a forward's lists
 void launch_blend_bwd(const Table& T, int batch, const BlendBwdArgs& a, int num_sms, cudaStream_t s);
 
 // ---- insertion probability (Sec. 3.2, Eq. 4-6) -------------------------------
