@@ -197,6 +197,9 @@ __device__ __forceinline__ FwdPair fwd_pair(const DenseRec& d, float px0, float 
 // 4 GB: with independent warps its forward took 37 ms, 22 ms with the sharing).  A warp that finds the tile
 // exhausted takes a new one from the global queue and installs it; if another
 // warp installed one meanwhile, it renders its own tile alone.  No warp waits.
+// (The first tile is installed for all: four warps that each took one left a
+// small image's tiles to a quarter of the blocks, 93 us instead of 31 on
+// 256 x 256 pixels.)
 __device__ __forceinline__ uint2 next_block(unsigned long long* shared, uint2* own, unsigned int* work)
 {
     const uint2 o = *own;   // a tile held alone: {tile, next block}
@@ -240,7 +243,7 @@ blend_fwd_kernel(const __grid_constant__ Table Tb, BlendFwdArgs a)
     constexpr int BY = kBlendThreads / BX, BPR = BX / kBlk;   // blocks per tile row
     __shared__ __align__(128) FwdSmem s_warp[kFwdWarps];
     __shared__ unsigned long long s_queue;
-    if (threadIdx.x == 0) s_queue = (unsigned long long)kBlocksPerTile;   // no tile
+    if (threadIdx.x == 0) s_queue = (unsigned long long)atomicAdd(a.work, 1u) << 32;   // the first tile
     const int lane = threadIdx.x & 31;
     FwdSmem& S = s_warp[threadIdx.x >> 5];
     if (lane == 0) {
