@@ -1,7 +1,8 @@
-"""The forward walks a tile's list in chunks of 32 entries per 8x8 pixel
-block: list lengths around the chunk edges, pixels that stop inside a chunk,
-image edges inside a block, and records whose form is too ill-conditioned for
-the culling threshold, against the oracle."""
+"""The blends walk a tile's list in chunks of 32 entries per 8x8 pixel block,
+the backward its composited entries in groups of eight: list lengths around
+those edges, pixels that stop inside a chunk, image edges inside a block, and
+records whose form is too ill-conditioned for the culling threshold, against
+the oracle."""
 import numpy as np
 import pytest
 
@@ -13,6 +14,7 @@ if not torch.cuda.is_available():  # pragma: no cover - CPU machines
 
 import oracle  # noqa: E402
 from paper_2512_08498_gb300 import scenes  # noqa: E402
+from paper_2512_08498_gb300.rasterizer import Rasterizer, to_camera_views  # noqa: E402
 
 import _parity as P  # noqa: E402
 
@@ -37,3 +39,31 @@ def test_list_lengths(n, logit, tile):
     P.compare_pixels(g, o, ref)
     P.compare_counters(g, o, ref, with_bwd=True)
     P.compare_images(g, ref)
+
+
+@pytest.mark.parametrize("tile", [(16, 16), (32, 8), (8, 32)])
+@pytest.mark.parametrize("depth", [False, True])
+@pytest.mark.parametrize("n,logit", [(1, 0.0), (7, -1.0), (8, -1.0), (9, -1.0), (16, 5.5), (31, -2.0), (32, -2.0),
+                                     (33, -2.0), (40, -2.5), (65, -3.0), (97, 3.0)])
+def test_backward_groups(n, logit, depth, tile):
+    # n entries that every pixel may composite (all of them at low opacity;
+    # at logit 5.5 the 0.99 clamp acts), with and without a depth gradient
+    views = [scenes.pinhole(21, 13, f=20.0), scenes.pinhole(9, 17, f=20.0)]
+    sc = scenes.random_scene(70 + n, n, views, 1, z_range=(2.0, 4.0), xy_half=0.3, log_scale_range=(-2.0, -0.5), tile=tile,
+                             bg=(0.2, 0.1, 0.4))
+    sc.opacity_logits[:] = logit
+    o = oracle.Oracle(sc, tile=tile)
+    ref = o.forward()
+    up_o, up_g = P.upstream(sc, o, ref, depth_w=0.05 if depth else 0.0)
+    dev = P.device()
+    r = Rasterizer(tile=tile, sh_degree=1, bg=sc.bg, device=dev)
+    params, cams = P.params_of(sc, dev), to_camera_views(sc.views, dev)
+    _, _, _, saved = r.forward(params, cams)
+    d_rgb, d_dep, d_alp = (torch.from_numpy(x).to(dev) for x in up_g)
+    grads = r.backward(params, cams, saved, d_rgb, d_dep if depth else None, d_alp, want_focal=True)
+    g = dict(info=saved.info(), grec=r.debug_record_grads(saved).cpu().numpy(),
+             grads={k: t.cpu().numpy().astype(np.float64) for k, t in zip(P.PARAM_NAMES + ["pose", "focal"], grads)})
+    assert g["info"]["bwd_pairs"] > 0
+    go = o.backward(up_o[0], up_o[1], up_o[2], want_grec=True)
+    P.compare_grads(g, go)
+    P.compare_record_grads(g, go)
