@@ -88,8 +88,26 @@ struct ProfRecord {
     bool pending = false;
 };
 
+// Saved states that were destroyed, kept for the next gsr_saved_create of their
+// context: a saved state holds about 17 device buffers and a pinned one, whose
+// allocation and release cost a forward that makes its own state (one per call
+// of the autograd function) 0.9 ms of the 1.2 ms of a 256 x 256 step.  At most
+// kPoolStates states of kPoolBytes together are kept; they go when the context
+// is destroyed or a device allocation fails.  Shared by the context and its
+// states, with a lock: a state may be destroyed from another host thread
+// (the autograd engine's) or after its context.
+struct SavedPool {
+    static constexpr size_t kPoolStates = 2, kPoolBytes = (size_t)2 << 30;
+    std::mutex m;
+    std::vector<gsr_saved*> states;
+    size_t bytes = 0;
+    bool closed = false;
+    void drain(bool close);
+};
+
 struct gsr_ctx {
     gsr_config cfg;
+    std::shared_ptr<SavedPool> pool = std::make_shared<SavedPool>();
     int device = 0;
     int num_sms = 0;
     std::string err;
@@ -115,6 +133,7 @@ struct gsr_ctx {
     float auto_prefix = 1.0f;
     ~gsr_ctx()
     {
+        pool->drain(true);
         for (auto& r : prof)
             for (auto& e : r.ev)
                 if (e) cudaEventDestroy(e);
@@ -190,8 +209,53 @@ struct gsr_saved {
     float prefix = 1.0f;
     int64_t region2 = -1;
     unsigned char* host_ctrl = nullptr;  // pinned mirror of the control block head
-    ~gsr_saved() { if (host_ctrl) cudaFreeHost(host_ctrl); }
+    // Recycling.  reusable: the state's only work is that of forwards and
+    // backwards on one stream outside a capture (anything else frees it when it
+    // is destroyed); done marks the end of that work (recorded when pending: the
+    // call did not wait for it), and the first forward of the state's next life
+    // waits for it.  grown: capacities inherited from an earlier life.
+    std::shared_ptr<SavedPool> pool;
+    bool reusable = false, pending = false, grown = false;
+    cudaStream_t last_stream = nullptr;
+    cudaEvent_t done = nullptr;
+    ~gsr_saved()
+    {
+        if (host_ctrl) cudaFreeHost(host_ctrl);
+        if (done) cudaEventDestroy(done);
+    }
+    size_t bytes() const
+    {
+        size_t n = 0;
+        for (const DevMem* d : {&rec, &vis_key, &sorted_k, &vis_aux, &kstart, &tile_key, &tile_val, &ranges, &tfinal,
+                                &ncontrib, &wmask, &ctrl, &open_tiles, &depthpos, &tile_need})
+            n += d->bytes;
+        return n;
+    }
+    // Work of this state was enqueued on `stream`; waited: and waited for.
+    void touched(cudaStream_t stream, bool waited)
+    {
+        if (pending && stream != last_stream) reusable = false;   // on two streams
+        last_stream = stream;
+        pending = !waited;
+        if (waited || !reusable) return;
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
+            cudaEventRecord(done, stream) != cudaSuccess)
+            reusable = false;
+    }
 };
+
+void SavedPool::drain(bool close)
+{
+    std::vector<gsr_saved*> v;
+    {
+        std::lock_guard<std::mutex> lock(m);
+        v.swap(states);
+        bytes = 0;
+        closed = closed || close;
+    }
+    for (gsr_saved* s : v) delete s;
+}
 
 static gsr_status fail(gsr_ctx* ctx, gsr_status code, const std::string& msg)
 {
@@ -287,18 +351,51 @@ gsr_status gsr_saved_create(gsr_ctx* ctx, gsr_saved** out)
 {
     if (!ctx || !out) return GSR_ERR_INVALID_ARG;
     *out = nullptr;
-    gsr_saved* s = new (std::nothrow) gsr_saved();
-    if (!s) return fail(ctx, GSR_ERR_OUT_OF_MEMORY, "saved state");
-    s->ctx = ctx;
+    gsr_saved* s = nullptr;
+    {
+        std::lock_guard<std::mutex> lock(ctx->pool->m);
+        if (!ctx->pool->states.empty()) {
+            s = ctx->pool->states.back();
+            ctx->pool->states.pop_back();
+            ctx->pool->bytes -= s->bytes();
+        }
+    }
+    if (s) {
+        s->batch = 256;
+        s->flags = 0;
+        s->filled = s->have_grads = false;
+        s->prefix = 1.0f;
+        s->region2 = -1;
+        s->grown = true;
+    } else {
+        s = new (std::nothrow) gsr_saved();
+        if (!s) return fail(ctx, GSR_ERR_OUT_OF_MEMORY, "saved state");
+        s->ctx = ctx;
+        cudaError_t e = cudaMallocHost((void**)&s->host_ctrl, kCtrlHead);
+        if (e != cudaSuccess) { delete s; return cuda_fail(ctx, e, "cudaMallocHost"); }
+        s->pool = ctx->pool;
+        s->reusable = cudaEventCreateWithFlags(&s->done, cudaEventDisableTiming) == cudaSuccess;
+    }
     std::memset(&s->table, 0, sizeof(Table));
-    cudaError_t e = cudaMallocHost((void**)&s->host_ctrl, kCtrlHead);
-    if (e != cudaSuccess) { delete s; return cuda_fail(ctx, e, "cudaMallocHost"); }
     std::memset(s->host_ctrl, 0, kCtrlHead);
     *out = s;
     return GSR_OK;
 }
 
-void gsr_saved_destroy(gsr_saved* s) { delete s; }
+void gsr_saved_destroy(gsr_saved* s)
+{
+    if (s && s->reusable) {
+        const size_t b = s->bytes();
+        std::lock_guard<std::mutex> lock(s->pool->m);
+        if (!s->pool->closed && s->pool->states.size() < SavedPool::kPoolStates &&
+            s->pool->bytes + b <= SavedPool::kPoolBytes) {
+            s->pool->states.push_back(s);
+            s->pool->bytes += b;
+            return;
+        }
+    }
+    delete s;
+}
 
 gsr_status gsr_saved_get_info(const gsr_saved* s, gsr_saved_info* info)
 {
@@ -473,17 +570,22 @@ static size_t open_words(int64_t n) { return (size_t)((std::max<int64_t>(n, 1) +
 static gsr_status size_saved(gsr_ctx* ctx, gsr_saved* s, const Table& T)
 {
     cudaError_t e;
-    if (s->rec_cap == 0) {
+    // (a recycled state has at least the capacities a new one starts with)
+    const bool grown = s->grown;
+    s->grown = false;
+    if (s->rec_cap == 0 || grown) {
         int64_t cap = T.n_records;
         if (cap > (64ll << 20)) cap = std::max<int64_t>(64ll << 20, cap / 3);
-        s->rec_cap = std::max<int64_t>(cap, 1);
+        s->rec_cap = std::max<int64_t>(s->rec_cap, std::max<int64_t>(cap, 1));
     }
-    if (s->inst_cap == 0) s->inst_cap = std::max<int64_t>(4 * s->rec_cap, 1 << 20);
+    if (s->inst_cap == 0 || grown) s->inst_cap = std::max<int64_t>(s->inst_cap, std::max<int64_t>(4 * s->rec_cap, 1 << 20));
     // the emission keeps two counts per record in the tile-sort destination
     // keys while they are free
     s->inst_cap = std::max<int64_t>(s->inst_cap, 2 * s->rec_cap);
     // a kept tile row holds >= 1 instance; rows are typically a third of them
-    if (s->row_cap == 0) s->row_cap = std::max<int64_t>(std::max<int64_t>(s->inst_cap / 2, 2 * s->rec_cap), 1 << 18);
+    if (s->row_cap == 0 || grown)
+        s->row_cap = std::max<int64_t>(s->row_cap,
+                                       std::max<int64_t>(std::max<int64_t>(s->inst_cap / 2, 2 * s->rec_cap), 1 << 18));
     const int64_t rc = s->rec_cap, ic = s->inst_cap;
     if ((e = s->rec.ensure((size_t)rc * kRecordBytes)) != cudaSuccess) return cuda_fail(ctx, e, "alloc records");
     if ((e = s->vis_key.ensure((size_t)rc * 4)) != cudaSuccess) return cuda_fail(ctx, e, "alloc keys");
@@ -751,13 +853,30 @@ gsr_status gsr_forward(gsr_ctx* ctx, const gsr_gaussians* g, const gsr_view* vie
     s->flags = ctx->cfg.flags;
     s->filled = false;
     s->have_grads = false;
+    // a recycled state's earlier work comes first
+    if (s->grown && s->pending) {
+        const cudaError_t e = cudaStreamWaitEvent(cs, s->done, 0);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "recycled state");
+        s->pending = false;
+    }
+    const bool reusable = s->reusable;
+    s->reusable = false;   // until this call has succeeded
     for (int attempt = 0; attempt < 4; ++attempt) {
-        if ((st = size_saved(ctx, s, T)) != GSR_OK) return st;
+        if ((st = size_saved(ctx, s, T)) == GSR_ERR_OUT_OF_MEMORY) {
+            (void)cudaGetLastError();
+            ctx->pool->drain(false);
+            st = size_saved(ctx, s, T);
+        }
+        if (st != GSR_OK) return st;
         enqueue_forward(ctx, s, g, out, cs);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(ctx, e, "forward launch");
         s->filled = true;
-        if (ctx->cfg.flags & GSR_FLAG_NO_SYNC) return GSR_OK;
+        if (ctx->cfg.flags & GSR_FLAG_NO_SYNC) {
+            s->reusable = reusable;
+            s->touched(cs, false);
+            return GSR_OK;
+        }
         uint32_t status = 0;
         if ((st = read_status(ctx, s, cs, &status)) != GSR_OK) return st;
         if (status & kErrTimeout) { s->filled = false; return fail(ctx, GSR_ERR_TIMEOUT, "device wait timed out"); }
@@ -765,6 +884,8 @@ gsr_status gsr_forward(gsr_ctx* ctx, const gsr_gaussians* g, const gsr_view* vie
         if (status & kErrInternal) { s->filled = false; return fail(ctx, GSR_ERR_CUDA, "internal consistency check failed"); }
         if (!(status & (kErrRecCapacity | kErrInstCapacity | kErrFullCapacity))) {
             update_auto_prefix(ctx, s);
+            s->reusable = reusable;
+            s->touched(cs, true);
             return GSR_OK;
         }
         const unsigned long long* c = reinterpret_cast<const unsigned long long*>(s->host_ctrl + kCtrlCounters);
@@ -845,10 +966,21 @@ gsr_status gsr_backward(gsr_ctx* ctx, const gsr_gaussians* g, const gsr_view* vi
     if (((uintptr_t)grads->quats & 15u) != 0) return fail(ctx, GSR_ERR_INVALID_ARG, "grad quats must be 16-byte aligned");
     const Table& T = s->table;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
-    cudaError_t e = ctx->grad_rec.ensure((size_t)s->rec_cap * kGradBytes);
+    auto ensure = [&](DevMem& m, size_t bytes) {
+        cudaError_t e = m.ensure(bytes);
+        if (e == cudaErrorMemoryAllocation) {
+            (void)cudaGetLastError();
+            ctx->pool->drain(false);
+            e = m.ensure(bytes);
+        }
+        return e;
+    };
+    cudaError_t e = ensure(ctx->grad_rec, (size_t)s->rec_cap * kGradBytes);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "alloc record gradients");
-    if ((e = ctx->bwd_queue.ensure((size_t)s->rec_cap * 4)) != cudaSuccess)
+    if ((e = ensure(ctx->bwd_queue, (size_t)s->rec_cap * 4)) != cudaSuccess)
         return cuda_fail(ctx, e, "alloc extended-precision queue");
+    const bool reusable = s->reusable;
+    s->reusable = false;   // until this call has succeeded
     unsigned char* ctrl = s->ctrl.as<unsigned char>();
     unsigned long long* counters = reinterpret_cast<unsigned long long*>(ctrl + kCtrlCounters);
     uint32_t* status = reinterpret_cast<uint32_t*>(ctrl + kCtrlStatus);
@@ -931,10 +1063,16 @@ gsr_status gsr_backward(gsr_ctx* ctx, const gsr_gaussians* g, const gsr_view* vi
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "backward launch");
     s->have_grads = true;
-    if (ctx->cfg.flags & GSR_FLAG_NO_SYNC) return GSR_OK;
+    if (ctx->cfg.flags & GSR_FLAG_NO_SYNC) {
+        s->reusable = reusable;
+        s->touched(cs, false);
+        return GSR_OK;
+    }
     uint32_t st = 0;
     gsr_status r = read_status(ctx, s, cs, &st);
     if (r != GSR_OK) return r;
+    s->reusable = reusable;
+    s->touched(cs, true);
     if (st & kErrTimeout) return fail(ctx, GSR_ERR_TIMEOUT, "device wait timed out");
     if (st & kErrInternal) return fail(ctx, GSR_ERR_CUDA, "internal consistency check failed");
     return GSR_OK;
@@ -1246,6 +1384,7 @@ gsr_status gsr_frequency_schedule(gsr_ctx* ctx, int n_frames, const float* x_gt,
 gsr_status gsr_debug_lists(gsr_saved* s, uint64_t* keys, uint32_t* vals, uint32_t* ranges, void* stream)
 {
     if (!s || !s->filled) return GSR_ERR_INVALID_ARG;
+    s->reusable = false;   // its buffers are read on any stream
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     DebugArgs a{};
     a.tile_key = s->tile_key.as<uint32_t>();
@@ -1268,6 +1407,7 @@ gsr_status gsr_debug_list_slice(gsr_saved* s, int64_t first, int64_t count, uint
                                 void* stream)
 {
     if (!s || !s->filled || first < 0 || count < 0) return GSR_ERR_INVALID_ARG;
+    s->reusable = false;   // its buffers are read on any stream
     DebugArgs a{};
     a.tile_key = s->tile_key.as<uint32_t>();
     a.tile_val = s->tile_val.as<uint32_t>();
@@ -1288,6 +1428,7 @@ gsr_status gsr_debug_list_slice(gsr_saved* s, int64_t first, int64_t count, uint
 gsr_status gsr_debug_records(gsr_saved* s, float* rec, int32_t* rect, uint32_t* flags, void* stream)
 {
     if (!s || !s->filled) return GSR_ERR_INVALID_ARG;
+    s->reusable = false;   // its buffers are read on any stream
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     const int64_t nr = s->table.n_records;
     if (rec) cudaMemsetAsync(rec, 0, (size_t)nr * 64, cs);
@@ -1312,6 +1453,7 @@ gsr_status gsr_debug_records(gsr_saved* s, float* rec, int32_t* rect, uint32_t* 
 gsr_status gsr_debug_pixels(gsr_saved* s, float* t_final, uint32_t* n_contrib, void* stream)
 {
     if (!s || !s->filled) return GSR_ERR_INVALID_ARG;
+    s->reusable = false;   // its buffers are read on any stream
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     const size_t np = (size_t)s->table.n_pixels;
     if (t_final) cudaMemcpyAsync(t_final, s->tfinal.p, np * 4, cudaMemcpyDeviceToDevice, cs);
@@ -1322,6 +1464,7 @@ gsr_status gsr_debug_pixels(gsr_saved* s, float* t_final, uint32_t* n_contrib, v
 gsr_status gsr_debug_record_grads(gsr_saved* s, float* grec, void* stream)
 {
     if (!s || !s->filled || !s->have_grads || !grec) return GSR_ERR_INVALID_ARG;
+    s->reusable = false;   // its buffers are read on any stream
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     cudaMemsetAsync(grec, 0, (size_t)s->table.n_records * 48, cs);
     DebugArgs a{};

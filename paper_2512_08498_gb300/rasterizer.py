@@ -208,9 +208,8 @@ class Rasterizer:
             a = arr[i]
             a.width, a.height = int(v.width), int(v.height)
             a.fx, a.fy, a.cx, a.cy = float(v.fx), float(v.fy), float(v.cx), float(v.cy)
-            vm = np.ascontiguousarray(np.asarray(v.viewmat, np.float32).reshape(16))
-            for k in range(16):
-                a.viewmat[k] = float(vm[k])
+            vm = np.ascontiguousarray(v.viewmat, np.float32).reshape(16)
+            C.memmove(a.viewmat, vm.ctypes.data, 64)
             if v.subset is not None:
                 if not (v.subset.is_cuda and v.subset.dtype in (torch.int32,) and v.subset.is_contiguous()):
                     raise ValueError("subset must be a contiguous int32 CUDA tensor")
@@ -462,27 +461,39 @@ def l1_loss_grad(rgb: torch.Tensor, target: torch.Tensor, dl: Optional[torch.Ten
     return dl, loss
 
 
-def _require_zero(name: str, t: Optional[torch.Tensor], shape) -> None:
+def _require_zero(inputs):
     """The pose and focal inputs are perturbations at which the gradient is
     taken (the renderer uses the views' own matrices and intrinsics): they
-    must be zeros of the given shape.  Reads them back to the host."""
-    if t is None:
-        return
-    if tuple(t.shape) != tuple(shape):
-        raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
-    if bool((t.detach() != 0).any()):
-        raise ValueError(f"{name} must be zero: its gradient is taken at zero; fold a non-zero update into "
-                         "the views (viewmat / fx, fy) instead")
+    must be zeros of the given shape.  inputs: (name, tensor or None, shape).
+    Checks the shapes and enqueues the tests of the values; returns a
+    function that reads them back to the host and raises (called after the
+    render, whose own wait they share)."""
+    tests = []
+    for name, t, shape in inputs:
+        if t is None:
+            continue
+        if tuple(t.shape) != tuple(shape):
+            raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
+        tests.append((name, t.detach().any()))
+
+    def check():
+        for name, nonzero in tests:
+            if bool(nonzero):
+                raise ValueError(f"{name} must be zero: its gradient is taken at zero; fold a non-zero update into "
+                                 "the views (viewmat / fx, fy) instead")
+    return check
 
 
 class _RasterizeFn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, means, log_scales, quats, opacity_logits, sh, pose_delta, focal_delta, raster, views):
-        _require_zero("pose_delta", pose_delta, (len(views), 6))
-        _require_zero("focal_delta", focal_delta, (len(views), 2))
+        ctx.set_materialize_grads(False)   # an output without a gradient stays None in backward
+        check_zero = _require_zero([("pose_delta", pose_delta, (len(views), 6)),
+                                    ("focal_delta", focal_delta, (len(views), 2))])
         params = (means.detach().contiguous(), log_scales.detach().contiguous(), quats.detach().contiguous(),
                   opacity_logits.detach().contiguous(), sh.detach().contiguous())
         rgb, depth, alpha, saved = raster.forward(params, views)
+        check_zero()
         ctx.raster, ctx.views, ctx.saved, ctx.params = raster, views, saved, params
         ctx.want_pose = pose_delta is not None
         ctx.want_focal = focal_delta is not None
