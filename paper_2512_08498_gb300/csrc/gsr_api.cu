@@ -112,7 +112,8 @@ struct gsr_ctx {
     int num_sms = 0;
     std::string err;
     DevMem tmp_keys, tmp_vals, hist, grad_rec, bwd_queue, dup_rows, ins_scratch, freq_scratch, merge_scratch;
-    std::map<int, DevMem> fft_twiddles;   // transform length -> W_n^t table
+    struct Fft { DevMem twiddles; FftPlan plan; };
+    std::map<int, Fft> fft;   // transform length -> W_n^t table and passes
     int hist_blocks = 2048;
     std::map<std::string, gsr_config> tune_cache;
     static constexpr int kProfRing = 64;
@@ -1262,26 +1263,32 @@ gsr_status gsr_merge(gsr_ctx* ctx, const gsr_merge_params* p, const gsr_view* vi
     return GSR_OK;
 }
 
-// Twiddle table of one transform length, W_n^t = exp(-2 pi i t / n) for
+// The plan of one transform length with its table W_n^t = exp(-2 pi i t / n),
 // t in [0, n), computed in double and rounded once; built on first use.
-static cudaError_t fft_twiddles(gsr_ctx* ctx, int n, const float2** out)
+static gsr_status fft_lookup(gsr_ctx* ctx, int n, FftPlan* out)
 {
-    DevMem& d = ctx->fft_twiddles[n];
-    if (!d.p) {
+    auto it = ctx->fft.find(n);
+    if (it == ctx->fft.end()) {
+        FftPlan plan;
+        if (!fft_plan(n, &plan)) return fail(ctx, GSR_ERR_NOT_SUPPORTED, "dft: transform length");
+        gsr_ctx::Fft& f = ctx->fft[n];
         std::vector<float2> h((size_t)n);
         for (int t = 0; t < n; ++t) {
             const double ang = 2.0 * 3.14159265358979323846 * (double)t / (double)n;
             h[(size_t)t] = make_float2((float)std::cos(ang), (float)-std::sin(ang));
         }
-        cudaError_t e = d.ensure((size_t)n * sizeof(float2));
-        if (e == cudaSuccess) e = cudaMemcpy(d.p, h.data(), (size_t)n * sizeof(float2), cudaMemcpyHostToDevice);
+        cudaError_t e = f.twiddles.ensure((size_t)n * sizeof(float2));
+        if (e == cudaSuccess) e = cudaMemcpy(f.twiddles.p, h.data(), (size_t)n * sizeof(float2), cudaMemcpyHostToDevice);
         if (e != cudaSuccess) {
-            ctx->fft_twiddles.erase(n);
-            return e;
+            ctx->fft.erase(n);
+            return cuda_fail(ctx, e, "dft twiddles");
         }
+        f.plan = plan;
+        f.plan.tw = f.twiddles.as<float2>();
+        it = ctx->fft.find(n);
     }
-    *out = ctx->fft_twiddles[n].as<float2>();
-    return cudaSuccess;
+    *out = it->second.plan;
+    return GSR_OK;
 }
 
 gsr_status gsr_dft_energy(gsr_ctx* ctx, const gsr_image* images, int n_images, float* x, void* stream)
@@ -1313,20 +1320,27 @@ gsr_status gsr_dft_energy(gsr_ctx* ctx, const gsr_image* images, int n_images, f
     float2* inter = reinterpret_cast<float2*>(ctx->freq_scratch.as<unsigned char>() + acc_bytes);
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     cudaMemsetAsync(xacc, 0, (size_t)n_images * sizeof(double), cs);
+    // columns per column item: four (a 32-byte sector) unless the call's columns
+    // are too few to give every SM two items
+    int64_t columns = 0;
+    for (int k = 0; k < n_images; ++k) columns += images[k].width / images[k].factor / 2 + 1;
+    const int max_c = columns >= 8 * (int64_t)ctx->num_sms ? 4 : (columns >= 4 * (int64_t)ctx->num_sms ? 2 : 1);
     FreqTable* T = new FreqTable;   // ~17 KB: off the stack
     std::unique_ptr<FreqTable> own(T);
     int i = 0;
     while (i < n_images) {
         std::memset(T, 0, sizeof(FreqTable));
         size_t used = 0;
-        int row_smem = 0, col_smem = 0;
+        int row_smem = 0, col_smem = 0, row_threads = 0, col_threads = 0;
         const int first = i;
         while (i < n_images && T->n_images < kFreqMaxImages && used + need[(size_t)i] <= cap) {
             const gsr_image& im = images[i];
             FreqImage& F = T->img[T->n_images];
             F.src = im.data; F.W = im.width; F.H = im.height; F.factor = im.factor;
             F.Wd = im.width / im.factor; F.Hd = im.height / im.factor; F.Wh = F.Wd / 2 + 1;
-            F.C = F.Hd <= 1228 ? 4 : (F.Hd <= 2457 ? 2 : 1);   // 20 C Hd bytes of shared memory <= 96 KB
+            // at most 100 KB of shared memory per block
+            F.C = std::min(max_c, F.Hd <= 1200 ? 4 : (F.Hd <= 2400 ? 2 : 1));
+            F.RC = max_c == 4 && F.Wd <= 1920 ? 3 : 1;
             F.inter = (int64_t)(used / sizeof(float2));
             F.row_base = T->row_items;
             F.col_base = T->col_items;
@@ -1338,25 +1352,35 @@ gsr_status gsr_dft_energy(gsr_ctx* ctx, const gsr_image* images, int n_images, f
                         if (T->plan[p].n == lens[d]) plans[d] = p;
                     if (plans[d] < 0) {
                         if (T->n_plans == kFreqMaxPlans) break;
-                        FftPlan& P = T->plan[T->n_plans];
-                        if (!fft_plan(lens[d], &P)) return fail(ctx, GSR_ERR_NOT_SUPPORTED, "dft: transform length");
-                        if ((e = fft_twiddles(ctx, lens[d], &P.tw)) != cudaSuccess) return cuda_fail(ctx, e, "dft twiddles");
+                        const gsr_status ps = fft_lookup(ctx, lens[d], &T->plan[T->n_plans]);
+                        if (ps != GSR_OK) return ps;
                         plans[d] = T->n_plans++;
                     }
                 }
                 if (plans[0] < 0 || plans[1] < 0) break;   // plan table full: next launch
                 F.row_plan = plans[0]; F.col_plan = plans[1];
-                T->row_items += (int64_t)3 * ((F.Hd + 1) / 2);
+                T->row_items += (int64_t)(3 / F.RC) * ((F.Hd + 1) / 2);
                 T->col_items += (F.Wh + F.C - 1) / F.C;
-                row_smem = std::max(row_smem, 16 * F.Wd);
-                col_smem = std::max(col_smem, 20 * F.C * F.Hd);
+                row_smem = std::max(row_smem, 16 * F.RC * fft_span(F.Wd));
+                col_smem = std::max(col_smem, 16 * F.C * fft_span(F.Hd) + 4 * F.C * F.Hd);
+                // work items of the passes: butterflies, or the output pairs of a
+                // direct pass
+                auto most = [](const FftPlan& P) {
+                    int m = 1;
+                    for (int st = 0; st < P.n_stages; ++st)
+                        m = std::max(m, P.st[st].R > 16 || P.st[st].R == 7 || P.st[st].R == 11 || P.st[st].R == 13
+                                            ? (P.st[st].R + 1) / 2 * P.st[st].m : P.st[st].m);
+                    return m;
+                };
+                row_threads = std::max(row_threads, F.RC * most(T->plan[F.row_plan]));
+                col_threads = std::max(col_threads, F.C * most(T->plan[F.col_plan]));
             }
             used += need[(size_t)i];
             ++T->n_images;
             ++i;
         }
         if (T->n_images == 0) return fail(ctx, GSR_ERR_NOT_SUPPORTED, "dft: empty launch table");
-        launch_dft_energy(*T, inter, xacc + first, row_smem, col_smem, ctx->num_sms, cs);
+        launch_dft_energy(*T, inter, xacc + first, row_smem, col_smem, row_threads, col_threads, ctx->num_sms, cs);
         if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "dft launch");
     }
     launch_dft_finalize(xacc, x, n_images, cs);

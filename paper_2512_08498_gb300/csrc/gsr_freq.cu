@@ -8,42 +8,100 @@
 // the frames drawn for optimisation and r' = X(I^n) / X(I~) (Eq. 12), I^n the
 // ground truth at downsampling factor n, raises the level when below tau_f.
 //
-// The DFT is a mixed-radix Stockham transform (radix 4, 2, 3, 5 butterflies
-// and a direct radix-p pass for any other prime) run in shared memory, in two
-// passes over each image:
-//   rows     two real rows of one channel packed as one complex sequence;
-//            after the transform the Hermitian split gives both rows' spectra
-//            for k = 0 .. W/2 (the other half is their conjugate mirror),
-//            written to a half-spectrum buffer [3][H][W/2 + 1];
+// The DFT is a mixed-radix Stockham transform in as few passes as the composite
+// radices 16, 15, 12, 10, 9, 8, 6, 5, 4, 3, 2 give (1600 = 16 10 10, 900 = 10 10
+// 9), after a direct pass for each other prime, in two passes over each image:
+//   rows     two real rows of a channel packed as one complex sequence; after
+//            the transform the Hermitian split gives both rows' spectra for
+//            k = 0 .. W/2 (the other half is their conjugate mirror), written
+//            to a half-spectrum buffer [3][H][W/2 + 1];
 //   columns  C adjacent columns of that buffer, one channel after the other,
 //            transformed along y; |F_c|^2 summed over the channels in shared
 //            memory, then sqrt and summed with weight 2 for the columns whose
 //            mirror k' = W - k is not stored (1 for k = 0 and k = W/2).
+// The first pass of a transform loads from memory, the last one of a column
+// adds |F_c|^2, so only the passes between them go through shared memory.
 // Box downsampling (I^n) is applied while loading the rows.  Values are FP32
 // (twiddles from a host table computed in double); the magnitudes are summed
 // per thread in FP32 and across threads and blocks in FP64.
+//
+// Bound by latency: barriers and the index arithmetic around them (issue slots
+// 50-55 %, DRAM 10-25 %).  Against radix-4, 2, 3 and 5 passes (five for 1600 and
+// 900) with separate load and magnitude steps, a direct pass per output and four
+// columns per item whatever the image: 18 images of 1600 x 900 columns 282 ->
+// 200 us, rows 246 -> 249; nine images of 333 x 251 and smaller (prime heights)
+// columns 122 -> 44 us.  The radix-16 passes need the padding (rows 296 us
+// without).
+#include <algorithm>
 #include <cmath>
+#include <vector>
 
 #include "gsr_common.cuh"
 #include "gsr_kernels.h"
 
 namespace gsr {
 
-constexpr int kRowThreads = 128;
-constexpr int kColThreads = 256;
+// Largest blocks; a launch takes as many threads as its largest pass has
+// butterflies (whole warps), so that a pass is one round where it can be.
+constexpr int kRowThreads = 512;
+constexpr int kColThreads = 512;
 
 static uint32_t recip32(int d) { return d <= 1 ? 0u : (uint32_t)((((uint64_t)1 << 32) + (uint64_t)d - 1) / (uint64_t)d); }
 
+// The fewest passes over the composite radices for n = 2^a 3^b 5^c (ties to the
+// larger first radix), by the exponents; false if a pass more than
+// 2 kFftMaxStages were needed.
+static bool fft_radices(int n, int* radix, int& k)
+{
+    static constexpr struct { int r, e[3]; } kRadix[] = {
+        {16, {4, 0, 0}}, {15, {0, 1, 1}}, {12, {2, 1, 0}}, {10, {1, 0, 1}}, {9, {0, 2, 0}}, {8, {3, 0, 0}},
+        {6, {1, 1, 0}}, {5, {0, 0, 1}}, {4, {2, 0, 0}}, {3, {0, 1, 0}}, {2, {1, 0, 0}}};
+    int e[3] = {0, 0, 0};
+    const int base[3] = {2, 3, 5};
+    for (int i = 0; i < 3; ++i)
+        while (n % base[i] == 0) { n /= base[i]; ++e[i]; }
+    if (n != 1) return false;
+    // best[x]: passes of 2^x0 3^x1 5^x2 and the first one's radix
+    struct Best { int passes, first; };
+    const int ny = e[1] + 1, nz = e[2] + 1;
+    std::vector<Best> best((size_t)(e[0] + 1) * ny * nz, Best{0, -1});
+    auto at = [&](int x, int y, int z) -> Best& { return best[((size_t)x * ny + y) * nz + z]; };
+    for (int x = 0; x <= e[0]; ++x)
+        for (int y = 0; y <= e[1]; ++y)
+            for (int z = 0; z <= e[2]; ++z) {
+                if (x + y + z == 0) continue;
+                Best& b = at(x, y, z);
+                b.passes = 1 << 20;
+                for (int i = 0; i < (int)(sizeof(kRadix) / sizeof(kRadix[0])); ++i) {
+                    const int* r = kRadix[i].e;
+                    if (r[0] > x || r[1] > y || r[2] > z) continue;
+                    const int p = 1 + at(x - r[0], y - r[1], z - r[2]).passes;
+                    if (p < b.passes) b = Best{p, i};
+                }
+            }
+    if (at(e[0], e[1], e[2]).passes > 2 * kFftMaxStages) return false;
+    for (k = 0; e[0] + e[1] + e[2] > 0;) {
+        const auto& r = kRadix[at(e[0], e[1], e[2]).first];
+        radix[k++] = r.r;
+        for (int i = 0; i < 3; ++i) e[i] -= r.e[i];
+    }
+    return true;
+}
+
 bool fft_plan(int n, FftPlan* P)
 {
+    if (n < 1 || n > kFreqMaxDim) return false;
     int radix[2 * kFftMaxStages];
     int k = 0, rest = n;
-    while (rest % 4 == 0 && k < kFftMaxStages) { radix[k++] = 4; rest /= 4; }
-    for (int p = 2; p <= 5 && rest > 1; ++p)
-        while (rest % p == 0 && k < kFftMaxStages) { radix[k++] = p; rest /= p; }
+    for (int p : {2, 3, 5})
+        while (rest % p == 0) rest /= p;
+    const int smooth = n / rest;
+    // other primes first: their direct pass then needs no twiddles
     for (int p = 7; rest > 1 && k < kFftMaxStages; p += 2)
         while (rest % p == 0 && k < kFftMaxStages) { radix[k++] = p; rest /= p; }
-    if (rest != 1 || n < 1 || n > kFreqMaxDim) return false;
+    int ks = 0, rs[2 * kFftMaxStages];
+    if (rest != 1 || !fft_radices(smooth, rs, ks) || k + ks > kFftMaxStages) return false;
+    for (int i = 0; i < ks; ++i) radix[k++] = rs[i];
     P->n = n;
     P->n_stages = k;
     int Ns = 1;
@@ -111,82 +169,219 @@ template <> __device__ __forceinline__ void butterfly<5>(float2* v)
     v[2] = cadd(m2, r2); v[3] = csub(m2, r2);
 }
 
-// One Stockham pass over nseq sequences of length n stored back to back.
-// Butterfly j (of m = n / R) reads src[j + r m], r < R, twiddled by
-// W_{Ns R}^{r (j mod Ns)}, and writes its R outputs to
-// dst[(j - j mod Ns) R + j mod Ns + q Ns], q < R; Ns is the product of the
-// radices of the earlier passes.  One twiddle is loaded per butterfly, its
-// powers formed by complex products.
-template <int R>
-__device__ __forceinline__ void fft_pass(const float2* __restrict__ src, float2* __restrict__ dst, int nseq, int n,
-                                         const FftStage& S, const float2* __restrict__ tw)
+// cos and sin of 2 pi t / N for t < N, rounded once (series in double, at
+// compile time).
+template <int N>
+struct UnitRoots {
+    float c[N], s[N];
+    constexpr UnitRoots() : c(), s()
+    {
+        for (int t = 0; t < N; ++t) {
+            // angle folded into [-pi, pi]
+            const double x = 2.0 * 3.14159265358979323846 * (double)(2 * t > N ? t - N : t) / (double)N;
+            double tc = 1.0, ts = x, sc = 1.0, ss = x;
+            for (int i = 1; i < 20; ++i) {
+                tc *= -x * x / (double)((2 * i - 1) * (2 * i));
+                ts *= -x * x / (double)((2 * i) * (2 * i + 1));
+                sc += tc;
+                ss += ts;
+            }
+            c[t] = (float)sc;
+            s[t] = (float)ss;
+        }
+    }
+};
+
+// N1 N2-point DFT from N1- and N2-point ones: input n = N2 n1 + n2, output
+// k = k1 + N1 k2, twiddles W_N^(n2 k1) between the two.
+template <int N1, int N2>
+__device__ __forceinline__ void dft_composite(float2* v)
+{
+    constexpr int N = N1 * N2;
+    constexpr UnitRoots<N> w;
+    float2 t[N];
+#pragma unroll
+    for (int n2 = 0; n2 < N2; ++n2) {
+        float2 u[N1];
+#pragma unroll
+        for (int n1 = 0; n1 < N1; ++n1) u[n1] = v[N2 * n1 + n2];
+        butterfly<N1>(u);
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) {
+            const int e = n2 * k1;
+            t[N2 * k1 + n2] = e == 0 ? u[k1] : cmul(u[k1], make_float2(w.c[e], -w.s[e]));
+        }
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < N1; ++k1) {
+        butterfly<N2>(t + N2 * k1);
+#pragma unroll
+        for (int k2 = 0; k2 < N2; ++k2) v[k1 + N1 * k2] = t[N2 * k1 + k2];
+    }
+}
+template <> __device__ __forceinline__ void butterfly<6>(float2* v) { dft_composite<2, 3>(v); }
+template <> __device__ __forceinline__ void butterfly<8>(float2* v) { dft_composite<2, 4>(v); }
+template <> __device__ __forceinline__ void butterfly<9>(float2* v) { dft_composite<3, 3>(v); }
+template <> __device__ __forceinline__ void butterfly<10>(float2* v) { dft_composite<2, 5>(v); }
+template <> __device__ __forceinline__ void butterfly<12>(float2* v) { dft_composite<3, 4>(v); }
+template <> __device__ __forceinline__ void butterfly<15>(float2* v) { dft_composite<3, 5>(v); }
+template <> __device__ __forceinline__ void butterfly<16>(float2* v) { dft_composite<4, 4>(v); }
+
+// Where element i of a sequence lies in its shared-memory buffer: one place of
+// padding per 16, because the first pass of radix 16 writes at a stride of 16
+// (70 % of the row pass's shared-memory wavefronts were bank conflicts).
+__device__ __forceinline__ int fft_at(int i) { return i + (i >> 4); }
+// (fft_span(n), the length of such a buffer, is in gsr_kernels.h)
+
+// One Stockham pass over nseq sequences of length n.  Butterfly j (of
+// m = n / R) of sequence s takes its inputs from load(s, j + r m), r < R,
+// twiddled by W_{Ns R}^{r (j mod Ns)}, and gives its R outputs to
+// store(s, (j - j mod Ns) R + j mod Ns + q Ns, value), q < R; Ns is the product
+// of the radices of the earlier passes.  One twiddle is loaded per butterfly,
+// its powers formed by complex products w^(2i) = w^i w^i, w^(2i+1) = w^(2i) w.
+// Consecutive threads take consecutive sequences if SEQ_FAST (the columns,
+// adjacent in memory), else consecutive butterflies.
+template <int R, bool SEQ_FAST, typename Load, typename Store>
+__device__ __forceinline__ void fft_pass(int nseq, const FftStage& S, const float2* __restrict__ tw, Load load, Store store)
 {
     const int m = S.m, Ns = S.Ns, step = S.step;
     const uint32_t mag_m = S.mag_m, mag_ns = S.mag_ns;
     for (int t = threadIdx.x; t < nseq * m; t += blockDim.x) {
-        const int s = udiv16(t, mag_m), j = t - s * m;
+        int s, j;
+        if (SEQ_FAST) { j = t / nseq; s = t - j * nseq; }
+        else { s = udiv16(t, mag_m); j = t - s * m; }
         const int jb = udiv16(j, mag_ns), jm = j - jb * Ns;
-        const float2* in = src + s * n + j;
         float2 v[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = in[r * m];
+        for (int r = 0; r < R; ++r) v[r] = load(s, j + r * m);
         if (jm != 0) {
-            const float2 w1 = __ldg(tw + jm * step);
-            float2 w = w1;
+            float2 w[R];
+            w[1] = __ldg(tw + jm * step);
 #pragma unroll
-            for (int r = 1; r < R; ++r) {
-                v[r] = cmul(v[r], w);
-                if (r + 1 < R) w = cmul(w, w1);
-            }
+            for (int r = 2; r < R; ++r) w[r] = (r & 1) ? cmul(w[r - 1], w[1]) : cmul(w[r / 2], w[r / 2]);
+#pragma unroll
+            for (int r = 1; r < R; ++r) v[r] = cmul(v[r], w[r]);
         }
         butterfly<R>(v);
-        float2* out = dst + s * n + jb * Ns * R + jm;
+        const int o = jb * Ns * R + jm;
 #pragma unroll
-        for (int q = 0; q < R; ++q) out[q * Ns] = v[q];
+        for (int q = 0; q < R; ++q) store(s, o + q * Ns, v[q]);
     }
 }
 
-// The same pass for a prime radix R > 5: one thread per output, the R-point
-// DFT by its definition; the combined twiddle of input r for output q is
-// W_{Ns R}^{r (j mod Ns + q Ns)}.
-__device__ void fft_pass_direct(const float2* __restrict__ src, float2* __restrict__ dst, int nseq, int n,
-                                const FftStage& S, const float2* __restrict__ tw)
+// The same pass for a prime radix R > 5, the R-point DFT by its definition
+// with the outputs q and R - q taken together: from s_r = x_r + x_{R-r} and
+// d_r = x_r - x_{R-r} (x the twiddled inputs, r <= h = (R - 1) / 2),
+//   X_q, X_{R-q} = x_0 + sum_r s_r cos(2 pi q r / R) -+ i sum_r d_r sin(2 pi q r / R),
+// a quarter of the products of the separate sums.  a holds the sequences
+// (stored back to back) and is overwritten with s and d.
+template <typename Store>
+__device__ void fft_pass_prime(float2* __restrict__ a, int nseq, int n, const FftStage& S, const float2* __restrict__ tw,
+                               Store store)
 {
-    const int R = S.R, m = S.m, Ns = S.Ns, NsR = Ns * R, step = S.step;
-    for (int t = threadIdx.x; t < nseq * n; t += blockDim.x) {
-        const int s = t / n, u = t - s * n;
-        const int j = udiv16(u, S.mag_r), q = u - j * R;
+    const int R = S.R, m = S.m, Ns = S.Ns, step = S.step, h = (R - 1) / 2, root = n / R;
+    const int per = h * m, per_out = (h + 1) * m;
+    for (int t = threadIdx.x; t < nseq * per; t += blockDim.x) {
+        const int s = t / per, u = t - s * per;
+        const int r = u / m + 1, j = u - (r - 1) * m;
         const int jb = udiv16(j, S.mag_ns), jm = j - jb * Ns;
-        const float2* in = src + s * n;
-        const int e = jm + q * Ns;   // < Ns R
-        float2 acc = in[j];
-        int idx = 0;
-        for (int r = 1; r < R; ++r) {
-            idx += e;
-            if (idx >= NsR) idx -= NsR;
-            acc = cadd(acc, cmul(in[j + r * m], __ldg(tw + idx * step)));
+        float2* x = a + s * fft_span(n);
+        float2 &xp = x[fft_at(j + r * m)], &xq = x[fft_at(j + (R - r) * m)];
+        float2 p = xp, q = xq;
+        if (jm != 0) {
+            p = cmul(p, __ldg(tw + r * jm * step));
+            q = cmul(q, __ldg(tw + (R - r) * jm * step));
         }
-        dst[s * n + jb * NsR + jm + q * Ns] = acc;
+        xp = cadd(p, q);
+        xq = csub(p, q);
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < nseq * per_out; t += blockDim.x) {
+        const int s = t / per_out, u = t - s * per_out;
+        const int q = u / m, j = u - q * m;
+        const int jb = udiv16(j, S.mag_ns), jm = j - jb * Ns;
+        const float2* x = a + s * fft_span(n);
+        const float2 x0 = x[fft_at(j)];
+        float2 c = x0, d = make_float2(0.0f, 0.0f);
+        int idx = 0;
+#pragma unroll 4
+        for (int r = 1; r <= h; ++r) {
+            idx += q;
+            if (idx >= R) idx -= R;
+            const float2 w = __ldg(tw + idx * root);   // cos, -sin
+            const float2 sr = x[fft_at(j + r * m)], dr = x[fft_at(j + (R - r) * m)];
+            c.x = fmaf(sr.x, w.x, c.x);
+            c.y = fmaf(sr.y, w.x, c.y);
+            d.x = fmaf(dr.y, -w.y, d.x);    // -i d sin
+            d.y = fmaf(dr.x, w.y, d.y);
+        }
+        const int o = jb * Ns * R + jm;
+        store(s, o + q * Ns, cadd(c, d));
+        if (q > 0) store(s, o + (R - q) * Ns, csub(c, d));
     }
 }
 
-// Transform nseq sequences held in a; b is scratch of the same size.
-// Returns the buffer that holds the result.  All threads of the block call it.
-__device__ float2* fft_run(float2* a, float2* b, int nseq, const FftPlan& P)
+// Pass st of plan P over nseq sequences.  A prime pass reads from `a` (first
+// filled through load if it is the plan's first pass).
+template <bool SEQ_FAST, typename Load, typename Store>
+__device__ __forceinline__ void fft_stage(const FftPlan& P, int st, int nseq, float2* a, Load load, Store store)
 {
-    for (int st = 0; st < P.n_stages; ++st) {
-        const FftStage& S = P.st[st];
-        switch (S.R) {
-        case 4: fft_pass<4>(a, b, nseq, P.n, S, P.tw); break;
-        case 2: fft_pass<2>(a, b, nseq, P.n, S, P.tw); break;
-        case 3: fft_pass<3>(a, b, nseq, P.n, S, P.tw); break;
-        case 5: fft_pass<5>(a, b, nseq, P.n, S, P.tw); break;
-        default: fft_pass_direct(a, b, nseq, P.n, S, P.tw); break;
+    const FftStage& S = P.st[st];
+    switch (S.R) {
+    case 16: fft_pass<16, SEQ_FAST>(nseq, S, P.tw, load, store); break;
+    case 15: fft_pass<15, SEQ_FAST>(nseq, S, P.tw, load, store); break;
+    case 12: fft_pass<12, SEQ_FAST>(nseq, S, P.tw, load, store); break;
+    case 10: fft_pass<10, SEQ_FAST>(nseq, S, P.tw, load, store); break;
+    case 9: fft_pass<9, SEQ_FAST>(nseq, S, P.tw, load, store); break;
+    case 8: fft_pass<8, SEQ_FAST>(nseq, S, P.tw, load, store); break;
+    case 6: fft_pass<6, SEQ_FAST>(nseq, S, P.tw, load, store); break;
+    case 5: fft_pass<5, SEQ_FAST>(nseq, S, P.tw, load, store); break;
+    case 4: fft_pass<4, SEQ_FAST>(nseq, S, P.tw, load, store); break;
+    case 3: fft_pass<3, SEQ_FAST>(nseq, S, P.tw, load, store); break;
+    case 2: fft_pass<2, SEQ_FAST>(nseq, S, P.tw, load, store); break;
+    default:
+        if (st == 0) {
+            for (int t = threadIdx.x; t < nseq * P.n; t += blockDim.x) {
+                const int x = SEQ_FAST ? t / nseq : t % P.n, s = SEQ_FAST ? t - x * nseq : t / P.n;
+                a[s * fft_span(P.n) + fft_at(x)] = load(s, x);
+            }
+            __syncthreads();
         }
-        __syncthreads();
-        float2* t = a; a = b; b = t;
+        fft_pass_prime(a, nseq, P.n, S, P.tw, store);
+        break;
     }
-    return a;
+    __syncthreads();
+}
+
+// Transform nseq sequences: the first pass takes its inputs through load, the
+// last gives its outputs to store, the ones between run in shared memory (a and
+// b, nseq fft_span(n) places each).  All threads of the block call it; it ends with a
+// barrier.
+template <bool SEQ_FAST, typename Load, typename Store>
+__device__ __forceinline__ void fft_run(const FftPlan& P, int nseq, float2* a, float2* b, Load load, Store store)
+{
+    const int n = fft_span(P.n), last = P.n_stages - 1;
+    if (last < 0) {   // length 1
+        for (int s = threadIdx.x; s < nseq; s += blockDim.x) store(s, 0, load(s, 0));
+        __syncthreads();
+        return;
+    }
+    if (last == 0) {
+        fft_stage<SEQ_FAST>(P, 0, nseq, a, load, store);
+        return;
+    }
+    // (a prime first pass stages its inputs in a, so its outputs go to b)
+    fft_stage<SEQ_FAST>(P, 0, nseq, a, load, [=](int s, int i, float2 v) { b[s * n + fft_at(i)] = v; });
+    float2 *src = b, *dst = a;
+    for (int st = 1; st < last; ++st) {
+        float2 *from = src, *to = dst;
+        fft_stage<false>(P, st, nseq, from, [=](int s, int i) { return from[s * n + fft_at(i)]; },
+                         [=](int s, int i, float2 v) { to[s * n + fft_at(i)] = v; });
+        src = to;
+        dst = from;
+    }
+    float2* from = src;
+    fft_stage<false>(P, last, nseq, from, [=](int s, int i) { return from[s * n + fft_at(i)]; }, store);
 }
 
 __device__ __forceinline__ int image_of(const FreqTable& T, int64_t item, bool rows)
@@ -200,63 +395,60 @@ __device__ __forceinline__ int image_of(const FreqTable& T, int64_t item, bool r
     return lo;
 }
 
-// Row pass: item = (image, row pair, channel).  Rows y0 = 2p and y0 + 1 of
-// channel c (box-averaged over factor x factor source pixels) are the real
-// and imaginary parts of one sequence Z; their spectra are
+// Row pass: item = (image, row pair, group of I.RC channels).  Rows y0 = 2p and
+// y0 + 1 of a channel (box-averaged over factor x factor source pixels) are the
+// real and imaginary parts of one sequence Z; their spectra are
 // A(k) = (Z(k) + conj Z(-k)) / 2 and B(k) = (Z(k) - conj Z(-k)) / (2i).
-__global__ void __launch_bounds__(kRowThreads)
+__global__ void __launch_bounds__(kRowThreads, 2)
 dft_rows_kernel(const __grid_constant__ FreqTable T, float2* __restrict__ inter)
 {
-    extern __shared__ float2 sm[];
+    extern __shared__ float2 sm[];   // two buffers of the group's rows
     for (int64_t item = blockIdx.x; item < T.row_items; item += gridDim.x) {
         const FreqImage& I = T.img[image_of(T, item, true)];
         const int64_t local = item - I.row_base;
-        const int c = (int)(local % 3), y0 = 2 * (int)(local / 3);
+        const int RC = I.RC, per = 3 / RC;
+        const int c0 = (int)(local % per) * RC, y0 = 2 * (int)(local / per);
         const int Wd = I.Wd, f = I.factor;
+        const int64_t W = I.W, hw = (int64_t)I.H * I.W;
         const bool two = y0 + 1 < I.Hd;
-        const float* __restrict__ plane = I.src + (int64_t)c * I.H * I.W;
-        float2* a = sm;
-        float2* b = sm + Wd;
-        if (f == 1) {
-            // four loads per row in flight per thread
-            const float* __restrict__ r0 = plane + (int64_t)y0 * I.W;
-            const float* __restrict__ r1 = r0 + (two ? I.W : 0);
-            for (int x = threadIdx.x; x < Wd; x += 4 * kRowThreads) {
-                float p0[4], p1[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int xi = x + u * kRowThreads;
-                    p0[u] = xi < Wd ? __ldg(r0 + xi) : 0.0f;
-                    p1[u] = xi < Wd ? __ldg(r1 + xi) : 0.0f;
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int xi = x + u * kRowThreads;
-                    if (xi < Wd) a[xi] = make_float2(p0[u], two ? p1[u] : 0.0f);
-                }
-            }
-        } else {
+        const float* __restrict__ r0 = I.src + c0 * hw + (int64_t)y0 * f * W;
+        const FftPlan& P = T.plan[I.row_plan];
+        const int span = fft_span(Wd);
+        float2 *a = sm, *b = sm + RC * span;
+        // the last pass reads the buffer its predecessor wrote (b, a, b, ...) and
+        // writes the other; a single pass writes b
+        float2* z = (P.n_stages & 1) ? b : a;
+        if (f != 1) {
+            // the means of f x f source pixels, staged in a
             const float inv = 1.0f / (float)(f * f);
-            for (int x = threadIdx.x; x < Wd; x += kRowThreads) {
+            for (int t = threadIdx.x; t < RC * Wd; t += blockDim.x) {
+                const int c = t / Wd, x = t - c * Wd;
                 float p0 = 0.0f, p1 = 0.0f;
                 for (int dy = 0; dy < f; ++dy) {
-                    const float* r0 = plane + (int64_t)(y0 * f + dy) * I.W + (int64_t)x * f;
-                    for (int dx = 0; dx < f; ++dx) p0 += __ldg(r0 + dx);
-                    if (two) {
-                        const float* r1 = plane + (int64_t)((y0 + 1) * f + dy) * I.W + (int64_t)x * f;
-                        for (int dx = 0; dx < f; ++dx) p1 += __ldg(r1 + dx);
-                    }
+                    const float* q = r0 + c * hw + dy * W + (int64_t)x * f;
+                    for (int dx = 0; dx < f; ++dx) p0 += __ldg(q + dx);
+                    if (two)
+                        for (int dx = 0; dx < f; ++dx) p1 += __ldg(q + (int64_t)f * W + dx);
                 }
-                a[x] = make_float2(p0 * inv, p1 * inv);
+                a[c * span + fft_at(x)] = make_float2(p0 * inv, p1 * inv);
             }
+            __syncthreads();
         }
-        __syncthreads();
-        const float2* z = fft_run(a, b, 1, T.plan[I.row_plan]);
-        float2* o = inter + I.inter + ((int64_t)c * I.Hd + y0) * I.Wh;
-        for (int k = threadIdx.x; k < I.Wh; k += blockDim.x) {
-            const float2 z1 = z[k], z2 = z[k == 0 ? 0 : Wd - k];
-            o[k] = make_float2(0.5f * (z1.x + z2.x), 0.5f * (z1.y - z2.y));
-            if (two) o[I.Wh + k] = make_float2(0.5f * (z1.y + z2.y), 0.5f * (z2.x - z1.x));
+        fft_run<false>(P, RC, a, b,
+                       [=](int c, int x) {
+                           if (f != 1) return a[c * span + fft_at(x)];
+                           const float* q = r0 + c * hw + x;
+                           return make_float2(__ldg(q), two ? __ldg(q + W) : 0.0f);
+                       },
+                       [=](int c, int k, float2 v) { z[c * span + fft_at(k)] = v; });
+        for (int c = 0; c < RC; ++c) {
+            float2* o = inter + I.inter + ((int64_t)(c0 + c) * I.Hd + y0) * I.Wh;
+            const float2* zc = z + c * span;
+            for (int k = threadIdx.x; k < I.Wh; k += blockDim.x) {
+                const float2 z1 = zc[fft_at(k)], z2 = zc[fft_at(k == 0 ? 0 : Wd - k)];
+                o[k] = make_float2(0.5f * (z1.x + z2.x), 0.5f * (z1.y - z2.y));
+                if (two) o[I.Wh + k] = make_float2(0.5f * (z1.y + z2.y), 0.5f * (z2.x - z1.x));
+            }
         }
         __syncthreads();   // the buffers are rewritten by the next item
     }
@@ -264,7 +456,7 @@ dft_rows_kernel(const __grid_constant__ FreqTable T, float2* __restrict__ inter)
 
 // Column pass: item = (image, C adjacent half-spectrum columns).  Shared
 // memory: two C x Hd complex buffers and C x Hd floats of sum_c |F_c|^2.
-__global__ void __launch_bounds__(kColThreads)
+__global__ void __launch_bounds__(kColThreads, 2)
 dft_cols_kernel(const __grid_constant__ FreqTable T, const float2* __restrict__ inter, double* __restrict__ xacc)
 {
     extern __shared__ float2 sm[];
@@ -277,43 +469,23 @@ dft_cols_kernel(const __grid_constant__ FreqTable T, const float2* __restrict__ 
         const int k0 = (int)(item - I.col_base) * I.C;
         const int nc = min(I.C, Wh - k0), ne = nc * Hd;
         float2* a = sm;
-        float2* b = sm + I.C * Hd;
-        float* acc = reinterpret_cast<float*>(sm + 2 * I.C * Hd);
+        float2* b = sm + I.C * fft_span(Hd);
+        float* acc = reinterpret_cast<float*>(sm + 2 * I.C * fft_span(Hd));
         for (int e = tid; e < ne; e += blockDim.x) acc[e] = 0.0f;
-        // loads: thread = (row group, column kk), C a power of two
-        const int lc = I.C == 4 ? 2 : (I.C == 2 ? 1 : 0);
-        const int kk = tid & (I.C - 1), ty = tid >> lc, ystep = kColThreads >> lc;
+        __syncthreads();
         for (int c = 0; c < 3; ++c) {
-            const float2* __restrict__ plane = inter + I.inter + (int64_t)c * Hd * Wh + k0 + kk;
-            if (kk < nc) {
-                for (int y = ty; y < Hd; y += 4 * ystep) {
-                    float2 v[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int yi = y + u * ystep;
-                        v[u] = yi < Hd ? plane[(int64_t)yi * Wh] : make_float2(0.0f, 0.0f);
-                    }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int yi = y + u * ystep;
-                        if (yi < Hd) a[kk * Hd + yi] = v[u];
-                    }
-                }
-            }
-            __syncthreads();
-            const float2* F = fft_run(a, b, nc, T.plan[I.col_plan]);
-            for (int e = tid; e < ne; e += blockDim.x) {
-                const float2 v = F[e];
-                acc[e] += v.x * v.x + v.y * v.y;
-            }
-            __syncthreads();
+            // the last pass adds |F_c|^2 where a thread's butterflies put their
+            // outputs, the same places for every channel
+            const float2* __restrict__ plane = inter + I.inter + (int64_t)c * Hd * Wh + k0;
+            fft_run<true>(T.plan[I.col_plan], nc, a, b, [=](int kk, int y) { return __ldg(plane + (int64_t)y * Wh + kk); },
+                          [=](int kk, int y, float2 v) { acc[kk * Hd + y] += v.x * v.x + v.y * v.y; });
         }
         float part = 0.0f;
         for (int q = 0; q < nc; ++q) {
             const int k = k0 + q;
             const float w = (k == 0 || 2 * k == I.Wd) ? 1.0f : 2.0f;
             float sq = 0.0f;
-            for (int y = tid; y < Hd; y += kColThreads) sq += sqrtf(acc[q * Hd + y]);
+            for (int y = tid; y < Hd; y += blockDim.x) sq += sqrtf(acc[q * Hd + y]);
             part += w * sq;
         }
         double d = (double)part;
@@ -323,8 +495,7 @@ dft_cols_kernel(const __grid_constant__ FreqTable T, const float2* __restrict__ 
         __syncthreads();
         if (tid == 0) {
             double s = 0.0;
-#pragma unroll
-            for (int w = 0; w < kColThreads / 32; ++w) s += s_red[w];
+            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += s_red[w];
             atomicAdd(xacc + ii, s);
         }
         __syncthreads();   // s_red and the buffers are rewritten by the next item
@@ -397,26 +568,28 @@ static int resident_blocks(K kernel, int threads, int smem)
     return n;
 }
 
-void launch_dft_energy(const FreqTable& T, float2* inter, double* xacc, int row_smem, int col_smem, int num_sms,
-                       cudaStream_t s)
+void launch_dft_energy(const FreqTable& T, float2* inter, double* xacc, int row_smem, int col_smem, int row_threads,
+                       int col_threads, int num_sms, cudaStream_t s)
 {
     static std::atomic<int> attr_set[kMaxDevices];
     per_device_once(attr_set, [] {
-        cudaFuncSetAttribute(dft_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFreqMaxDim * 16);
+        cudaFuncSetAttribute(dft_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
         cudaFuncSetAttribute(dft_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
         return 1;
     });
+    row_threads = std::min(kRowThreads, std::max(64, (row_threads + 31) / 32 * 32));
+    col_threads = std::min(kColThreads, std::max(64, (col_threads + 31) / 32 * 32));
     if (T.row_items > 0) {
-        int64_t grid = (int64_t)num_sms * resident_blocks(dft_rows_kernel, kRowThreads, row_smem);
+        int64_t grid = (int64_t)num_sms * resident_blocks(dft_rows_kernel, row_threads, row_smem);
         if (grid > T.row_items) grid = T.row_items;
         GSR_COUNT_LAUNCH();
-        dft_rows_kernel<<<(unsigned)grid, kRowThreads, row_smem, s>>>(T, inter);
+        dft_rows_kernel<<<(unsigned)grid, row_threads, row_smem, s>>>(T, inter);
     }
     if (T.col_items > 0) {
-        int64_t grid = (int64_t)num_sms * resident_blocks(dft_cols_kernel, kColThreads, col_smem);
+        int64_t grid = (int64_t)num_sms * resident_blocks(dft_cols_kernel, col_threads, col_smem);
         if (grid > T.col_items) grid = T.col_items;
         GSR_COUNT_LAUNCH();
-        dft_cols_kernel<<<(unsigned)grid, kColThreads, col_smem, s>>>(T, inter, xacc);
+        dft_cols_kernel<<<(unsigned)grid, col_threads, col_smem, s>>>(T, inter, xacc);
     }
 }
 

@@ -307,7 +307,7 @@ struct FftPlan {
 struct FreqImage {
     const float* src;            // planar RGB [3][H][W]
     int W, H, factor;            // source size and box-downsampling factor
-    int Wd, Hd, Wh, C;           // transformed size, Wh = Wd/2 + 1, columns per column item
+    int Wd, Hd, Wh, C, RC;       // transformed size, Wh = Wd/2 + 1, columns per column item, channels per row item
     int row_plan, col_plan;      // plans of length Wd and Hd
     int64_t inter;               // offset (float2) of the half spectra [3][Hd][Wh]
     int64_t row_base, col_base;  // first row-pass / column-pass item
@@ -320,9 +320,11 @@ struct FreqTable {
     FreqImage img[kFreqMaxImages];
 };
 
+// Places of a sequence of n values in shared memory (one of padding per 16).
+__host__ __device__ inline int fft_span(int n) { return n + n / 16 + 1; }
 bool fft_plan(int n, FftPlan* plan);   // passes of length n (tw left to the caller); false if unsupported
-void launch_dft_energy(const FreqTable& T, float2* inter, double* xacc, int row_smem, int col_smem, int num_sms,
-                       cudaStream_t s);
+void launch_dft_energy(const FreqTable& T, float2* inter, double* xacc, int row_smem, int col_smem, int row_threads,
+                       int col_threads, int num_sms, cudaStream_t s);
 void launch_dft_finalize(const double* xacc, float* x, int n, cudaStream_t s);
 void launch_frequency_schedule(int n_frames, const float* x_gt, const float* x_gt_level, const float* x_rendered,
                                float tau_f, const float* uniforms, int n_samples, float* r, float* r_level,
