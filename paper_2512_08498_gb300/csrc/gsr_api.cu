@@ -111,6 +111,7 @@ struct gsr_ctx {
     int device = 0;
     int num_sms = 0;
     std::string err;
+    DevMem row_work;   // lists by tile rows: see row_lists_layout
     DevMem tmp_keys, tmp_vals, hist, grad_rec, bwd_queue, dup_rows, ins_scratch, freq_scratch, merge_scratch;
     struct Fft { DevMem twiddles; FftPlan plan; };
     std::map<int, Fft> fft;   // transform length -> W_n^t table and passes
@@ -209,6 +210,7 @@ struct gsr_saved {
     // starts (-1: one region).
     float prefix = 1.0f;
     int64_t region2 = -1;
+    bool row_lists = false;              // the last forward's lists were made by tile rows (tile_key is scratch)
     unsigned char* host_ctrl = nullptr;  // pinned mirror of the control block head
     // Recycling.  reusable: the state's only work is that of forwards and
     // backwards on one stream outside a capture (anything else frees it when it
@@ -565,6 +567,44 @@ static float choose_prefix(const unsigned long long* H, const unsigned long long
     return best_b < kSatBuckets && best <= kTake * one ? (float)sat_edge(best_b) : 1.0f;
 }
 
+// Lists by tile rows: the runs of the records' tiles are sorted by tile row and
+// expanded into the lists, instead of expanding and sorting the instances.  It
+// takes the batches of 65536 records and more (fewer are bound by launches, of
+// which it has four more: 10 us of a 240 us step on 10k records) whose views are
+// at most kRowListMaxTiles tiles wide; and not the allocation-free forward.
+constexpr int64_t kRowListMinRecords = 65536;
+static bool use_row_lists(const Table& T)
+{
+    return T.n_records >= kRowListMinRecords && row_list_stride(T) <= kRowListMaxTiles;
+}
+
+// Its scratch in gsr_ctx::row_work; returns the bytes.
+static size_t row_lists_layout(const Table& T, int64_t row_cap, unsigned char* base, RowListArgs* a)
+{
+    size_t at = 0;
+    auto take = [&](size_t bytes) {
+        unsigned char* p = base + at;
+        at += (bytes + 255) & ~(size_t)255;
+        return p;
+    };
+    const size_t rows = (size_t)row_list_rows(T), chunks = (size_t)row_list_chunks(T, row_cap);
+    const size_t stride = (size_t)row_list_stride(T);
+    unsigned char *range = take(rows * 8), *cfirst = take(rows * 4), *rfirst = take(rows * 4);
+    unsigned char *tfirst = take((size_t)T.n_tiles * 8), *crow = take(chunks * 4), *ccount = take(chunks * stride * 4);
+    if (a) {
+        a->row_range = reinterpret_cast<uint2*>(range);
+        a->chunk_first = reinterpret_cast<uint32_t*>(cfirst);
+        a->row_first = reinterpret_cast<uint32_t*>(rfirst);
+        a->tile_first = reinterpret_cast<uint2*>(tfirst);
+        a->chunk_row = reinterpret_cast<uint32_t*>(crow);
+        a->chunk_count = reinterpret_cast<uint32_t*>(ccount);
+        a->n_trows = (int64_t)rows;
+        a->chunk_cap = (int64_t)chunks;
+        a->stride = (int)stride;
+    }
+    return at;
+}
+
 // Words of a bit array over n tiles (or blocks).
 static size_t open_words(int64_t n) { return (size_t)((std::max<int64_t>(n, 1) + 31) / 32); }
 
@@ -587,6 +627,8 @@ static gsr_status size_saved(gsr_ctx* ctx, gsr_saved* s, const Table& T)
     if (s->row_cap == 0 || grown)
         s->row_cap = std::max<int64_t>(s->row_cap,
                                        std::max<int64_t>(std::max<int64_t>(s->inst_cap / 2, 2 * s->rec_cap), 1 << 18));
+    // (the runs' keys and order are sorted in list-sized buffers)
+    s->inst_cap = std::max<int64_t>(s->inst_cap, s->row_cap);
     const int64_t rc = s->rec_cap, ic = s->inst_cap;
     if ((e = s->rec.ensure((size_t)rc * kRecordBytes)) != cudaSuccess) return cuda_fail(ctx, e, "alloc records");
     if ((e = s->vis_key.ensure((size_t)rc * 4)) != cudaSuccess) return cuda_fail(ctx, e, "alloc keys");
@@ -619,6 +661,9 @@ static gsr_status size_saved(gsr_ctx* ctx, gsr_saved* s, const Table& T)
     if ((e = ctx->tmp_vals.ensure((size_t)tmp * 4)) != cudaSuccess) return cuda_fail(ctx, e, "alloc sort scratch");
     if ((e = ctx->hist.ensure((size_t)256 * (ctx->hist_blocks + 1) * 4)) != cudaSuccess) return cuda_fail(ctx, e, "alloc histogram");
     if ((e = ctx->dup_rows.ensure((size_t)s->row_cap * 16)) != cudaSuccess) return cuda_fail(ctx, e, "alloc tile rows");
+    if (use_row_lists(T) &&
+        (e = ctx->row_work.ensure(row_lists_layout(T, s->row_cap, nullptr, nullptr))) != cudaSuccess)
+        return cuda_fail(ctx, e, "alloc row lists");
     return GSR_OK;
 }
 
@@ -679,7 +724,9 @@ static void enqueue_forward(gsr_ctx* ctx, gsr_saved* s, const gsr_gaussians* g, 
     // histograms): taken by forwards that synchronise, the only ones whose
     // statistics are read back
     const bool hist = ctx->cfg.list_prefix == 0.0f && !(ctx->cfg.flags & GSR_FLAG_NO_SYNC);
-    const int bits = tile_bits(T.n_tiles);
+    const bool by_rows = use_row_lists(T);
+    s->row_lists = by_rows;
+    const int bits = tile_bits(by_rows ? row_list_rows(T) : T.n_tiles);
     const int passes = (bits + 7) / 8;
     BlendFwdArgs ba;
     ba.rec = s->rec.as<float4>();
@@ -742,11 +789,45 @@ static void enqueue_forward(gsr_ctx* ctx, gsr_saved* s, const gsr_gaussians* g, 
         if (second) prof_extend(pr, {GSR_PHASE_DUPLICATE, GSR_PHASE_TILE_SORT, GSR_PHASE_RANGES, GSR_PHASE_BLEND_FWD});
         const int m0 = second ? 6 : 2;   // first profiling mark of these phases
         prof_mark(pr, m0, st);
-        launch_duplicate(T, da, ctx->num_sms, st);
-        prof_mark(pr, m0 + 1, st);
-        radix_sort_pairs(xk, xv, yk, yv, false, inst_count, s->inst_cap, bits, rs, st);
-        prof_mark(pr, m0 + 2, st);
-        launch_ranges(rk, inst_count, s->inst_cap, s->ranges.as<uint2>(), T.n_tiles, base, status, ctx->num_sms, st);
+        if (by_rows) {
+            // runs: keys in the list region's key array, the sort's other keys
+            // (and before it the counts) in tmp_keys, the order in tmp_vals
+            // after the last pass (through the list array, filled last)
+            uint32_t *tk = ctx->tmp_keys.as<uint32_t>(), *tv = ctx->tmp_vals.as<uint32_t>();
+            uint32_t *v0 = (passes & 1) ? rv : tv, *v1 = (passes & 1) ? tv : rv;
+            da.counts = reinterpret_cast<uint2*>(tk);
+            da.row_key = rk;
+            da.runs = ctx->dup_rows.as<uint2>();
+            da.n_rows = counters + (second ? kCntRuns2 : kCntRuns);
+            launch_duplicate(T, da, ctx->num_sms, st);
+            prof_mark(pr, m0 + 1, st);
+            radix_sort_pairs(rk, v0, tk, v1, true, da.n_rows, s->row_cap, bits, rs, st);
+            prof_mark(pr, m0 + 2, st);
+            RowListArgs ra{};
+            row_lists_layout(T, s->row_cap, ctx->row_work.as<unsigned char>(), &ra);
+            ra.n_rows = da.n_rows;
+            ra.order = tv;
+            ra.runs = da.runs;
+            ra.sorted = ctx->dup_rows.as<uint2>() + s->row_cap;
+            ra.n_chunks = reinterpret_cast<uint32_t*>(counters + kCntChunks);
+            ra.ticket = ra.n_chunks + 1;
+            ra.vals = s->tile_val.as<uint32_t>();
+            ra.ranges = s->ranges.as<uint2>();
+            ra.open_tiles = da.open_tiles;
+            ra.status = status;
+            ra.inst_cap = s->inst_cap;
+            ra.base = (uint32_t)base;
+            cudaMemsetAsync(ra.row_range, 0, (size_t)ra.n_trows * 8, st);
+            launch_ranges((passes & 1) ? tk : rk, da.n_rows, s->row_cap, ra.row_range, ra.n_trows, 0, status,
+                          ctx->num_sms, st);
+            launch_row_lists(T, ra, ctx->num_sms, st);
+        } else {
+            launch_duplicate(T, da, ctx->num_sms, st);
+            prof_mark(pr, m0 + 1, st);
+            radix_sort_pairs(xk, xv, yk, yv, false, inst_count, s->inst_cap, bits, rs, st);
+            prof_mark(pr, m0 + 2, st);
+            launch_ranges(rk, inst_count, s->inst_cap, s->ranges.as<uint2>(), T.n_tiles, base, status, ctx->num_sms, st);
+        }
         ba.round = r;
         ba.work = reinterpret_cast<unsigned int*>(ctrl + (second ? kCtrlWorkFwd2 : kCtrlWorkFwd));
         prof_mark(pr, m0 + 3, st);
@@ -1409,6 +1490,12 @@ gsr_status gsr_debug_lists(gsr_saved* s, uint64_t* keys, uint32_t* vals, uint32_
 {
     if (!s || !s->filled) return GSR_ERR_INVALID_ARG;
     s->reusable = false;   // its buffers are read on any stream
+    if (s->row_lists && keys) {
+        // lists by tile rows keep no tile keys: written here from the ranges
+        cudaMemsetAsync(s->tile_key.p, 0, s->tile_key.bytes, static_cast<cudaStream_t>(stream));
+        launch_tile_keys(s->ranges.as<uint2>(), s->table.n_tiles, s->tile_key.as<uint32_t>(),
+                         static_cast<cudaStream_t>(stream));
+    }
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     DebugArgs a{};
     a.tile_key = s->tile_key.as<uint32_t>();
@@ -1432,6 +1519,12 @@ gsr_status gsr_debug_list_slice(gsr_saved* s, int64_t first, int64_t count, uint
 {
     if (!s || !s->filled || first < 0 || count < 0) return GSR_ERR_INVALID_ARG;
     s->reusable = false;   // its buffers are read on any stream
+    if (s->row_lists && keys) {
+        // lists by tile rows keep no tile keys: written here from the ranges
+        cudaMemsetAsync(s->tile_key.p, 0, s->tile_key.bytes, static_cast<cudaStream_t>(stream));
+        launch_tile_keys(s->ranges.as<uint2>(), s->table.n_tiles, s->tile_key.as<uint32_t>(),
+                         static_cast<cudaStream_t>(stream));
+    }
     DebugArgs a{};
     a.tile_key = s->tile_key.as<uint32_t>();
     a.tile_val = s->tile_val.as<uint32_t>();

@@ -44,6 +44,9 @@ enum : int {
     kCntFullInst = 7,    // instances of the 3-sigma rectangles (the lists before tile culling)
     kCntInstances2 = 8,  // kept instances of the second round of a two-round forward
     kCntOpenTiles = 9,   // tiles the first round of a two-round forward left open
+    kCntRuns = 10,       // runs of the list round by tile rows (0 after an overflow)
+    kCntRuns2 = 11,      // the same for the second round
+    kCntChunks = 12,     // their chunks (u32) and the placement's ticket (u32)
     kCntSlots = 16,
 };
 
@@ -193,7 +196,42 @@ struct DuplicateArgs {
     // [kSatBuckets] if set (an unfiltered emission of every record): the
     // kept instances of the records of depth share in each saturation bucket
     unsigned long long* inst_hist = nullptr;
+    // lists by tile rows (launch_row_lists): the runs and their tile row ids
+    // instead of the expanded instances
+    uint32_t* row_key = nullptr;            // [row_cap]
+    uint2* runs = nullptr;                  // [row_cap] {record, first column | count << 16}
+    unsigned long long* n_rows = nullptr;   // runs written (0 after an overflow)
 };
+
+// Tile lists from depth-ordered runs sorted by tile row (see gsr_sort.cu).
+constexpr int kRowListMaxTiles = 1024;      // tile columns of a view (4 bytes of row_count's shared memory per warp)
+constexpr int64_t kRowChunksMin = 8192;     // chunks wanted of small run counts
+struct RowListArgs {
+    const unsigned long long* n_rows;
+    const uint32_t* order;         // [n_rows] run index in sorted order
+    const uint2* runs;             // [row_cap] by run index
+    uint2* sorted;                 // [row_cap] scratch: the runs in sorted order
+    uint2* row_range;              // [n_trows] the tile rows' runs (zero: none)
+    uint32_t* chunk_first;         // [n_trows]
+    uint32_t* row_first;           // [n_trows]
+    uint32_t* chunk_row;           // [chunk_cap]
+    uint32_t* chunk_count;         // [chunk_cap][stride]
+    uint2* tile_first;             // [n_tiles] {offset in the tile row's instances, count}
+    uint32_t* n_chunks;
+    uint32_t* ticket;              // set to zero by the plan
+    uint32_t* vals;                // list positions from 0: the region's start is in base
+    uint2* ranges;
+    const uint32_t* open_tiles;    // a second round lists these only
+    uint32_t* status;
+    int64_t n_trows, chunk_cap, inst_cap;
+    uint32_t base;                 // first list position of the region
+    int stride;                    // most tile columns of a view
+};
+int row_list_stride(const Table& T);
+int64_t row_list_rows(const Table& T);
+int64_t row_list_chunks(const Table& T, int64_t row_cap);
+void launch_row_lists(const Table& T, const RowListArgs& a, int num_sms, cudaStream_t s);
+void launch_tile_keys(const uint2* ranges, int64_t n_tiles, uint32_t* keys, cudaStream_t s);
 void launch_duplicate(const Table& T, const DuplicateArgs& a, int num_sms, cudaStream_t s);
 int64_t duplicate_blocks(int64_t rec_cap);     // look-back words of the scan
 int64_t duplicate_windows(int64_t inst_cap);   // win_cap for inst_cap kept instances

@@ -15,6 +15,8 @@
 // The radix passes are in gsr_radix.cu.  The instance emission uses a
 // single-pass decoupled look-back scan over the tile counts and spreads each
 // block's instances evenly over its threads.
+#include <algorithm>
+
 #include "gsr_common.cuh"
 #include "gsr_kernels.h"
 
@@ -155,13 +157,18 @@ __device__ __forceinline__ int dup_run(const Table& Tb, const DupRec& d, int ty,
 struct ViewTiles {
     int64_t base[kMaxViews];
     uint32_t tx[kMaxViews];
+    uint32_t row[kMaxViews];   // first tile row, the views' rows numbered through
 };
 
-__device__ __forceinline__ void load_view_tiles(const Table& Tb, ViewTiles& vt)
+__device__ __forceinline__ void load_view_tiles(const Table& Tb, ViewTiles& vt, int threads = kDupThreads)
 {
-    for (int v = threadIdx.x; v < Tb.n_views; v += kDupThreads) {
+    for (int v = threadIdx.x; v < Tb.n_views; v += threads) {
         vt.base[v] = Tb.v[v].tile_base;
         vt.tx[v] = (uint32_t)Tb.v[v].TX;
+    }
+    if (threadIdx.x == 0) {
+        uint32_t r = 0;
+        for (int v = 0; v < Tb.n_views; ++v) { vt.row[v] = r; r += (uint32_t)Tb.v[v].TY; }
     }
     __syncthreads();
 }
@@ -245,6 +252,11 @@ dup_scan_kernel(DuplicateArgs a)
         if (ti > (unsigned long long)a.inst_cap) atomicOr(a.status, kErrInstCapacity);
         if (tr > (unsigned long long)a.row_cap) atomicOr(a.status, kErrFullCapacity);
         if (emission_overflows(a)) atomicOr(a.status, kErrOverflow32);
+        // the run list of an emission that fits (none after an overflow: the
+        // call reports it)
+        if (a.n_rows)
+            *a.n_rows = ti > (unsigned long long)a.inst_cap || tr > (unsigned long long)a.row_cap || emission_overflows(a)
+                            ? 0ull : tr;
     }
     if (emission_overflows(a)) return;
     const int64_t n = emission_records(a);
@@ -302,6 +314,9 @@ dup_scan_kernel(DuplicateArgs a)
 // One thread per depth-ordered record: its kept rows' descriptors at its row
 // base and the window index (bases from dup_scan; instance and row positions
 // stay below 2^32 or the call reports an overflow).
+// RUNS: the runs for the lists by tile rows (tile row id as key, {record, first
+// column, count} as value) instead of the expansion's descriptors.
+template <bool RUNS>
 __global__ void __launch_bounds__(kDupThreads)
 dup_rows_kernel(const __grid_constant__ Table Tb, DuplicateArgs a)
 {
@@ -343,8 +358,17 @@ dup_rows_kernel(const __grid_constant__ Table Tb, DuplicateArgs a)
             const uint32_t t0 = (uint32_t)(tbase + (int64_t)ty * TX + first);
             // a second round's row lists the open tiles of the run only; its
             // descriptor keeps the run's first tile id
+            const int run = cnt;
             if (a.open_tiles) cnt = open_count(a.open_tiles, t0, cnt);
             if (cnt == 0) continue;
+            if constexpr (RUNS) {
+                if (rb < (unsigned long long)a.row_cap) {
+                    a.row_key[rb] = s_vt.row[d.view] + (uint32_t)ty;
+                    a.runs[rb] = make_uint2(k, (uint32_t)first | ((uint32_t)run << 16));
+                }
+                ++rb;
+                continue;
+            }
             if (rb < (unsigned long long)a.row_cap) {
                 a.rows[rb] = make_uint4(k, t0, (uint32_t)cnt, (uint32_t)ib);
                 // windows whose first instance lies in [ib, ib + cnt)
@@ -485,11 +509,419 @@ void launch_duplicate(const Table& T, const DuplicateArgs& a, int num_sms, cudaS
     GSR_COUNT_LAUNCH();
     dup_scan_kernel<<<(unsigned)sblocks, kDupThreads, 0, s>>>(a);
     GSR_COUNT_LAUNCH();
-    dup_rows_kernel<<<(unsigned)cblocks, kDupThreads, 0, s>>>(T, a);
+    if (a.runs) {
+        dup_rows_kernel<true><<<(unsigned)cblocks, kDupThreads, 0, s>>>(T, a);
+        return;   // the lists are made from the runs (launch_row_lists)
+    }
+    dup_rows_kernel<false><<<(unsigned)cblocks, kDupThreads, 0, s>>>(T, a);
     int64_t wblocks = duplicate_windows(a.inst_cap);
     if (wblocks > (int64_t)num_sms * 8) wblocks = (int64_t)num_sms * 8;
     GSR_COUNT_LAUNCH();
     dup_expand_kernel<<<(unsigned)wblocks, kDupThreads, 0, s>>>(a, (uint32_t)T.n_tiles);
+}
+
+// ---------------------------------------------------------------------------
+// lists by tile rows
+//
+// A record's kept tiles are runs, one per tile row, and there are several times
+// fewer runs than instances (2.7 on the six-camera rig, 10 on the 500k-Gaussian
+// 1080p view).  So instead of expanding the runs and sorting the instances by
+// tile, the runs are sorted by tile row (stable: depth order inside a row) and
+// each row's runs are expanded straight into its tiles' lists:
+//   row_plan    chunks of CH consecutive runs of one tile row (CH from the run
+//               count, so that small batches have enough chunks);
+//   row_count   per chunk: the runs in sorted order written back to back, and
+//               how many cover each tile column (differences, then a scan);
+//   row_scan    per tile row and column: the chunks' counts become offsets
+//               inside the tile's list, and the tiles' counts offsets inside the
+//               tile row's instances;
+//   row_offsets the tile rows' offsets in the list;
+//   row_place   the chunks' records appended to the lists of their tiles; the
+//               first chunk of a tile row writes the row's ranges.
+// The instances are written once (4 bytes) and never read back before the
+// blend.
+// ---------------------------------------------------------------------------
+constexpr int kRowWarps = 8;        // warps per block of row_count and row_place
+constexpr int kChunkMin = 32, kChunkMax = 4096;
+
+// CH runs per chunk: a power of two, at most about kRowChunksMin chunks while
+// it is below kChunkMax.
+__device__ __forceinline__ int row_chunk(int64_t n)
+{
+    int c = kChunkMin;
+    while (c < kChunkMax && n / c > kRowChunksMin) c *= 2;
+    return c;
+}
+
+__global__ void __launch_bounds__(1024)
+row_plan_kernel(RowListArgs a)
+{
+    __shared__ uint32_t s_warp[32];
+    __shared__ uint32_t s_total;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int64_t n = (int64_t)*a.n_rows;
+    const int ch = row_chunk(n);
+    uint32_t carry = 0;
+    for (int64_t r0 = 0; r0 < a.n_trows; r0 += 1024) {
+        const int64_t r = r0 + tid;
+        uint32_t c = 0;
+        if (r < a.n_trows && n > 0) {
+            const uint2 g = a.row_range[r];
+            c = (g.y - g.x + (uint32_t)ch - 1u) / (uint32_t)ch;
+        }
+        uint32_t incl = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) s_warp[wid] = incl;
+        __syncthreads();
+        if (wid == 0) {
+            const uint32_t x = s_warp[lane];
+            uint32_t ix = x;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xffffffffu, ix, o);
+                if (lane >= o) ix += t;
+            }
+            s_warp[lane] = ix - x;
+            if (lane == 31) s_total = ix;
+        }
+        __syncthreads();
+        const uint32_t first = carry + s_warp[wid] + incl - c;
+        if (r < a.n_trows) a.chunk_first[r] = first;
+        for (uint32_t i = 0; i < c; ++i)
+            if (first + i < (uint32_t)a.chunk_cap) a.chunk_row[first + i] = (uint32_t)r;
+        carry += s_total;
+        __syncthreads();
+    }
+    if (tid == 0) {
+        if (carry > (uint32_t)a.chunk_cap) atomicOr(a.status, kErrInternal);
+        *a.n_chunks = carry > (uint32_t)a.chunk_cap ? 0u : carry;
+        *a.ticket = 0u;
+    }
+}
+
+// The tile row r: its view, first tile id and column count.
+struct TileRow {
+    uint32_t first_tile;
+    int tx;
+};
+__device__ __forceinline__ TileRow tile_row(const ViewTiles& vt, const Table& Tb, uint32_t r)
+{
+    int v = 0, hi = Tb.n_views - 1;
+    while (v < hi) {
+        const int mid = (v + hi + 1) >> 1;
+        if (vt.row[mid] <= r) v = mid; else hi = mid - 1;
+    }
+    TileRow t;
+    t.tx = (int)vt.tx[v];
+    t.first_tile = (uint32_t)(vt.base[v] + (int64_t)(r - vt.row[v]) * vt.tx[v]);
+    return t;
+}
+
+// The runs [i0, i1) of chunk c of tile row r.
+__device__ __forceinline__ void chunk_runs(const RowListArgs& a, uint32_t c, uint32_t r, int ch, uint32_t& i0, uint32_t& i1)
+{
+    const uint2 g = a.row_range[r];
+    i0 = g.x + (c - a.chunk_first[r]) * (uint32_t)ch;
+    i1 = min(g.y, i0 + (uint32_t)ch);
+}
+
+__device__ __forceinline__ bool tile_open(const uint32_t* __restrict__ m, uint32_t t)
+{
+    return !m || ((m[t >> 5] >> (t & 31u)) & 1u);
+}
+
+__global__ void __launch_bounds__(32 * kRowWarps)
+row_count_kernel(const __grid_constant__ Table Tb, RowListArgs a)
+{
+    extern __shared__ int s_diff[];   // [kRowWarps][stride + 1]
+    __shared__ ViewTiles s_vt;
+    load_view_tiles(Tb, s_vt, 32 * kRowWarps);
+    const int lane = threadIdx.x & 31;
+    int* diff = s_diff + (threadIdx.x >> 5) * (a.stride + 1);
+    const int ch = row_chunk((int64_t)*a.n_rows);
+    const uint32_t nc = *a.n_chunks;
+    for (uint32_t c = blockIdx.x * kRowWarps + (threadIdx.x >> 5); c < nc; c += gridDim.x * kRowWarps) {
+        const uint32_t r = a.chunk_row[c];
+        const TileRow tr = tile_row(s_vt, Tb, r);
+        uint32_t i0, i1;
+        chunk_runs(a, c, r, ch, i0, i1);
+        for (int x = lane; x <= tr.tx; x += 32) diff[x] = 0;
+        __syncwarp();
+        // four gathers in flight per lane
+        for (uint32_t i = i0 + lane; i < i1; i += 128) {
+            uint32_t o[4];
+            uint2 d[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) o[u] = i + 32u * u < i1 ? a.order[i + 32u * u] : 0u;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) d[u] = i + 32u * u < i1 ? a.runs[o[u]] : make_uint2(0u, 0u);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (i + 32u * u >= i1) break;
+                a.sorted[i + 32u * u] = d[u];
+                const int x0 = min((int)(d[u].y & 0xffffu), tr.tx), x1 = min(x0 + (int)(d[u].y >> 16), tr.tx);
+                atomicAdd(diff + x0, 1);
+                atomicAdd(diff + x1, -1);
+            }
+        }
+        __syncwarp();
+        int carry = 0;
+        uint32_t* out = a.chunk_count + (size_t)c * a.stride;
+        for (int x0 = 0; x0 < tr.tx; x0 += 32) {
+            const int x = x0 + lane;
+            int v = x < tr.tx ? diff[x] : 0;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += t;
+            }
+            v += carry;
+            carry = __shfl_sync(0xffffffffu, v, 31);
+            if (x < tr.tx) out[x] = tile_open(a.open_tiles, tr.first_tile + (uint32_t)x) ? (uint32_t)v : 0u;
+        }
+        __syncwarp();
+    }
+}
+
+constexpr int kScanThreads = 256;
+__global__ void __launch_bounds__(kScanThreads)
+row_scan_kernel(const __grid_constant__ Table Tb, RowListArgs a)
+{
+    __shared__ ViewTiles s_vt;
+    __shared__ unsigned long long s_warp[kDupThreads / 32];
+    load_view_tiles(Tb, s_vt, kScanThreads);
+    static_assert(kScanThreads == kDupThreads, "block_excl_scan64");
+    const uint32_t nc = *a.n_chunks;
+    const int ch = row_chunk((int64_t)*a.n_rows);
+    for (int64_t r = blockIdx.x; r < a.n_trows; r += gridDim.x) {
+        const TileRow tr = tile_row(s_vt, Tb, (uint32_t)r);
+        const uint2 g = a.row_range[r];
+        const uint32_t n = nc ? (g.y - g.x + (uint32_t)ch - 1u) / (uint32_t)ch : 0u;
+        uint32_t* base = a.chunk_count + (size_t)a.chunk_first[r] * a.stride;
+        unsigned long long carry = 0;
+        for (int x0 = 0; x0 < tr.tx; x0 += kScanThreads) {
+            const int x = x0 + (int)threadIdx.x;
+            uint32_t run = 0;
+            if (x < tr.tx) {
+                uint32_t* p = base + x;
+                uint32_t i = 0;
+                for (; i + 8 <= n; i += 8) {   // eight loads in flight
+                    uint32_t v[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) v[u] = p[(size_t)(i + u) * a.stride];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) { p[(size_t)(i + u) * a.stride] = run; run += v[u]; }
+                }
+                for (; i < n; ++i) { const uint32_t v = p[(size_t)i * a.stride]; p[(size_t)i * a.stride] = run; run += v; }
+            }
+            unsigned long long total;
+            const unsigned long long ex = block_excl_scan64(run, s_warp, &total);
+            if (x < tr.tx) {
+                const uint32_t first = (uint32_t)(carry + ex);
+                a.tile_first[tr.first_tile + x] = make_uint2(first, run);
+            }
+            carry += total;
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) a.row_first[r] = (uint32_t)carry;   // row_offsets turns the totals into offsets
+    }
+}
+
+__global__ void __launch_bounds__(1024)
+row_offsets_kernel(RowListArgs a)
+{
+    __shared__ uint32_t s_warp[32];
+    __shared__ uint32_t s_total;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    uint32_t carry = a.base;
+    for (int64_t r0 = 0; r0 < a.n_trows; r0 += 1024) {
+        const int64_t r = r0 + tid;
+        const uint32_t c = r < a.n_trows ? a.row_first[r] : 0u;
+        uint32_t incl = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) s_warp[wid] = incl;
+        __syncthreads();
+        if (wid == 0) {
+            const uint32_t x = s_warp[lane];
+            uint32_t ix = x;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xffffffffu, ix, o);
+                if (lane >= o) ix += t;
+            }
+            s_warp[lane] = ix - x;
+            if (lane == 31) s_total = ix;
+        }
+        __syncthreads();
+        if (r < a.n_trows) a.row_first[r] = carry + s_warp[wid] + incl - c;
+        carry += s_total;
+        __syncthreads();
+    }
+}
+
+// Bits [0, n) of a word, n <= 32.
+__device__ __forceinline__ uint32_t low_bits(int n) { return (uint32_t)((1ull << n) - 1ull); }
+
+// 32 x 32 bit transpose over the warp: lane c's bit r becomes what lane r's
+// bit c was (halves, quarters, ... exchanged between lanes).
+__device__ __forceinline__ uint32_t transpose_bits(uint32_t x, int lane)
+{
+    constexpr uint32_t kKeep[5] = {0x0000ffffu, 0x00ff00ffu, 0x0f0f0f0fu, 0x33333333u, 0x55555555u};
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const int s = 16 >> i;
+        const uint32_t k = kKeep[i], y = __shfl_xor_sync(0xffffffffu, x, s);
+        x = (lane & s) ? ((x & ~k) | ((y & ~k) >> s)) : ((x & k) | ((y & k) << s));
+    }
+    return x;
+}
+
+// One warp per chunk and group of 32 tile columns, a column per lane.  Of 32
+// runs at a time, each lane turns one run into the bits of the columns it
+// covers; transposed, a lane has the runs that cover its column, in order, and
+// appends their records to its list.  Eight entries are collected in shared
+// memory until they fill an aligned 32-byte sector (stores of 4 bytes to a sector
+// per lane, one run at a time: 870 us on the 500k-Gaussian 1080p view's 74 M
+// entries, 214 on the rig's 19 M; a run at a time with the sectors collected:
+// 504 and 362).
+__global__ void __launch_bounds__(32 * kRowWarps)
+row_place_kernel(const __grid_constant__ Table Tb, RowListArgs a)
+{
+    __shared__ ViewTiles s_vt;
+    __shared__ uint32_t s_pend[kRowWarps][32][32];   // pending entries by position & 31, per lane
+    __shared__ uint32_t s_rec[kRowWarps][32];
+    load_view_tiles(Tb, s_vt, 32 * kRowWarps);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t(*pend)[32] = s_pend[w];
+    const int ch = row_chunk((int64_t)*a.n_rows);
+    const uint32_t groups = (uint32_t)(a.stride + 31) / 32u;
+    const unsigned long long items = (unsigned long long)*a.n_chunks * groups;
+    const unsigned long long end = (unsigned long long)a.base + (unsigned long long)a.inst_cap;
+    // items from a queue: their work varies with the runs per column (one hot
+    // column of 32 makes 32 steps of 32 runs)
+    for (;;) {
+        unsigned long long it = 0;
+        if (lane == 0) it = atomicAdd(a.ticket, 1u);
+        it = __shfl_sync(0xffffffffu, it, 0);
+        if (it >= items) break;
+        const uint32_t c = (uint32_t)(it / groups);
+        const int c0 = (int)(it % groups) * 32, x = c0 + lane;
+        const uint32_t r = a.chunk_row[c];
+        const TileRow tr = tile_row(s_vt, Tb, r);
+        if (c0 >= tr.tx) continue;
+        uint32_t i0, i1;
+        chunk_runs(a, c, r, ch, i0, i1);
+        uint32_t first = 0;
+        bool listed = false;
+        if (x < tr.tx) {
+            const uint2 t = a.tile_first[tr.first_tile + x];
+            const uint32_t at = a.row_first[r] + t.x;
+            first = at + a.chunk_count[(size_t)c * a.stride + x];
+            if (c == a.chunk_first[r] && t.y) a.ranges[tr.first_tile + x] = make_uint2(at, at + t.y);
+            listed = tile_open(a.open_tiles, tr.first_tile + (uint32_t)x);
+        }
+        uint32_t p = first, done = first;   // entries appended and written up to here
+        auto write = [&](uint32_t hi) {     // [done, hi) one by one
+            for (; done < hi; ++done)
+                if ((unsigned long long)done < end) a.vals[done] = pend[done & 31u][lane];
+        };
+        uint2 d = i0 + lane < i1 ? a.sorted[i0 + lane] : make_uint2(0u, 0u);
+        for (uint32_t i = i0; i < i1; i += 32) {
+            const int x0 = (int)(d.y & 0xffffu) - c0, x1 = x0 + (int)(d.y >> 16);   // (an empty run past the end)
+            uint32_t word = low_bits(min(max(x1, 0), 32)) & ~low_bits(min(max(x0, 0), 32));
+            s_rec[w][lane] = d.x;
+            if (i + 32u + lane < i1) d = a.sorted[i + 32 + lane];
+            else d = make_uint2(0u, 0u);
+            word = transpose_bits(word, lane);
+            if (!listed) word = 0u;
+            __syncwarp();
+            // sixteen runs at a time, so that at most 7 + 16 entries are pending
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                uint32_t m = half ? word & 0xffff0000u : word & 0xffffu;
+                // branch-free: a lane without a run left writes its next place
+                // and does not advance
+                while (__any_sync(0xffffffffu, m != 0u)) {
+                    pend[p & 31u][lane] = s_rec[w][(__ffs(m) - 1) & 31];
+                    p += m != 0u ? 1u : 0u;
+                    m &= m - 1u;
+                }
+                while (__any_sync(0xffffffffu, (p >> 3) != (done >> 3))) {
+                    if ((p >> 3) != (done >> 3)) {
+                        if ((done & 7u) == 0u && (unsigned long long)done + 8ull <= end) {
+                            const uint32_t(*q)[32] = pend + (done & 31u);
+                            uint4* o = reinterpret_cast<uint4*>(a.vals + done);
+                            o[0] = make_uint4(q[0][lane], q[1][lane], q[2][lane], q[3][lane]);
+                            o[1] = make_uint4(q[4][lane], q[5][lane], q[6][lane], q[7][lane]);
+                            done += 8u;
+                        } else {
+                            write((done | 7u) + 1u);
+                        }
+                    }
+                }
+            }
+            __syncwarp();   // the records are rewritten by the next 32 runs
+        }
+        write(p);
+    }
+}
+
+// Positions of each tile's range get the tile's id (for the parity exports).
+__global__ void tile_keys_kernel(const uint2* __restrict__ ranges, int64_t n_tiles, uint32_t* __restrict__ keys)
+{
+    for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+        const uint2 g = ranges[t];
+        for (uint32_t i = g.x + threadIdx.x; i < g.y; i += blockDim.x) keys[i] = (uint32_t)t;
+    }
+}
+
+void launch_tile_keys(const uint2* ranges, int64_t n_tiles, uint32_t* keys, cudaStream_t s)
+{
+    GSR_COUNT_LAUNCH();
+    tile_keys_kernel<<<(unsigned)std::min<int64_t>(std::max<int64_t>(n_tiles, 1), 65535), 128, 0, s>>>(ranges, n_tiles, keys);
+}
+
+int row_list_stride(const Table& T)
+{
+    int tx = 1;
+    for (int v = 0; v < T.n_views; ++v) tx = std::max(tx, T.v[v].TX);
+    return tx;
+}
+
+int64_t row_list_rows(const Table& T)
+{
+    int64_t n = 0;
+    for (int v = 0; v < T.n_views; ++v) n += T.v[v].TY;
+    return n;
+}
+
+int64_t row_list_chunks(const Table& T, int64_t row_cap)
+{
+    return 2 * kRowChunksMin + row_cap / kChunkMax + row_list_rows(T) + 1;
+}
+
+void launch_row_lists(const Table& T, const RowListArgs& a, int num_sms, cudaStream_t s)
+{
+    const size_t smem = (size_t)kRowWarps * (a.stride + 1) * 4;
+    const unsigned blocks = (unsigned)std::min<int64_t>((a.chunk_cap + kRowWarps - 1) / kRowWarps, (int64_t)num_sms * 6);
+    GSR_COUNT_LAUNCH();
+    row_plan_kernel<<<1, 1024, 0, s>>>(a);
+    GSR_COUNT_LAUNCH();
+    row_count_kernel<<<blocks, 32 * kRowWarps, smem, s>>>(T, a);
+    GSR_COUNT_LAUNCH();
+    row_scan_kernel<<<(unsigned)std::min<int64_t>(a.n_trows, (int64_t)num_sms * 8), kScanThreads, 0, s>>>(T, a);
+    GSR_COUNT_LAUNCH();
+    row_offsets_kernel<<<1, 1024, 0, s>>>(a);
+    GSR_COUNT_LAUNCH();
+    row_place_kernel<<<blocks, 32 * kRowWarps, 0, s>>>(T, a);
 }
 
 // Four keys per thread (one 16-byte load, the keys array starts 16-byte
