@@ -539,7 +539,9 @@ void launch_duplicate(const Table& T, const DuplicateArgs& a, int num_sms, cudaS
 //   row_place   the chunks' records appended to the lists of their tiles; the
 //               first chunk of a tile row writes the row's ranges.
 // The instances are written once (4 bytes) and never read back before the
-// blend.
+// blend.  The sorted order is an index into the runs, so after a wait that gave
+// up in the sort or the scan (stale order, stale keys) every one of these
+// kernels skips its work.
 // ---------------------------------------------------------------------------
 constexpr int kRowWarps = 8;        // warps per block of row_count and row_place
 constexpr int kChunkMin = 32, kChunkMax = 4096;
@@ -556,6 +558,7 @@ __device__ __forceinline__ int row_chunk(int64_t n)
 __global__ void __launch_bounds__(1024)
 row_plan_kernel(RowListArgs a)
 {
+    if (earlier_wait_timed_out(a.status)) return;
     __shared__ uint32_t s_warp[32];
     __shared__ uint32_t s_total;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -567,7 +570,7 @@ row_plan_kernel(RowListArgs a)
         uint32_t c = 0;
         if (r < a.n_trows && n > 0) {
             const uint2 g = a.row_range[r];
-            c = (g.y - g.x + (uint32_t)ch - 1u) / (uint32_t)ch;
+            c = g.y > g.x ? (g.y - g.x + (uint32_t)ch - 1u) / (uint32_t)ch : 0u;
         }
         uint32_t incl = c;
 #pragma unroll
@@ -637,12 +640,14 @@ __device__ __forceinline__ bool tile_open(const uint32_t* __restrict__ m, uint32
 __global__ void __launch_bounds__(32 * kRowWarps)
 row_count_kernel(const __grid_constant__ Table Tb, RowListArgs a)
 {
+    if (earlier_wait_timed_out(a.status)) return;
     extern __shared__ int s_diff[];   // [kRowWarps][stride + 1]
     __shared__ ViewTiles s_vt;
     load_view_tiles(Tb, s_vt, 32 * kRowWarps);
     const int lane = threadIdx.x & 31;
     int* diff = s_diff + (threadIdx.x >> 5) * (a.stride + 1);
-    const int ch = row_chunk((int64_t)*a.n_rows);
+    const uint32_t n = (uint32_t)*a.n_rows;   // below 2^30 (dup_scan)
+    const int ch = row_chunk((int64_t)n);
     const uint32_t nc = *a.n_chunks;
     for (uint32_t c = blockIdx.x * kRowWarps + (threadIdx.x >> 5); c < nc; c += gridDim.x * kRowWarps) {
         const uint32_t r = a.chunk_row[c];
@@ -658,7 +663,7 @@ row_count_kernel(const __grid_constant__ Table Tb, RowListArgs a)
 #pragma unroll
             for (int u = 0; u < 4; ++u) o[u] = i + 32u * u < i1 ? a.order[i + 32u * u] : 0u;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) d[u] = i + 32u * u < i1 ? a.runs[o[u]] : make_uint2(0u, 0u);
+            for (int u = 0; u < 4; ++u) d[u] = i + 32u * u < i1 && o[u] < n ? a.runs[o[u]] : make_uint2(0u, 0u);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 if (i + 32u * u >= i1) break;
@@ -691,6 +696,7 @@ constexpr int kScanThreads = 256;
 __global__ void __launch_bounds__(kScanThreads)
 row_scan_kernel(const __grid_constant__ Table Tb, RowListArgs a)
 {
+    if (earlier_wait_timed_out(a.status)) return;
     __shared__ ViewTiles s_vt;
     __shared__ unsigned long long s_warp[kDupThreads / 32];
     load_view_tiles(Tb, s_vt, kScanThreads);
@@ -734,6 +740,7 @@ row_scan_kernel(const __grid_constant__ Table Tb, RowListArgs a)
 __global__ void __launch_bounds__(1024)
 row_offsets_kernel(RowListArgs a)
 {
+    if (earlier_wait_timed_out(a.status)) return;
     __shared__ uint32_t s_warp[32];
     __shared__ uint32_t s_total;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -795,6 +802,7 @@ __device__ __forceinline__ uint32_t transpose_bits(uint32_t x, int lane)
 __global__ void __launch_bounds__(32 * kRowWarps)
 row_place_kernel(const __grid_constant__ Table Tb, RowListArgs a)
 {
+    if (earlier_wait_timed_out(a.status)) return;
     __shared__ ViewTiles s_vt;
     __shared__ uint32_t s_pend[kRowWarps][32][32];   // pending entries by position & 31, per lane
     __shared__ uint32_t s_rec[kRowWarps][32];

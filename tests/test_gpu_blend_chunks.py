@@ -67,3 +67,33 @@ def test_backward_groups(n, logit, depth, tile):
     go = o.backward(up_o[0], up_o[1], up_o[2], want_grec=True)
     P.compare_grads(g, go)
     P.compare_record_grads(g, go)
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), -float("inf")])
+@pytest.mark.parametrize("depth", [False, True])
+def test_non_finite_upstream_gradient_stays_with_its_pixel(depth, bad):
+    # two small Gaussians in one 8x8 block; only the first reaches the pixel
+    # (1, 1), so the second's gradients are those of a zero there
+    sc = scenes.random_scene(7, 2, [scenes.pinhole(16, 16, f=20.0)], 0)
+    for i, u in enumerate((1.5, 6.5)):
+        sc.means[i] = ((u - 8.0) * 2.0 / 20.0, (u - 8.0) * 2.0 / 20.0, 2.0)
+    sc.log_scales[:] = (-5.0, -3.5, -3.0)
+    sc.opacity_logits[:] = 1.0
+    dev = P.device()
+    r = Rasterizer(sh_degree=0, bg=sc.bg, device=dev)
+    params, cams = P.params_of(sc, dev), to_camera_views(sc.views, dev)
+    _, _, alpha, saved = r.forward(params, cams)
+    assert float(alpha[17]) > 0.1 and float(alpha[6 * 16 + 6]) > 0.1
+    g = torch.Generator(device=dev)
+    g.manual_seed(3)
+    up_rgb, up_dep = torch.randn(3 * 256, generator=g, device=dev), torch.randn(256, generator=g, device=dev)
+    got = []
+    for value in (0.0, bad):
+        d_rgb, d_dep = up_rgb.clone(), up_dep.clone()
+        d_rgb[17] = d_dep[17] = value
+        got.append(r.backward(params, cams, saved, d_rgb, d_dep if depth else None)[:5])
+    for a, b in zip(*got):
+        # the same terms but for the exponential's rounding (16 ulp at most, 1e-6),
+        # in sums that cancel to no less than a hundredth
+        assert torch.allclose(a[1], b[1], rtol=1e-4, atol=1e-4 * float(a[1].abs().max()))
+    assert not bool(torch.isfinite(got[1][4][0]).all())

@@ -12,6 +12,7 @@ if not torch.cuda.is_available():  # pragma: no cover - CPU machines
     pytest.skip("no CUDA device", allow_module_level=True)
 
 import oracle  # noqa: E402
+from paper_2512_08498_gb300 import _lib as L  # noqa: E402
 from paper_2512_08498_gb300 import scenes  # noqa: E402
 from paper_2512_08498_gb300.rasterizer import Rasterizer, to_camera_views  # noqa: E402
 
@@ -66,3 +67,20 @@ def test_two_rounds_and_growth(prefix):
             else:
                 # the order of the backward's atomic additions
                 assert float((a - b).norm()) <= 1e-6 * float(a.norm()), k
+
+
+def test_timeout_skips_the_row_lists():
+    # an earlier kernel's wait gives up: the lists' kernels skip their work, the
+    # call reports it, and the next one renders
+    sc = _scene((16, 16))
+    dev = P.device()
+    params, cams = P.params_of(sc, dev), to_camera_views(sc.views, dev)
+    r = Rasterizer(sh_degree=0, device=dev)
+    want = [t.clone() for t in r.forward(params, cams)[:3]]
+    r.debug_set_wait(wait_ns=200_000, withhold_prefix=True)
+    with pytest.raises(L.GsrError) as e:
+        r.forward(params, cams)
+    assert e.value.code == L.GSR_ERR_TIMEOUT
+    r.debug_set_wait(0, False)
+    for a, b in zip(want, r.forward(params, cams)[:3]):
+        assert torch.equal(a, b)
