@@ -507,6 +507,7 @@ struct BwdSmem {
     // {u, v, qa, qb}, {qc, sigma, z, record}, {r, g, b, culling threshold}
     float4 dense[2][kDense][3];
     uint2 own;                                 // see next_block
+    unsigned odd;                // lanes with an upstream gradient that is not finite
     unsigned long long stat[2];                // contributor counts, composited (8x4 block, entry) pairs
 };
 
@@ -535,6 +536,8 @@ __device__ __forceinline__ void row_moments(const float4& a, const float4& b, fl
 }
 
 // Adds the group's n entries (dense records D) to the records' gradients.
+// Zero weights are left out of the sums where some pixel's upstream gradient is
+// not finite (S.odd).
 template <bool DEPTH>
 __device__ __forceinline__ void reduce_group(const BwdSmem& S, const float4 (*D)[3], int n, int lane, float cx, float cy,
                                              double* __restrict__ grad_rec, int64_t cap)
@@ -558,6 +561,19 @@ __device__ __forceinline__ void reduce_group(const BwdSmem& S, const float4 (*D)
             s1 = fmaf(w4[j], d.y, s1);
             s2 = fmaf(w4[j], d.z, s2);
             if constexpr (DEPTH) sd = fmaf(w4[j], d.w, sd);
+        }
+    }
+    if (S.odd != 0u) {
+        sd = s0 = s1 = s2 = 0.0f;
+#pragma unroll 1
+        for (int i = 0; i < 16; ++i) {
+            const float4 t = S.wg[e][(4 * q + (i >> 2)) ^ e], d = S.dcd[q][i];
+            const float w = (i & 2) ? ((i & 1) ? t.w : t.z) : ((i & 1) ? t.y : t.x);
+            if (w == 0.0f) continue;
+            s0 = fmaf(w, d.x, s0);
+            s1 = fmaf(w, d.y, s1);
+            s2 = fmaf(w, d.z, s2);
+            if constexpr (DEPTH) sd = fmaf(w, d.w, sd);
         }
     }
     const float4 q0 = D[e][0], q1 = D[e][1];
@@ -656,6 +672,14 @@ blend_bwd_kernel(const __grid_constant__ Table Tb, BlendBwdArgs a)
         }
         const int warp_last = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(lst[0], lst[1]));
         if (warp_last == 0) continue;
+        // A pixel whose upstream gradient is not finite spoils the gradients of
+        // the entries that it composites and no others of the block: such a
+        // block takes the exact path, which selects instead of multiplying by
+        // zero.
+        const unsigned odd = __ballot_sync(0xffffffffu, !(fabsf(X[0]) + fabsf(X[1]) <= 3.0e38f) ||
+                                                     !(fabsf(dc[0].x) + fabsf(dc[0].y) + fabsf(dc[0].z) + fabsf(dc[0].w) <= 3.0e38f) ||
+                                                     !(fabsf(dc[1].x) + fabsf(dc[1].y) + fabsf(dc[1].z) + fabsf(dc[1].w) <= 3.0e38f));
+        if (lane == 0) S.odd = odd;
         S.dcd[lane >> 3][2 * (lane & 7)] = dc[0];
         S.dcd[lane >> 3][2 * (lane & 7) + 1] = dc[1];
         {
@@ -711,7 +735,7 @@ blend_bwd_kernel(const __grid_constant__ Table Tb, BlendBwdArgs a)
                 d[1].w = __uint_as_float(kcur);
                 ind = !(d[2].w > -3.0e38f);
             }
-            indefinite = __any_sync(0xffffffffu, ind) || (left > 0 && indefinite);
+            indefinite = __any_sync(0xffffffffu, ind || (lane == 0 && S.odd != 0u)) || (left > 0 && indefinite);
 #pragma unroll
             for (int p = 0; p < 2; ++p)
                 if (lst[p] > 0 && (lst[p] - 1) / kChunk == c) start[p] = staged + __popc(m >> ((lst[p] - 1) & 31) >> 1);
@@ -782,7 +806,7 @@ blend_bwd_kernel(const __grid_constant__ Table Tb, BlendBwdArgs a)
                         const float ga = iom * fmaf(T[p], t.cdot[p], -X[p]);
                         T[p] = T[p] * iom;
                         w[p] = al * T[p];
-                        gP[p] = ga * alg;
+                        gP[p] = EXACT.value && alg == 0.0f ? 0.0f : ga * alg;
                         X[p] = fmaf(w[p], t.cdot[p], X[p]);
                     }
                     const int at = (16 * e + ((lane >> 1) ^ e)) * 2;
