@@ -935,9 +935,13 @@ gsr_status gsr_forward(gsr_ctx* ctx, const gsr_gaussians* g, const gsr_view* vie
     s->flags = ctx->cfg.flags;
     s->filled = false;
     s->have_grads = false;
-    // a recycled state's earlier work comes first
+    // a recycled state's earlier work comes first (a capture cannot wait for an
+    // event from outside it: the host waits)
     if (s->grown && s->pending) {
-        const cudaError_t e = cudaStreamWaitEvent(cs, s->done, 0);
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        cudaError_t e = cudaStreamIsCapturing(cs, &cap);
+        if (e == cudaSuccess)
+            e = cap == cudaStreamCaptureStatusNone ? cudaStreamWaitEvent(cs, s->done, 0) : cudaEventSynchronize(s->done);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "recycled state");
         s->pending = false;
     }
