@@ -569,13 +569,17 @@ static float choose_prefix(const unsigned long long* H, const unsigned long long
 
 // Lists by tile rows: the runs of the records' tiles are sorted by tile row and
 // expanded into the lists, instead of expanding and sorting the instances.  It
-// takes the batches of 65536 records and more (fewer are bound by launches, of
-// which it has four more: 10 us of a 240 us step on 10k records) whose views are
-// at most kRowListMaxTiles tiles wide; and not the allocation-free forward.
-constexpr int64_t kRowListMinRecords = 65536;
+// takes the batches of 65536 records and 4096 tiles and more whose views are at
+// most kRowListMaxTiles tiles wide; and not the allocation-free forward.  Fewer
+// records are bound by launches (four more here: 10 us of a 240 us step on 10k
+// records).  Fewer tiles have few instances, and few tile rows that hold all the
+// runs: emission, sort and ranges together, sorted instances against rows, took
+// 0.125 / 0.136 ms at 960 tiles (100k records), 0.185 / 0.238 at 2000 (18 small
+// views), 0.165 / 0.151 at 4600 (210k records).
+constexpr int64_t kRowListMinRecords = 65536, kRowListMinTiles = 4096;
 static bool use_row_lists(const Table& T)
 {
-    return T.n_records >= kRowListMinRecords && row_list_stride(T) <= kRowListMaxTiles;
+    return T.n_records >= kRowListMinRecords && T.n_tiles >= kRowListMinTiles && row_list_stride(T) <= kRowListMaxTiles;
 }
 
 // Its scratch in gsr_ctx::row_work; returns the bytes.

@@ -594,8 +594,13 @@ row_plan_kernel(RowListArgs a)
         __syncthreads();
         const uint32_t first = carry + s_warp[wid] + incl - c;
         if (r < a.n_trows) a.chunk_first[r] = first;
-        for (uint32_t i = 0; i < c; ++i)
-            if (first + i < (uint32_t)a.chunk_cap) a.chunk_row[first + i] = (uint32_t)r;
+        // a tile row's chunks are written by the whole warp (few rows can have
+        // thousands)
+        for (int j = 0; j < 32; ++j) {
+            const uint32_t cj = __shfl_sync(0xffffffffu, c, j), fj = __shfl_sync(0xffffffffu, first, j);
+            for (uint32_t i = lane; i < cj; i += 32)
+                if (fj + i < (uint32_t)a.chunk_cap) a.chunk_row[fj + i] = (uint32_t)(r0 + (tid & ~31) + j);
+        }
         carry += s_total;
         __syncthreads();
     }
@@ -692,48 +697,69 @@ row_count_kernel(const __grid_constant__ Table Tb, RowListArgs a)
     }
 }
 
-constexpr int kScanThreads = 256;
-__global__ void __launch_bounds__(kScanThreads)
+// One block per tile row, 32 columns at a time, a column per lane; each warp
+// sums a segment of the row's chunks, and writes its offsets once the earlier
+// warps' sums are known.  (One thread per column down all the chunks: a small
+// image's few tile rows have a thousand chunks each, a chain of 70 us.)
+constexpr int kScanWarps = 16;
+__global__ void __launch_bounds__(32 * kScanWarps)
 row_scan_kernel(const __grid_constant__ Table Tb, RowListArgs a)
 {
     if (earlier_wait_timed_out(a.status)) return;
     __shared__ ViewTiles s_vt;
-    __shared__ unsigned long long s_warp[kDupThreads / 32];
-    load_view_tiles(Tb, s_vt, kScanThreads);
-    static_assert(kScanThreads == kDupThreads, "block_excl_scan64");
+    __shared__ uint32_t s_sum[kScanWarps][32];
+    load_view_tiles(Tb, s_vt, 32 * kScanWarps);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t nc = *a.n_chunks;
     const int ch = row_chunk((int64_t)*a.n_rows);
     for (int64_t r = blockIdx.x; r < a.n_trows; r += gridDim.x) {
         const TileRow tr = tile_row(s_vt, Tb, (uint32_t)r);
         const uint2 g = a.row_range[r];
-        const uint32_t n = nc ? (g.y - g.x + (uint32_t)ch - 1u) / (uint32_t)ch : 0u;
+        const uint32_t n = nc && g.y > g.x ? (g.y - g.x + (uint32_t)ch - 1u) / (uint32_t)ch : 0u;
+        const uint32_t seg = (n + kScanWarps - 1) / kScanWarps;
+        const uint32_t i0 = min((uint32_t)w * seg, n), i1 = min(i0 + seg, n);
         uint32_t* base = a.chunk_count + (size_t)a.chunk_first[r] * a.stride;
-        unsigned long long carry = 0;
-        for (int x0 = 0; x0 < tr.tx; x0 += kScanThreads) {
-            const int x = x0 + (int)threadIdx.x;
-            uint32_t run = 0;
-            if (x < tr.tx) {
-                uint32_t* p = base + x;
-                uint32_t i = 0;
-                for (; i + 8 <= n; i += 8) {   // eight loads in flight
+        uint32_t carry = 0;
+        for (int x0 = 0; x0 < tr.tx; x0 += 32) {
+            const int x = x0 + lane;
+            const bool in = x < tr.tx;
+            uint32_t* p = base + x;
+            uint32_t sum = 0;
+            if (in) {
+#pragma unroll 8
+                for (uint32_t i = i0; i < i1; ++i) sum += p[(size_t)i * a.stride];
+            }
+            s_sum[w][lane] = sum;
+            __syncthreads();
+            uint32_t run = 0, total = 0;
+#pragma unroll
+            for (int j = 0; j < kScanWarps; ++j) {
+                const uint32_t v = s_sum[j][lane];
+                if (j < w) run += v;
+                total += v;
+            }
+            if (in) {
+                uint32_t i = i0;
+                for (; i + 8 <= i1; i += 8) {   // eight loads in flight
                     uint32_t v[8];
 #pragma unroll
                     for (int u = 0; u < 8; ++u) v[u] = p[(size_t)(i + u) * a.stride];
 #pragma unroll
                     for (int u = 0; u < 8; ++u) { p[(size_t)(i + u) * a.stride] = run; run += v[u]; }
                 }
-                for (; i < n; ++i) { const uint32_t v = p[(size_t)i * a.stride]; p[(size_t)i * a.stride] = run; run += v; }
+                for (; i < i1; ++i) { const uint32_t v = p[(size_t)i * a.stride]; p[(size_t)i * a.stride] = run; run += v; }
             }
-            unsigned long long total;
-            const unsigned long long ex = block_excl_scan64(run, s_warp, &total);
-            if (x < tr.tx) {
-                const uint32_t first = (uint32_t)(carry + ex);
-                a.tile_first[tr.first_tile + x] = make_uint2(first, run);
+            uint32_t incl = total;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
             }
-            carry += total;
-            __syncthreads();
+            if (w == 0 && in) a.tile_first[tr.first_tile + x] = make_uint2(carry + incl - total, total);
+            carry += __shfl_sync(0xffffffffu, incl, 31);
+            __syncthreads();   // the sums are rewritten by the next columns
         }
-        if (threadIdx.x == 0) a.row_first[r] = (uint32_t)carry;   // row_offsets turns the totals into offsets
+        if (threadIdx.x == 0) a.row_first[r] = carry;   // row_offsets turns the totals into offsets
     }
 }
 
@@ -925,7 +951,7 @@ void launch_row_lists(const Table& T, const RowListArgs& a, int num_sms, cudaStr
     GSR_COUNT_LAUNCH();
     row_count_kernel<<<blocks, 32 * kRowWarps, smem, s>>>(T, a);
     GSR_COUNT_LAUNCH();
-    row_scan_kernel<<<(unsigned)std::min<int64_t>(a.n_trows, (int64_t)num_sms * 8), kScanThreads, 0, s>>>(T, a);
+    row_scan_kernel<<<(unsigned)std::min<int64_t>(a.n_trows, (int64_t)num_sms * 4), 32 * kScanWarps, 0, s>>>(T, a);
     GSR_COUNT_LAUNCH();
     row_offsets_kernel<<<1, 1024, 0, s>>>(a);
     GSR_COUNT_LAUNCH();

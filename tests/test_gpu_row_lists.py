@@ -1,4 +1,4 @@
-"""Tile lists made by tile rows (batches of 65536 records and more): the lists
+"""Tile lists made by tile rows (batches of 65536 records and 4096 tiles and more): the lists
 of small and large records over ragged views and every tile shape against the
 oracle, images equal to those of the same views in smaller batches (lists by
 sorted instances), two rounds equal to one, and growth from tiny buffers."""
@@ -24,7 +24,9 @@ N = 24_000
 def _scene(tile, log_scale=(-6.0, -2.0)):
     views = [scenes.pinhole(203, 77, f=150.0),
              scenes.pinhole(64, 130, f=90.0, viewmat=scenes.look_from([0.2, 0.0, -0.3], yaw_deg=9.0)),
-             scenes.pinhole(1, 1, f=2.0), scenes.pinhole(33, 17, f=40.0, viewmat=scenes.look_from([0.0, 0.1, 0.0], roll_deg=30.0))]
+             scenes.pinhole(1, 1, f=2.0), scenes.pinhole(33, 17, f=40.0, viewmat=scenes.look_from([0.0, 0.1, 0.0], roll_deg=30.0)),
+             # more than 4096 tiles, empty: it looks away
+             scenes.pinhole(1040, 1040, f=500.0, viewmat=scenes.look_from([0.0, 0.0, 0.0], yaw_deg=180.0))]
     return scenes.random_scene(11, N, views, 0, log_scale_range=log_scale, tile=tile)
 
 
