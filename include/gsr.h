@@ -101,14 +101,16 @@ typedef struct gsr_saved gsr_saved;
 
 typedef struct {
     int tile_w, tile_h;   /* screen tile: 16x16, 32x8 or 8x32                 */
-    int blend_batch;      /* 128, 256 or 512; kept for existing callers: the
-                             blends stage 32 list entries per warp whatever
-                             the value                                        */
+    int blend_batch;      /* Gaussians staged in shared memory per batch by
+                             the backward blend when blend_batch_bwd is 0:
+                             128, 256 or 512 (the forward stages 32 per warp) */
     int sh_degree;        /* 0 .. 3                                           */
     float near_plane;     /* records with camera z <= near are culled (0.2)   */
     float bg[3];          /* background colour                                */
     uint32_t flags;       /* GSR_FLAG_*                                       */
-    int blend_batch_bwd;  /* 0, 128 (default), 256 or 512; as blend_batch     */
+    int blend_batch_bwd;  /* Gaussians staged per batch by the backward blend:
+                             0 (the forward's blend_batch), 128 (default),
+                             256 or 512                                       */
     float list_prefix;    /* how the forward builds the tile lists:
                              >= 1 (default): one round, every tile's full
                              list;
@@ -421,10 +423,11 @@ GSR_API gsr_status gsr_l1_loss_grad(const float* rgb, const float* target, int64
                             float* loss_out, void* stream);
 
 /* Autotuner: time forward+backward for every tile shape in
- * {16x16, 32x8, 8x32} on this batch (with the given upstream gradient), keep
- * the fastest in the context's configuration and return it in *best (may be
- * NULL).  Results are cached per batch signature (view sizes, subset sizes,
- * SH degree). */
+ * {16x16, 32x8, 8x32} x blend batch in {128, 256, 512} on this batch (with
+ * the given upstream gradient), then the backward's own batch
+ * (blend_batch_bwd) for the fastest, keep the fastest in the context's
+ * configuration and return it in *best (may be NULL).  Results are cached
+ * per batch signature (view sizes, subset sizes, SH degree). */
 GSR_API gsr_status gsr_tune(gsr_ctx* ctx, const gsr_gaussians* g, const gsr_view* views, int n_views,
                     const gsr_outputs* out, gsr_saved* saved, const float* dl_drgb,
                     const gsr_grads* grads, gsr_config* best, void* stream);
@@ -465,8 +468,8 @@ GSR_API gsr_status gsr_debug_record_grads(gsr_saved* saved, float* grec, void* s
 
 /* Device-wait limit and a test-only fault of the look-back (failure
  * detection, tested without a GPU fault).  Every device-side wait of the
- * context's later calls (the radix sort's mbarrier waits on bulk copies,
- * decoupled look-back spins) gives up after wait_ns nanoseconds (0 = the default, 2 s), sets the
+ * context's later calls (mbarrier waits on bulk copies, decoupled look-back
+ * spins) gives up after wait_ns nanoseconds (0 = the default, 2 s), sets the
  * timeout bit of the call's status word and lets its kernel finish; every
  * kernel after it in the call then skips its work, and the call (or
  * gsr_check) returns GSR_ERR_TIMEOUT.  flags: 0, or GSR_DEBUG_WITHHOLD_PREFIX:

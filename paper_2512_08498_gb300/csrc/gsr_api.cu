@@ -1026,17 +1026,12 @@ gsr_status gsr_check(gsr_ctx* ctx, gsr_saved* s, void* stream)
 }  // extern "C"
 
 namespace gsr {
-// The record gradients of the visible records (16-byte words; see GradRec).
-__global__ void zero_grad_rec_kernel(double* base, const unsigned long long* n_dev, int64_t cap)
+__global__ void zero_grad_rec_kernel(float4* g, const unsigned long long* n_dev, int64_t cap)
 {
     const unsigned long long nv = *n_dev;
-    const int64_t n = (int64_t)(nv < (unsigned long long)cap ? nv : (unsigned long long)cap);
-    float4* g = reinterpret_cast<float4*>(base);
-    float4* h = reinterpret_cast<float4*>(base + 8 * cap);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < 4 * n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t n = 3 * (int64_t)(nv < (unsigned long long)cap ? nv : (unsigned long long)cap);
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         g[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (i < n) h[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
 }
 }  // namespace gsr
 
@@ -1065,7 +1060,7 @@ gsr_status gsr_backward(gsr_ctx* ctx, const gsr_gaussians* g, const gsr_view* vi
         }
         return e;
     };
-    cudaError_t e = ensure(ctx->grad_rec, (size_t)s->rec_cap * kGradBytes);
+    cudaError_t e = ensure(ctx->grad_rec, (size_t)s->rec_cap * kGradFloats * 4);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "alloc record gradients");
     if ((e = ensure(ctx->bwd_queue, (size_t)s->rec_cap * 4)) != cudaSuccess)
         return cuda_fail(ctx, e, "alloc extended-precision queue");
@@ -1108,7 +1103,7 @@ gsr_status gsr_backward(gsr_ctx* ctx, const gsr_gaussians* g, const gsr_view* vi
     cudaMemsetAsync(counters + kCntWarpBwd, 0, 8, cs);
     cudaMemsetAsync(ctrl + kCtrlGradRows, 0, 8, cs);
     GSR_COUNT_LAUNCH();
-    zero_grad_rec_kernel<<<(unsigned)std::max(1, ctx->num_sms * 8), 256, 0, cs>>>(ctx->grad_rec.as<double>(),
+    zero_grad_rec_kernel<<<(unsigned)std::max(1, ctx->num_sms * 8), 256, 0, cs>>>(ctx->grad_rec.as<float4>(),
                                                                                   counters + kCntVisible, s->rec_cap);
 
     BlendBwdArgs bb;
@@ -1122,13 +1117,14 @@ gsr_status gsr_backward(gsr_ctx* ctx, const gsr_gaussians* g, const gsr_view* vi
     bb.dl_rgb = dl_drgb;
     bb.dl_depth = dl_ddepth;
     bb.dl_alpha = dl_dalpha;
-    bb.grad_rec = ctx->grad_rec.as<double>();
-    bb.rec_cap = s->rec_cap;
+    bb.grad_rec = ctx->grad_rec.as<float4>();
     bb.work = reinterpret_cast<unsigned int*>(ctrl + kCtrlWorkBwd);
     bb.status = status;
     bb.counters = counters;
+    bb.wait_ns = ctx->wait_ns;
     prof_mark(pr, 1, cs);
-    launch_blend_bwd(T, bb, ctx->num_sms, cs);
+    // the backward's staging batch is free (it reads wmask by list position)
+    launch_blend_bwd(T, ctx->cfg.blend_batch_bwd ? ctx->cfg.blend_batch_bwd : s->batch, bb, ctx->num_sms, cs);
     prof_mark(pr, 2, cs);
 
     PreprocessBwdArgs pb;
@@ -1136,8 +1132,7 @@ gsr_status gsr_backward(gsr_ctx* ctx, const gsr_gaussians* g, const gsr_view* vi
     pb.opacity = g->opacity_logits; pb.sh = g->sh;
     pb.vis_aux = s->vis_aux.as<uint4>();
     pb.kstart = s->kstart.as<uint32_t>();
-    pb.grad_rec = ctx->grad_rec.as<double>();
-    pb.rec_cap = s->rec_cap;
+    pb.grad_rec = ctx->grad_rec.as<float4>();
     pb.grad_means = grads->means; pb.grad_log_scales = grads->log_scales; pb.grad_quats = grads->quats;
     pb.grad_opacity = grads->opacity_logits; pb.grad_sh = grads->sh; pb.grad_pose = grads->pose;
     pb.grad_focal = grads->focal;
@@ -1595,7 +1590,7 @@ gsr_status gsr_debug_record_grads(gsr_saved* s, float* grec, void* stream)
     DebugArgs a{};
     a.rec = s->rec.as<float4>();
     a.vis_aux = s->vis_aux.as<uint4>();
-    a.grad_rec = s->ctx->grad_rec.as<double>();
+    a.grad_rec = s->ctx->grad_rec.as<float4>();
     a.counters = reinterpret_cast<const unsigned long long*>(s->ctrl.as<unsigned char>() + kCtrlCounters);
     a.rec_cap = s->rec_cap;
     a.inst_cap = s->inst_cap;
@@ -1631,37 +1626,51 @@ gsr_status gsr_tune(gsr_ctx* ctx, const gsr_gaussians* g, const gsr_view* views,
     }
     const gsr_config base = ctx->cfg;
     const int shapes[3][2] = {{16, 16}, {32, 8}, {8, 32}};
+    const int batches[3] = {128, 256, 512};
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
         return fail(ctx, GSR_ERR_CUDA, "event create");
     float best_ms = 1e30f;
     gsr_config best_cfg = base;
     gsr_status result = GSR_OK;
-    for (const auto& shape : shapes) {
-        gsr_config c = base;
-        c.tile_w = shape[0];
-        c.tile_h = shape[1];
-        c.flags &= ~GSR_FLAG_NO_SYNC;
-        ctx->cfg = c;
-        // warm-up (also sizes buffers for this shape)
-        gsr_status r = gsr_forward(ctx, g, views, n_views, out, s, stream);
-        if (r == GSR_OK) r = gsr_backward(ctx, g, views, n_views, s, dl_drgb, nullptr, nullptr, grads, stream);
-        if (r != GSR_OK) { result = r; continue; }
-        ctx->cfg.flags |= GSR_FLAG_NO_SYNC;
-        const int reps = 3;
-        cudaEventRecord(e0, cs);
-        for (int i = 0; i < reps; ++i) {
-            gsr_forward(ctx, g, views, n_views, out, s, stream);
-            gsr_backward(ctx, g, views, n_views, s, dl_drgb, nullptr, nullptr, grads, stream);
+    // every shape x batch (both passes on one batch), then the backward's batch
+    // for the winner (it stages records independently of the forward)
+    for (int k = 0; k < 9 + 3; ++k) {
+        {
+            gsr_config c = base;
+            if (k < 9) {
+                c.tile_w = shapes[k / 3][0];
+                c.tile_h = shapes[k / 3][1];
+                c.blend_batch = batches[k % 3];
+                c.blend_batch_bwd = 0;
+            } else {
+                if (best_ms >= 1e29f) break;
+                c = best_cfg;
+                c.blend_batch_bwd = batches[k - 9];
+                if (c.blend_batch_bwd == c.blend_batch) continue;   // timed already
+            }
+            c.flags &= ~GSR_FLAG_NO_SYNC;
+            ctx->cfg = c;
+            // warm-up (also sizes buffers for this shape)
+            gsr_status r = gsr_forward(ctx, g, views, n_views, out, s, stream);
+            if (r == GSR_OK) r = gsr_backward(ctx, g, views, n_views, s, dl_drgb, nullptr, nullptr, grads, stream);
+            if (r != GSR_OK) { result = r; continue; }
+            ctx->cfg.flags |= GSR_FLAG_NO_SYNC;
+            const int reps = 3;
+            cudaEventRecord(e0, cs);
+            for (int i = 0; i < reps; ++i) {
+                gsr_forward(ctx, g, views, n_views, out, s, stream);
+                gsr_backward(ctx, g, views, n_views, s, dl_drgb, nullptr, nullptr, grads, stream);
+            }
+            cudaEventRecord(e1, cs);
+            cudaEventSynchronize(e1);
+            float ms = 0.0f;
+            cudaEventElapsedTime(&ms, e0, e1);
+            uint32_t status = 0;
+            read_status(ctx, s, cs, &status);
+            if (status) continue;
+            if (ms < best_ms) { best_ms = ms; best_cfg = c; best_cfg.flags = base.flags; }
         }
-        cudaEventRecord(e1, cs);
-        cudaEventSynchronize(e1);
-        float ms = 0.0f;
-        cudaEventElapsedTime(&ms, e0, e1);
-        uint32_t status = 0;
-        read_status(ctx, s, cs, &status);
-        if (status) continue;
-        if (ms < best_ms) { best_ms = ms; best_cfg = c; best_cfg.flags = base.flags; }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);

@@ -3,8 +3,12 @@
 // One persistent launch per direction covers every (view, tile) of the batch:
 // work comes from an atomic tile counter, so views of uneven size and tiles of
 // uneven list length share one grid of (SMs x resident blocks).  A tile has
-// 256 pixels; a warp takes one of its 8x8 pixel blocks and waits for no other
-// warp.
+// 256 pixels.  The forward gives an 8x8 pixel block to a warp that waits for
+// no other (see below); the backward gives the tile to a block of eight warps
+// over 8x4 pixels each and walks the list in batches of BATCH records, each
+// gathered into shared memory with one bulk async copy (cp.async.bulk, the TMA
+// engine) per record (the 48 bytes it reads), completing on an mbarrier,
+// double-buffered so the gather of batch b+1 overlaps the arithmetic of batch b.
 //
 // Culling: every record carries a conservative box outside which its
 // binary32 alpha is certainly below 1/255 (see alpha_box in
@@ -26,8 +30,9 @@
 //   evaluated as T_k (dC . c + dD z) - X / (1 - alpha_k) with the single
 //   running scalar X = dC . S_C + dD S_D - dA T_final;
 //   then the chain to (u, v, qa, qb, qc, sigma, colour, z), reduced over the
-//   block's pixels through per-warp slot buffers and added to the per-record
-//   gradient.
+//   warp through per-warp slot buffers (one entry per lane pair, see
+//   slots_reduce), over the CTA in shared memory, and added to the
+//   per-record gradient with one vector atomic per 16 bytes.
 #include <type_traits>
 
 #include "gsr_common.cuh"
@@ -35,7 +40,31 @@
 
 namespace gsr {
 
-constexpr int kTilePixels = 256;
+constexpr int kBlendThreads = 256;
+constexpr int kWarps = kBlendThreads / 32;
+
+template <int BX, int BY>
+struct TileShape {
+    static_assert(BX * BY == kBlendThreads, "tile must hold 256 pixels");
+    static constexpr int WX = 8, WY = 4;          // warp footprint
+    static constexpr int WPR = BX / WX;           // warps per tile row
+    __device__ static int lx(int tid) { return ((tid >> 5) % WPR) * WX + (tid & 7); }
+    __device__ static int ly(int tid) { return ((tid >> 5) / WPR) * WY + ((tid & 31) >> 3); }
+};
+
+// Gather `cnt` records (list positions [first, first + cnt)) into dst.
+template <int NQ>
+__device__ __forceinline__ void issue_batch(const uint32_t* vals, const float4* rec, uint32_t first, int cnt,
+                                            float4* dst, uint64_t* bar, uint32_t* idx_out)
+{
+    const int tid = threadIdx.x;
+    if (tid == 0) mbar_arrive_expect_tx(bar, (uint32_t)cnt * NQ * 16u);
+    for (int t = tid; t < cnt; t += kBlendThreads) {
+        const uint32_t k = vals[first + t];
+        if (idx_out) idx_out[t] = k;
+        bulk_g2s(dst + NQ * t, rec + 4 * (size_t)k, NQ * 16, bar);
+    }
+}
 
 // Largest value of the quadratic form P(x, y) = x (qa x + qb y) + qc y^2
 // (negative definite) over the rectangle [x0, x1] x [y0, y1] of pixel
@@ -81,7 +110,7 @@ constexpr int kFwdWarps = 4;            // warps per block (they share nothing)
 constexpr int kFwdThreads = 32 * kFwdWarps;
 constexpr int kChunk = 32;              // list entries per step: one per lane
 constexpr int kBlk = 8;                 // the pixel block's side
-constexpr int kBlocksPerTile = kTilePixels / (kBlk * kBlk);
+constexpr int kBlocksPerTile = kBlendThreads / (kBlk * kBlk);
 
 // A surviving record as the walk reads it.
 struct DenseRec {
@@ -211,7 +240,7 @@ __global__ void __launch_bounds__(kFwdThreads, 6)
 blend_fwd_kernel(const __grid_constant__ Table Tb, BlendFwdArgs a)
 {
     if (earlier_wait_timed_out(a.status)) return;
-    constexpr int BY = kTilePixels / BX, BPR = BX / kBlk;   // blocks per tile row
+    constexpr int BY = kBlendThreads / BX, BPR = BX / kBlk;   // blocks per tile row
     __shared__ __align__(128) FwdSmem s_warp[kFwdWarps];
     __shared__ unsigned long long s_queue;
     if (threadIdx.x == 0) s_queue = (unsigned long long)atomicAdd(a.work, 1u) << 32;   // the first tile
@@ -455,398 +484,389 @@ blend_fwd_kernel(const __grid_constant__ Table Tb, BlendFwdArgs a)
     }
 }
 
-// ---------------------------------------------------------------------------
-// backward
-// ---------------------------------------------------------------------------
-// One warp takes one 8x8 pixel block, two horizontally adjacent pixels per
-// lane as in the forward, and nothing in it waits for another warp.  The
-// block's composited entries come from the forward's mask words, 32 list
-// positions at a time from the back; their records (48 bytes) are staged
-// densely, last entry first, by asynchronous copies issued one chunk ahead, and
-// walked in groups of kSlots.
-//
-// Reduction over the block's 64 pixels, transposed.  For each walked entry
-// every lane stores, for its two pixels, gP = dL/dP2 and w = alpha T (both zero
-// where the pixel does not composite the entry), and per group four lanes sum
-// one entry over two pixel rows each.  The record gradient needs
+// Backward reduction over a warp's 32 pixels, transposed.  For each walked
+// entry every lane stores two scalars in its warp's slot buffer -- gP =
+// dL/dP2 and w = alpha T (both zero where the pixel does not composite the
+// entry) -- and every kSlots entries the warp reduces the buffer with one
+// entry per lane pair, so a lane sums over pixels serially instead of the
+// warp summing ten values per entry with shuffles.  The record gradient needs
 //   sum gP dx, sum gP dy, sum gP dx^2, sum gP dx dy, sum gP dy^2,
 //   sum gP / sigma (= sum dL/dalpha G where alpha is not clamped),
 //   sum w dD, sum w dC (three channels),
 // with dx = px - u the same for every pixel up to the pixel's offset inside
-// the block: dx = xo - ux, xo = x - 3.5, ux = u minus the block centre (same
-// for y).  So a lane keeps the six moments M = sum gP {1, xo, yo, xo^2, xo yo,
-// yo^2} (constant weights) and shifts them once per entry:
+// the 8x4 block: dx = xo - ux, xo = x - 3.5 (x = lane & 7), ux = u minus the
+// block centre (same for y with yo = (lane >> 3) - 1.5).  So the warp keeps
+// the six moments M = sum gP {1, xo, yo, xo^2, xo yo, yo^2} (constant
+// weights) and shifts them once per entry:
 //   sum gP dx = Mx - ux M0, sum gP dx^2 = Mxx - 2 ux Mx + ux^2 M0,
 //   sum gP dx dy = Mxy - ux My - uy Mx + ux uy M0 (and y alike).
 // The shifted form has the rounding error of the direct sums (bounded by
-// the sums of |gP| dx^2 both ways).  Two shuffle steps add the four lanes, and
-// they add the record's ten sums to memory in binary64: a record's blocks
-// each add once (the tile's eight warps used to be summed in shared memory
-// first), and in binary32 the longer chain of additions showed in the
-// gradients of Gaussians that cover many tiles (1.6 times the error).
-//
-// Bound by instruction issue (81 % of the slots) with the shared-memory pipe close
-// behind (71 %: slot stores and the reduction's reads).  Against the tile's eight
-// 8x4 warps in step (batches of 128 records with two barriers each, sums of a
-// record over the warps in shared memory): a record's loads and row products serve
-// two pixels, one test covers the alpha thresholds and the clamp, and the record
-// sums, their flush and the barriers are gone.  1M-Gaussian six-camera rig 2.62 ->
-// 2.09 ms, 30-view window 11.5 -> 8.7, 60-view road 36.8 -> 28.1.  Summing w dC over
-// a lane's pixels in the walk instead of storing w (no reads of dC in the
-// reduction): 2.13 ms on the rig; binary32 additions to memory: 2.02 ms.
-// Keeping a non-finite upstream gradient to its pixel (S.odd) costs 0.04 ms there.
-// Where a batch's blocks do not fill the chip or a few lists are very long, the
-// walk of twice the pixels per warp is the longer chain: 0.066 -> 0.105 ms on 20k
-// Gaussians at 640 x 384 (the forward 0.061 -> 0.087).
-constexpr int kSlots = 8;
-constexpr int kLeft = kSlots;                  // dense positions kept for the entries left over from a chunk
-constexpr int kDense = kLeft + kChunk;
+// the sums of |gP| dx^2 both ways).  Per-pixel dC, dD come from s_dcd.
+constexpr int kSlots = 16;
+// Shared record sums: 10 floats per record at an odd stride, so lanes
+// adding to (or flushing) different records hit different banks.
+constexpr int kSumStride = 11;
+constexpr int kSlotStride = 32;   // floats per slot row: 32 pixels
+// 16-byte chunk c of slot row r is stored at chunk c ^ (r & 7): a row's
+// stores stay a permutation of its 32 banks, and the 16-byte reads of the
+// same chunk from eight different rows land in eight different bank groups.
+__device__ __forceinline__ int slot_chunk(int c, int r) { return c ^ (r & 7); }
+// The float of slot row r that holds pixel (lane) l: chunk l / 4, element l % 4.
+__device__ __forceinline__ int slot_col(int l, int r) { return l ^ ((r & 7) << 2); }
 
-struct BwdSmem {
-    // row e: the group's entry e; 16-byte piece c of a row (pixels 4c .. 4c + 3
-    // in row-major order) is stored at piece c ^ e, so that the reads of the same
-    // piece of eight rows land in eight different bank groups
-    float4 gp[kSlots][16], wg[kSlots][16];
-    float4 dcd[4][17];                         // (dC, dD) of the pixels, 16 per quarter and one of padding
-    // {u, v, qa, qb}, {qc, sigma, z, record}, {r, g, b, culling threshold}
-    float4 dense[2][kDense][3];
-    uint2 own;                                 // see next_block
-    unsigned odd;                              // lanes with an upstream gradient that is not finite
-    unsigned long long stat[2];                // contributor counts, composited (8x4 block, entry) pairs
-};
-
-__device__ __forceinline__ float rcp_approx(float x)
+// Slot j holds the entry at position i0 - j of the warp's walk list L.
+template <typename LT>
+__device__ __forceinline__ void slots_reduce(const float* __restrict__ sgp, const float* __restrict__ swg,
+                                             const float4* __restrict__ sdcd, int n, int lane, const LT* L,
+                                             int i0, const float4* B, float cxw, float cyw, float* s_grad)
 {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
-__device__ __forceinline__ float ex2_approx(float x)
-{
-    float r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
-// Sums over the row of eight pixels g: {1, xo, xo^2}, by the symmetry of xo.
-__device__ __forceinline__ void row_moments(const float4& a, const float4& b, float& r, float& x1, float& x2)
-{
-    const float s0 = a.w + b.x, s1 = a.z + b.y, s2 = a.y + b.z, s3 = a.x + b.w;
-    const float d0 = b.x - a.w, d1 = b.y - a.z, d2 = b.z - a.y, d3 = b.w - a.x;
-    r = (s0 + s1) + (s2 + s3);
-    x1 = fmaf(3.5f, d3, fmaf(2.5f, d2, fmaf(1.5f, d1, 0.5f * d0)));
-    x2 = fmaf(12.25f, s3, fmaf(6.25f, s2, fmaf(2.25f, s1, 0.25f * s0)));
-}
-
-// Adds the group's n entries (dense records D) to the records' gradients.
-// Zero weights are left out of the sums where some pixel's upstream gradient is
-// not finite (S.odd).
-template <bool DEPTH>
-__device__ __forceinline__ void reduce_group(const BwdSmem& S, const float4 (*D)[3], int n, int lane, float cx, float cy,
-                                             double* __restrict__ grad_rec, int64_t cap)
-{
-    const int e = lane & (kSlots - 1), q = lane >> 3;     // entry, pixel rows 2q and 2q + 1
-    float ra, xa, xxa, rb, xb, xxb;
-    row_moments(S.gp[e][(4 * q) ^ e], S.gp[e][(4 * q + 1) ^ e], ra, xa, xxa);
-    row_moments(S.gp[e][(4 * q + 2) ^ e], S.gp[e][(4 * q + 3) ^ e], rb, xb, xxb);
-    const float ya = 2.0f * (float)q - 3.5f, yb = ya + 1.0f;
-    const float m0 = ra + rb, mx = xa + xb, mxx = xxa + xxb;
-    const float my = fmaf(ya, ra, yb * rb), mxy = fmaf(ya, xa, yb * xb), myy = fmaf(ya * ya, ra, (yb * yb) * rb);
-    float sd = 0.0f, s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
+    const int e = lane & (kSlots - 1), h = lane >> 4;     // entry slot, pixel half (block rows 2h, 2h + 1)
+    const float* gp = sgp + e * kSlotStride;
+    const float* wg = swg + e * kSlotStride;
+    float g[16];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-        const float4 t = S.wg[e][(4 * q + c) ^ e];
+        const float4 t = *reinterpret_cast<const float4*>(gp + 4 * slot_chunk(4 * h + c, e));
+        g[4 * c] = t.x; g[4 * c + 1] = t.y; g[4 * c + 2] = t.z; g[4 * c + 3] = t.w;
+    }
+    float r0 = 0.0f, r1 = 0.0f, mxx = 0.0f, mx0 = 0.0f, mx1 = 0.0f;
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+        const float xo = (float)x - 3.5f;
+        r0 += g[x];
+        r1 += g[8 + x];
+        mxx = fmaf(xo * xo, g[x] + g[8 + x], mxx);
+        mx0 = fmaf(xo, g[x], mx0);
+        mx1 = fmaf(xo, g[8 + x], mx1);
+    }
+    const float y0 = 2.0f * (float)h - 1.5f, y1 = y0 + 1.0f;
+    float v[10];
+    v[0] = r0 + r1;
+    v[1] = mx0 + mx1;
+    v[2] = fmaf(y0, r0, y1 * r1);
+    v[3] = mxx;
+    v[4] = fmaf(y0, mx0, y1 * mx1);
+    v[5] = fmaf(y0 * y0, r0, (y1 * y1) * r1);
+    float sd = 0.0f, s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
+    const float4* dcd = sdcd + 16 * h;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const float4 t = *reinterpret_cast<const float4*>(wg + 4 * slot_chunk(4 * h + c, e));
         const float w4[4] = {t.x, t.y, t.z, t.w};
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const float4 d = S.dcd[q][4 * c + j];
+            const float4 d = dcd[4 * c + j];
             s0 = fmaf(w4[j], d.x, s0);
             s1 = fmaf(w4[j], d.y, s1);
             s2 = fmaf(w4[j], d.z, s2);
-            if constexpr (DEPTH) sd = fmaf(w4[j], d.w, sd);
+            sd = fmaf(w4[j], d.w, sd);
         }
     }
-    if (S.odd != 0u) {
-        sd = s0 = s1 = s2 = 0.0f;
-#pragma unroll 1
-        for (int i = 0; i < 16; ++i) {
-            const float4 t = S.wg[e][(4 * q + (i >> 2)) ^ e], d = S.dcd[q][i];
-            const float w = (i & 2) ? ((i & 1) ? t.w : t.z) : ((i & 1) ? t.y : t.x);
-            if (w == 0.0f) continue;
-            s0 = fmaf(w, d.x, s0);
-            s1 = fmaf(w, d.y, s1);
-            s2 = fmaf(w, d.z, s2);
-            if constexpr (DEPTH) sd = fmaf(w, d.w, sd);
-        }
-    }
-    const float4 q0 = D[e][0], q1 = D[e][1];
-    const float ux = q0.x - cx, uy = q0.y - cy;
-    const float sx = fmaf(-ux, m0, mx), sy = fmaf(-uy, m0, my);
-    const float sxx = fmaf(ux * ux, m0, fmaf(-2.0f * ux, mx, mxx));
-    const float sxy = fmaf(ux * uy, m0, fmaf(-ux, my, fmaf(-uy, mx, mxy)));
-    const float syy = fmaf(uy * uy, m0, fmaf(-2.0f * uy, my, myy));
-    // lanes with bit 3 clear end with {sx, sy, sxx, sxy}, the others with
-    // {syy, m0, sd, s0, s1, s2}
-    const bool hi = lane & 8;
-    const float a[4] = {sx, sy, sxx, sxy}, b[6] = {syy, m0, sd, s0, s1, s2};
-    float v[6];
+    v[6] = sd; v[7] = s0; v[8] = s1; v[9] = s2;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) v[i] = (hi ? b[i] : a[i]) + __shfl_xor_sync(0xffffffffu, hi ? a[i] : b[i], 8);
-#pragma unroll
-    for (int i = 4; i < 6; ++i) v[i] = b[i] + __shfl_xor_sync(0xffffffffu, b[i], 8);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], 16);
-    // the record's coefficients, ln2 and the sign of the mean gradient; the
-    // sum of dL/dalpha G over the pixels where alpha is not clamped = sum gP / sigma
-    const bool last = lane & 16;
-    float o0, o1, o2 = 0.0f;
-    if (!hi) {
-        o0 = last ? GSR_LN2 * v[2] : -GSR_LN2 * (2.0f * q0.z * v[0] + q0.w * v[1]);
-        o1 = last ? GSR_LN2 * v[3] : -GSR_LN2 * (q0.w * v[0] + 2.0f * q1.x * v[1]);
+    for (int j = 0; j < 10; ++j) v[j] += __shfl_xor_sync(0xffffffffu, v[j], 16);
+    if (e >= n) return;
+    const uint32_t k = L[i0 - e];
+    // layout of a record's sums: du dv dqa dqb dqc dsig dz dr dg db
+    float* sg = s_grad + k * kSumStride;
+    if (h == 0) {
+        const float4 r = B[3 * k];
+        const float ux = r.x - cxw, uy = r.y - cyw;
+        const float m0 = v[0];
+        atomicAdd(sg + 0, fmaf(-ux, m0, v[1]));
+        atomicAdd(sg + 1, fmaf(-uy, m0, v[2]));
+        atomicAdd(sg + 2, fmaf(ux * ux, m0, fmaf(-2.0f * ux, v[1], v[3])));
+        atomicAdd(sg + 3, fmaf(ux * uy, m0, fmaf(-ux, v[2], fmaf(-uy, v[1], v[4]))));
+        atomicAdd(sg + 4, fmaf(uy * uy, m0, fmaf(-2.0f * uy, v[2], v[5])));
     } else {
-        o0 = last ? v[3] : GSR_LN2 * v[0];
-        o1 = last ? v[4] : __fdividef(v[1], q1.y);
-        o2 = last ? v[5] : v[2];
-    }
-    if (e < n) {
-        const size_t k = __float_as_uint(q1.w);
-        double* p = grad_rec + 8 * k + (hi ? 2 : 0) + (last ? 1 : 0);
-        atomicAdd(p, (double)o0);
-        atomicAdd(p + 4, (double)o1);
-        if (hi && (DEPTH || last)) atomicAdd(grad_rec + 8 * (size_t)cap + 2 * k + (last ? 1 : 0), (double)o2);
+        atomicAdd(sg + 5, v[0]);
+        atomicAdd(sg + 6, v[6]);
+        atomicAdd(sg + 7, v[7]);
+        atomicAdd(sg + 8, v[8]);
+        atomicAdd(sg + 9, v[9]);
     }
 }
 
-// DEPTH: an upstream depth gradient is given (else its terms are zero).
-template <int BX, bool DEPTH>
-__global__ void __launch_bounds__(kFwdThreads, 6)
+// ---------------------------------------------------------------------------
+// backward
+// ---------------------------------------------------------------------------
+// The part of one (pixel, entry) pair of the backward that does not depend
+// on the running T and X: alpha, its decisions and the colour/depth dot.
+struct BwdPair {
+    int k;
+    bool front;    // P2 <= 0
+    bool near;     // alpha within 1e-6 relative of a threshold (see bwd_refine)
+    bool contrib;
+    float P2m, sa, al, iom, cdot;
+};
+
+__device__ __forceinline__ BwdPair bwd_pair(const float4* B, int k, float pxf, float pyf, float dC0, float dC1,
+                                            float dC2, float dD)
+{
+    BwdPair e;
+    e.k = k;
+    const float4 r0 = B[3 * k];
+    const float4 r1 = B[3 * k + 1];
+    const float4 r2 = B[3 * k + 2];
+    const float dx = __fsub_rn(pxf, r0.x), dy = __fsub_rn(pyf, r0.y);
+    const float P2 = __fmaf_rn(dx, __fmaf_rn(r0.z, dx, __fmul_rn(r0.w, dy)), __fmul_rn(__fmul_rn(r1.x, dy), dy));
+    // The value of 2^P2 here only feeds the adjoint, so the hardware
+    // approximation (ex2.approx, a few ulp from 2^x, as is the contract's
+    // polynomial) serves; the two decisions that must be the forward's --
+    // alpha >= 1/255 and the 0.99 clamp -- are re-taken with the contract's
+    // exponential whenever alpha lies near either threshold.  One test covers
+    // both: (sa - 1/255)(sa - 0.99) is within 1.1e-6 of zero for sa within
+    // about 1.1e-6 of either root (0.99 - 1/255 = 0.986), i.e. 1.1e-6 relative
+    // at 0.99 and 3e-4 relative at 1/255 -- several times what the two
+    // approximations can differ by (the rounding of the product is below
+    // 3e-8 there).
+    e.front = P2 <= 0.0f;
+    e.P2m = fminf(P2, 0.0f);
+    float G;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(G) : "f"(e.P2m));
+    e.sa = __fmul_rn(r1.y, G);
+    e.near = fabsf(__fmaf_rn(e.sa, __fsub_rn(e.sa, GSR_ALPHA_MIN + GSR_ALPHA_MAX), GSR_ALPHA_MIN * GSR_ALPHA_MAX)) <=
+             1.1e-6f;
+    e.cdot = dC0 * r2.x + dC1 * r2.y + dC2 * r2.z + dD * r1.z;
+    return e;
+}
+
+// The contract's exponential for the (rare) pairs near a threshold.  Taken
+// once per pair of entries on a warp vote, so the common case pays one vote
+// instead of a divergent branch per entry.
+__device__ __forceinline__ void bwd_refine(const float4* B, BwdPair& e1, BwdPair& e0)
+{
+    if (__any_sync(0xffffffffu, e1.near || e0.near)) {
+        if (e1.near) e1.sa = __fmul_rn(B[3 * e1.k + 1].y, exp2_nonpos(e1.P2m));
+        if (e0.near) e0.sa = __fmul_rn(B[3 * e0.k + 1].y, exp2_nonpos(e0.P2m));
+    }
+}
+
+// The decisions and 1 / (1 - alpha) from the (refined) alpha.
+__device__ __forceinline__ void bwd_finish(BwdPair& e, int lim)
+{
+    e.al = fminf(GSR_ALPHA_MAX, e.sa);
+    e.contrib = e.k < lim && e.front && e.al >= GSR_ALPHA_MIN;
+    e.iom = __fdividef(1.0f, 1.0f - e.al);   // 1 - al >= 0.01
+}
+
+// Dynamic shared memory of the backward: [2][BATCH][3] float4 records (the
+// first 48 bytes of each: mean, conic, opacity, depth, colour),
+// [BATCH][kSumStride] record sums, then per warp the slot buffers of gP and
+// w ([kSlots][kSlotStride] floats each) and the pixels' (dC, dD) (32 float4):
+// 55 KB at BATCH = 128, so four blocks share an SM.
+template <int BATCH>
+constexpr size_t bwd_smem_bytes()
+{
+    return (size_t)2 * BATCH * 48 + (size_t)BATCH * kSumStride * sizeof(float) +
+           (size_t)kWarps * (2 * kSlots * kSlotStride * sizeof(float) + 32 * sizeof(float4));
+}
+
+template <int BX, int BY, int BATCH>
+__global__ void __launch_bounds__(kBlendThreads, 4)
 blend_bwd_kernel(const __grid_constant__ Table Tb, BlendBwdArgs a)
 {
     if (earlier_wait_timed_out(a.status)) return;
-    constexpr int BY = kTilePixels / BX, BPR = BX / kBlk;   // blocks per tile row
-    __shared__ __align__(128) BwdSmem s_warp[kFwdWarps];
-    __shared__ unsigned long long s_queue;
-    if (threadIdx.x == 0) s_queue = (unsigned long long)atomicAdd(a.work, 1u) << 32;   // the first tile
-    const int lane = threadIdx.x & 31;
-    BwdSmem& S = s_warp[threadIdx.x >> 5];
-    if (lane == 0) {
-        S.own = make_uint2(0u, kBlocksPerTile);
-        S.stat[0] = S.stat[1] = 0ull;
+    using TS = TileShape<BX, BY>;
+    extern __shared__ __align__(128) float4 s_buf[];     // layout: see bwd_smem_bytes
+    __shared__ __align__(8) uint64_t s_bar[2];
+    __shared__ unsigned int s_item;
+    __shared__ uint32_t s_idx[2][BATCH];
+    __shared__ uint32_t s_maxlast;
+    using ListT = typename std::conditional<(BATCH <= 256), uint8_t, uint16_t>::type;
+    __shared__ ListT s_list[kWarps][BATCH];
+    float* s_grad = reinterpret_cast<float*>(s_buf + 2 * BATCH * 3);
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    float* s_slots = s_grad + BATCH * kSumStride;
+    float* sgp = s_slots + (size_t)w * 2 * kSlots * kSlotStride;   // this warp's gP slots
+    float* swg = sgp + kSlots * kSlotStride;                          // and its w slots
+    float4* sdcd = reinterpret_cast<float4*>(s_slots + (size_t)kWarps * 2 * kSlots * kSlotStride) + 32 * w;
+    if (tid == 0) {
+        mbar_init(&s_bar[0], 1);
+        mbar_init(&s_bar[1], 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    for (int i = tid; i < BATCH * kSumStride; i += kBlendThreads) s_grad[i] = 0.0f;
     __syncthreads();
-    // this lane's two pixels in a slot row: piece (lane >> 1) ^ e, half lane & 1
-    float2* const gp = reinterpret_cast<float2*>(S.gp) + (lane & 1);
-    float2* const wg = reinterpret_cast<float2*>(S.wg) + (lane & 1);
+    uint32_t par0 = 0u, par1 = 0u;
+    const int lx = TS::lx(tid), ly = TS::ly(tid);
+    unsigned long long pairs_total = 0, witer = 0;
+    bool failed = false;
+    ListT* L = s_list[w];
 
     for (;;) {
-        uint2 next = make_uint2(0u, 0u);
-        if (lane == 0) next = next_block(&s_queue, &S.own, a.work);
-        const unsigned int tile = __shfl_sync(0xffffffffu, next.x, 0), blk = __shfl_sync(0xffffffffu, next.y, 0);
-        if ((int64_t)tile >= Tb.n_tiles) break;
-        const int view = find_view_of_tile(Tb, tile);
+        if (tid == 0) { s_item = atomicAdd(a.work, 1u); s_maxlast = 0; }
+        __syncthreads();
+        const unsigned int item = s_item;
+        if ((int64_t)item >= Tb.n_tiles || failed) break;
+        const int view = find_view_of_tile(Tb, item);
         const DevView& V = Tb.v[view];
-        const int lt = (int)(tile - V.tile_base);
-        const int bx0 = (lt % V.TX) * BX + (int)(blk % BPR) * kBlk, by0 = (lt / V.TX) * BY + (int)(blk / BPR) * kBlk;
-        const uint2 rg = a.ranges[tile];
-        const float fx = __fadd_rn((float)(bx0 + 2 * (lane & 3)), 0.5f), fy = __fadd_rn((float)(by0 + (lane >> 2)), 0.5f);
-        const float fx1 = __fadd_rn(fx, 1.0f);
-        float T[2] = {1.0f, 1.0f}, X[2] = {0.0f, 0.0f};
-        float4 dc[2] = {make_float4(0.0f, 0.0f, 0.0f, 0.0f), make_float4(0.0f, 0.0f, 0.0f, 0.0f)};   // dC, dD
-        int lst[2] = {0, 0};
-        {
-            const int px = bx0 + 2 * (lane & 3), py = by0 + (lane >> 2);
+        const int lt = (int)(item - V.tile_base);
+        const int tx0 = (lt % V.TX) * BX, ty0 = (lt / V.TX) * BY;
+        const int px = tx0 + lx, py = ty0 + ly;
+        const bool inside = px < V.W && py < V.H;
+        const uint2 rg = a.ranges[item];
+        const float pxf = __fadd_rn((float)px, 0.5f), pyf = __fadd_rn((float)py, 0.5f);
+        float Tcur = 1.0f, Tf = 1.0f, dC0 = 0, dC1 = 0, dC2 = 0, dD = 0, dA = 0;
+        uint32_t mylast = 0;
+        if (inside) {
             const int64_t hw = (int64_t)V.W * V.H;
             const int64_t off = (int64_t)py * V.W + px;
             const int64_t pix = V.pix_base + off;
+            Tf = a.tfinal[pix];
+            Tcur = Tf;
+            mylast = a.ncontrib[pix];
             const float* g = a.dl_rgb + 3 * V.pix_base;
-#pragma unroll
-            for (int p = 0; p < 2; ++p) {
-                if (py >= V.H || px + p >= V.W) continue;
-                T[p] = a.tfinal[pix + p];
-                lst[p] = (int)a.ncontrib[pix + p];
-                dc[p].x = g[off + p]; dc[p].y = g[hw + off + p]; dc[p].z = g[2 * hw + off + p];
-                if constexpr (DEPTH) dc[p].w = a.dl_depth[pix + p];
-                const float dA = a.dl_alpha ? a.dl_alpha[pix + p] : 0.0f;
-                // X = dC . S_C + dD S_D - dA T_final, S the suffix sums of the
-                // later colour and depth terms (S_C starts at T_final bg): then
-                // dL/dalpha_k = T_k (dC . c_k + dD z_k) - X / (1 - alpha_k)
-                X[p] = T[p] * (dc[p].x * Tb.bg[0] + dc[p].y * Tb.bg[1] + dc[p].z * Tb.bg[2] - dA);
-            }
+            dC0 = g[off]; dC1 = g[hw + off]; dC2 = g[2 * hw + off];
+            if (a.dl_depth) dD = a.dl_depth[pix];
+            if (a.dl_alpha) dA = a.dl_alpha[pix];
         }
-        const int warp_last = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(lst[0], lst[1]));
-        if (warp_last == 0) continue;
-        // A pixel whose upstream gradient is not finite spoils the gradients of
-        // the entries that it composites and no others of the block: such a
-        // block takes the exact path, which selects instead of multiplying by
-        // zero.
-        const unsigned odd = __ballot_sync(0xffffffffu, !(fabsf(X[0]) + fabsf(X[1]) <= 3.0e38f) ||
-                                                     !(fabsf(dc[0].x) + fabsf(dc[0].y) + fabsf(dc[0].z) + fabsf(dc[0].w) <= 3.0e38f) ||
-                                                     !(fabsf(dc[1].x) + fabsf(dc[1].y) + fabsf(dc[1].z) + fabsf(dc[1].w) <= 3.0e38f));
-        if (lane == 0) S.odd = odd;
-        S.dcd[lane >> 3][2 * (lane & 7)] = dc[0];
-        S.dcd[lane >> 3][2 * (lane & 7) + 1] = dc[1];
-        {
-            const unsigned long long c = warp_sum((unsigned long long)lst[0] + (unsigned long long)lst[1]);
-            if (lane == 0) S.stat[0] += c;
-        }
-        const float cx = (float)(bx0 + kBlk / 2), cy = (float)(by0 + kBlk / 2);
-        const uint2* words = reinterpret_cast<const uint2*>(a.wmask + mask_base(rg.x, tile, a.region2, Tb.n_tiles)) + blk;
-        const uint32_t* vals = a.vals + rg.x;
-        const int n = (int)(rg.y - rg.x);
+        pairs_total += mylast;
+        sdcd[lane] = make_float4(dC0, dC1, dC2, dD);   // read by the slot reduction (after __syncwarp)
+        const float cxw = (float)(tx0 + (w % TS::WPR) * TS::WX + TS::WX / 2);
+        const float cyw = (float)(ty0 + (w / TS::WPR) * TS::WY + TS::WY / 2);
+        const int warp_last = (int)__reduce_max_sync(0xffffffffu, mylast);
+        if (lane == 0 && warp_last) atomicMax(&s_maxlast, (uint32_t)warp_last);
+        // this warp's 8x4 block: half (w / WPR) & 1 of the forward's 8x8 block
+        const uint32_t* words = a.wmask + mask_base(rg.x, item, a.region2, Tb.n_tiles) +
+                                2 * ((w / TS::WPR / 2) * TS::WPR + w % TS::WPR) + ((w / TS::WPR) & 1);
+        __syncthreads();
+        const int maxlast = (int)s_maxlast;
+        const int nb = (maxlast + BATCH - 1) / BATCH;
+        // X = dC . S_C + dD S_D - dA T_final, S the suffix sums of the later
+        // colour and depth terms (S_C starts at T_final bg): then
+        // dL/dalpha_k = T_k (dC . c_k + dD z_k) - X / (1 - alpha_k).
+        float X = Tf * (dC0 * Tb.bg[0] + dC1 * Tb.bg[1] + dC2 * Tb.bg[2] - dA);
 
-        // stage the composited entries of a chunk behind the left-over places
-        auto stage = [&](float4 (*dst)[3], uint32_t m, uint32_t k) {
-            if ((m >> lane) & 1u) {
-                float4* d = dst[kLeft + __popc(m >> lane >> 1)];
-                const float4* src = a.rec + 4 * (size_t)k;
-#pragma unroll
-                for (int i = 0; i < 3; ++i)
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_u32(d + i)), "l"(src + i) : "memory");
+        // batches from the back: the q-th processed batch covers list positions [bb*BATCH, ...)
+        if (nb > 0) {
+            const int bb = nb - 1;
+            issue_batch<3>(a.vals, a.rec, rg.x + bb * BATCH, min(BATCH, maxlast - bb * BATCH), s_buf, &s_bar[0],
+                        s_idx[0]);
+        }
+        for (int q = 0; q < nb; ++q) {
+            const int s = q & 1;
+            const int bb = nb - 1 - q;
+            const int cnt = min(BATCH, maxlast - bb * BATCH);
+            // exactly the (warp, entry) pairs the forward composited: lane j
+            // holds the mask word of the batch's entries 32 j .., read before the
+            // wait (past the warp's last composited entry none was written)
+            uint32_t mword = 0u;
+            if (lane < BATCH / kChunk && bb * BATCH + kChunk * lane < warp_last)
+                mword = words[(size_t)(bb * (BATCH / kChunk) + lane) * kMaskWords];
+            const bool ok = mbar_wait_bounded(&s_bar[s], s ? par1 : par0, a.status, a.wait_ns);
+            if (s) par1 ^= 1u; else par0 ^= 1u;
+            // (this barrier also orders the previous batch's flush before the
+            // reuse of its buffers and sums)
+            if (__syncthreads_or(!ok)) {
+                failed = true;
+                break;
             }
-            asm volatile("cp.async.commit_group;" ::: "memory");
-        };
-        auto load_val = [&](int c) { return c >= 0 && c * kChunk + lane < n ? vals[c * kChunk + lane] : 0u; };
-        auto load_words = [&](int c) { return c >= 0 ? words[(size_t)c * kBlocksPerTile] : make_uint2(0u, 0u); };
-        const int c_last = (warp_last - 1) / kChunk;
-        uint2 wd = load_words(c_last), wn = load_words(c_last - 1);
-        uint32_t kc = load_val(c_last), kn = load_val(c_last - 1);
-        stage(S.dense[c_last & 1], wd.x | wd.y, kc);
-        int left = 0;             // entries of earlier chunks not walked yet
-        int staged = 0;           // entries staged before this chunk
-        // a pixel takes part from its own last composited entry on: the
-        // position of that entry in the walk
-        int start[2] = {0x7fffffff, 0x7fffffff};
-        bool indefinite = false;  // among the left-over entries or the chunk's
-        unsigned int walked = 0;
-        // (one more turn walks what is left over)
-        for (int c = c_last; c >= 0 || (c == -1 && left > 0); --c) {
-            const int s = c & 1;
-            const uint32_t m = wd.x | wd.y;
-            walked += __popc(wd.x) + __popc(wd.y);
-            stage(S.dense[s ^ 1], wn.x | wn.y, kn);
-            const uint32_t kcur = kc;
-            wd = wn;
-            kc = kn;
-            wn = load_words(c - 2);
-            kn = load_val(c - 2);
-            asm volatile("cp.async.wait_group 1;" ::: "memory");
-            bool ind = false;
-            if ((m >> lane) & 1u) {
-                // the lane's own record: its index takes the place of an
-                // unused value
-                float4* d = S.dense[s][kLeft + __popc(m >> lane >> 1)];
-                d[1].w = __uint_as_float(kcur);
-                ind = !(d[2].w > -3.0e38f);
+            if (q + 1 < nb) {
+                const int nbb = bb - 1;
+                issue_batch<3>(a.vals, a.rec, rg.x + nbb * BATCH, min(BATCH, maxlast - nbb * BATCH),
+                            s_buf + (size_t)(s ^ 1) * BATCH * 3, &s_bar[s ^ 1], s_idx[s ^ 1]);
             }
-            indefinite = __any_sync(0xffffffffu, ind || (lane == 0 && S.odd != 0u)) || (left > 0 && indefinite);
+            const float4* B = s_buf + (size_t)s * BATCH * 3;
+            int nl = 0;
+            {
+                const uint32_t lt = (1u << lane) - 1u;
 #pragma unroll
-            for (int p = 0; p < 2; ++p)
-                if (lst[p] > 0 && (lst[p] - 1) / kChunk == c) start[p] = staged + __popc(m >> ((lst[p] - 1) & 31) >> 1);
-            __syncwarp();
-            const int avail = left + __popc(m);
-            int o = kLeft - left, walk = avail / kSlots * kSlots;
-            if (c < 0) {
-                // the block's last group is filled up with records that
-                // composite nowhere (sigma = 0)
-                if (lane < 3 * (kSlots - left)) (&S.dense[s][kLeft][0])[lane] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                __syncwarp();
-                walk = kSlots;
-            }
-            for (const int end = o + walk; o < end; o += kSlots) {
-                const float4 (*D)[3] = S.dense[s] + o;
-                const int rel0 = start[0] - (staged + o - kLeft), rel1 = start[1] - (staged + o - kLeft);
-                // One entry at the lane's two pixels up to alpha.  The value of
-                // 2^P2 here only feeds the adjoint, so the hardware approximation
-                // (ex2.approx, a few ulp from 2^x, as is the contract's
-                // polynomial) serves; the decisions that must be the forward's --
-                // alpha >= 1/255 and the 0.99 clamp -- are re-taken with the
-                // contract's exponential whenever alpha lies within 1.1e-6 of
-                // either threshold (3e-4 relative at 1/255: several times what
-                // the approximations can differ by).  Clamped pixels and records
-                // that need the P2 > 0 test take that path too.
-                struct Entry {
-                    float P[2], sa[2], cdot[2];
-                    float sig;
-                };
-                auto eval = [&](int e) {
-                    Entry t;
-                    const float4 q0 = D[e][0], q1 = D[e][1], q2 = D[e][2];
-                    const float dx0 = __fsub_rn(fx, q0.x), dx1 = __fsub_rn(fx1, q0.x), dy = __fsub_rn(fy, q0.y);
-                    const float tt = __fmul_rn(q0.w, dy), ss = __fmul_rn(__fmul_rn(q1.x, dy), dy);
-                    t.P[0] = __fmaf_rn(dx0, __fmaf_rn(q0.z, dx0, tt), ss);
-                    t.P[1] = __fmaf_rn(dx1, __fmaf_rn(q0.z, dx1, tt), ss);
-                    t.sig = q1.y;
-#pragma unroll
-                    for (int p = 0; p < 2; ++p) {
-                        t.sa[p] = __fmul_rn(q1.y, ex2_approx(t.P[p]));
-                        t.cdot[p] = dc[p].x * q2.x + dc[p].y * q2.y + dc[p].z * q2.z;
-                        if constexpr (DEPTH) t.cdot[p] += dc[p].w * q1.z;
-                    }
-                    return t;
-                };
-                auto near = [&](const Entry& t) {
-                    return t.sa[0] > GSR_ALPHA_MAX - 1.1e-6f || fabsf(t.sa[0] - GSR_ALPHA_MIN) <= 1.1e-6f ||
-                           t.sa[1] > GSR_ALPHA_MAX - 1.1e-6f || fabsf(t.sa[1] - GSR_ALPHA_MIN) <= 1.1e-6f;
-                };
-                // A pixel that does not composite the entry takes alpha = 0: its T
-                // and X stay, and gP and w are zero.
-                auto step = [&](const Entry& t, int e, auto EXACT) {
-                    float gP[2], w[2];
-#pragma unroll
-                    for (int p = 0; p < 2; ++p) {
-                        const bool active = e >= (p ? rel1 : rel0);
-                        float al, alg;   // alpha; alpha where it has a derivative
-                        if constexpr (EXACT.value) {
-                            const float sa = __fmul_rn(t.sig, exp2_walk(t.P[p]));
-                            al = active && t.P[p] <= 0.0f && fminf(GSR_ALPHA_MAX, sa) >= GSR_ALPHA_MIN
-                                     ? fminf(GSR_ALPHA_MAX, sa) : 0.0f;
-                            alg = sa < GSR_ALPHA_MAX ? al : 0.0f;
-                        } else {
-                            al = active && t.sa[p] >= GSR_ALPHA_MIN ? t.sa[p] : 0.0f;
-                            alg = al;
-                        }
-                        const float iom = rcp_approx(1.0f - al);   // 1 - al >= 0.01; 1 for al = 0
-                        const float ga = iom * fmaf(T[p], t.cdot[p], -X[p]);
-                        T[p] = T[p] * iom;
-                        w[p] = al * T[p];
-                        gP[p] = EXACT.value && alg == 0.0f ? 0.0f : ga * alg;
-                        X[p] = fmaf(w[p], t.cdot[p], X[p]);
-                    }
-                    const int at = (16 * e + ((lane >> 1) ^ e)) * 2;
-                    gp[at] = make_float2(gP[0], gP[1]);
-                    wg[at] = make_float2(w[0], w[1]);
-                };
-                // two entries at a time: the second's alpha (independent of T
-                // and X) overlaps the first's update
-#pragma unroll
-                for (int e = 0; e < kSlots; e += 2) {
-                    const Entry t0 = eval(e), t1 = eval(e + 1);
-                    if (__any_sync(0xffffffffu, indefinite || near(t0) || near(t1))) {
-                        step(t0, e, std::true_type{});
-                        step(t1, e + 1, std::true_type{});
-                    } else {
-                        step(t0, e, std::false_type{});
-                        step(t1, e + 1, std::false_type{});
+                for (int j = 0; j < BATCH / 32; ++j) {
+                    if (32 * j < cnt) {
+                        const uint32_t bal = __shfl_sync(0xffffffffu, mword, j);
+                        if ((bal >> lane) & 1u) L[nl + __popc(bal & lt)] = (ListT)(32 * j + lane);
+                        nl += __popc(bal);
                     }
                 }
                 __syncwarp();
-                reduce_group<DEPTH>(S, D, min(kSlots, kLeft + __popc(m) - o), lane, cx, cy, a.grad_rec, a.rec_cap);
+            }
+            witer += nl;
+            const int lim = (int)mylast - bb * BATCH;   // this pixel's entries k < lim
+            // The walk is back to front: each entry's adjoint needs T and X as
+            // left by the entry after it.  Branch-free: every lane evaluates
+            // the pair, and a lane that does not composite it stores zero gP
+            // and w into slot s of its warp's buffers.  Entries are taken two
+            // at a time so that the second's alpha (independent of T and X)
+            // overlaps the first's.
+            auto step = [&](const BwdPair& e, int s) {
+                const float Tk = Tcur * e.iom;
+                const float wgt = e.contrib ? e.al * Tk : 0.0f;
+                // the clamped alpha (sa >= 0.99) has no derivative
+                const float ga = (e.contrib && e.sa < GSR_ALPHA_MAX) ? Tk * e.cdot - e.iom * X : 0.0f;
+                // dL/dP2 / ln2; the record's coefficients, ln2 and the sign of
+                // the mean gradient are applied once per record when the
+                // shared sums are flushed
+                const float gP = ga * e.al;
+                X = fmaf(wgt, e.cdot, X);
+                Tcur = e.contrib ? Tk : Tcur;
+                const int at = s * kSlotStride + slot_col(lane, s);
+                sgp[at] = gP;
+                swg[at] = wgt;
+            };
+            auto pair = [&](int i1, int s) {
+                BwdPair e1 = bwd_pair(B, L[i1], pxf, pyf, dC0, dC1, dC2, dD);
+                BwdPair e0 = bwd_pair(B, L[i1 - 1], pxf, pyf, dC0, dC1, dC2, dD);
+                bwd_refine(B, e1, e0);
+                bwd_finish(e1, lim);
+                bwd_finish(e0, lim);
+                step(e1, s);
+                step(e0, s + 1);
+            };
+            int i = nl - 1;
+            // whole groups of kSlots entries, slot indices fixed at compile time
+            for (; i >= kSlots - 1; i -= kSlots) {
+#pragma unroll
+                for (int p = 0; p < kSlots; p += 2) pair(i - p, p);
+                __syncwarp();
+                slots_reduce(sgp, swg, sdcd, kSlots, lane, L, i, B, cxw, cyw, s_grad);
                 __syncwarp();
             }
-            staged += __popc(m);
-            left = max(0, avail - walk);
-            // the entries left over go in front of the next chunk's
-            if (lane < 3 * left) (&S.dense[s ^ 1][0][0])[3 * (kLeft - left) + lane] = (&S.dense[s][0][0])[3 * o + lane];
-            __syncwarp();
+            // the last (fewer than kSlots) entries
+            const int i0 = i;      // list position of slot 0's entry
+            int slot = 0;          // entries in the slot buffers (warp-uniform)
+            for (; i >= 1; i -= 2, slot += 2) pair(i, slot);
+            if (i == 0) {
+                BwdPair e = bwd_pair(B, L[0], pxf, pyf, dC0, dC1, dC2, dD);
+                if (__any_sync(0xffffffffu, e.near) && e.near) e.sa = __fmul_rn(B[3 * e.k + 1].y, exp2_nonpos(e.P2m));
+                bwd_finish(e, lim);
+                step(e, slot);
+                ++slot;
+            }
+            if (slot) {
+                __syncwarp();
+                slots_reduce(sgp, swg, sdcd, slot, lane, L, i0, B, cxw, cyw, s_grad);
+                __syncwarp();
+            }
+            __syncthreads();
+            for (int t = tid; t < cnt; t += kBlendThreads) {
+                float* sg = s_grad + t * kSumStride;
+                // sums of gP dx, gP dy -> d(u, v); gP dx^2, gP dx dy, gP dy^2 -> d(qa, qb, qc)
+                const float4 q0 = B[3 * t];
+                const float qc = B[3 * t + 1].x, sig = B[3 * t + 1].y;
+                const float sx = sg[0], sy = sg[1];
+                const float4 v0 = make_float4(-GSR_LN2 * (2.0f * q0.z * sx + q0.w * sy),
+                                              -GSR_LN2 * (q0.w * sx + 2.0f * qc * sy), GSR_LN2 * sg[2],
+                                              GSR_LN2 * sg[3]);
+                // sum dL/dalpha G over the pixels where alpha is not clamped = sum gP / sigma
+                const float4 v1 = make_float4(GSR_LN2 * sg[4], sg[5] / sig, sg[6], 0.0f);
+                const float4 v2 = make_float4(sg[7], sg[8], sg[9], 0.0f);
+                const uint32_t k = s_idx[s][t];
+                if (v0.x != 0.0f || v0.y != 0.0f || v0.z != 0.0f || v0.w != 0.0f || v1.x != 0.0f || v1.y != 0.0f ||
+                    v1.z != 0.0f || v2.x != 0.0f || v2.y != 0.0f || v2.z != 0.0f) {
+                    atomicAdd(a.grad_rec + 3 * (size_t)k, v0);
+                    atomicAdd(a.grad_rec + 3 * (size_t)k + 1, v1);
+                    atomicAdd(a.grad_rec + 3 * (size_t)k + 2, v2);
+                }
+#pragma unroll
+                for (int c = 0; c < 10; ++c) sg[c] = 0.0f;
+            }
         }
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        if (lane == 0) S.stat[1] += walked;
+        __syncthreads();   // every thread has read s_item / s_maxlast of this tile; the flush is done
     }
-    if (lane == 0) {
-        if (S.stat[0]) atomicAdd(a.counters + kCntBwdPairs, S.stat[0]);
-        if (S.stat[1]) atomicAdd(a.counters + kCntWarpBwd, S.stat[1]);
-    }
+    pairs_total = warp_sum(pairs_total);
+    if (lane == 0 && pairs_total) atomicAdd(a.counters + kCntBwdPairs, pairs_total);
+    if (lane == 0 && witer) atomicAdd(a.counters + kCntWarpBwd, witer);
 }
 
 // ---------------------------------------------------------------------------
@@ -878,30 +898,28 @@ static void fwd_one(const Table& T, const BlendFwdArgs& a, int num_sms, cudaStre
     else fwd_launch<BX, false>(T, a, num_sms, s);
 }
 
-template <int BX, bool DEPTH>
-static void bwd_launch(const Table& T, const BlendBwdArgs& a, int num_sms, cudaStream_t s)
+template <int BX, int BY, int BATCH>
+static void bwd_one(const Table& T, const BlendBwdArgs& a, int num_sms, cudaStream_t s)
 {
-    auto kern = blend_bwd_kernel<BX, DEPTH>;
+    auto kern = blend_bwd_kernel<BX, BY, BATCH>;
+    const size_t smem = bwd_smem_bytes<BATCH>();
+    // function attributes and occupancy are per device
     static std::atomic<int> per_sm_dev[kMaxDevices];
     const int per_sm = per_device_once(per_sm_dev, [&] {
         int n = 0;
-        // six blocks of 36 KB fit an SM only with all of the unified L1 as shared memory
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        // all of the unified L1 as shared memory: four blocks of the
+        // 128-record variant fit (the kernel keeps records in shared memory,
+        // not in L1)
         cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kFwdThreads, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kBlendThreads, smem);
         return n < 1 ? 1 : n;
     });
     int64_t grid = (int64_t)num_sms * per_sm;
     if (grid > T.n_tiles) grid = T.n_tiles;
     if (grid < 1) return;
     GSR_COUNT_LAUNCH();
-    kern<<<(unsigned)grid, kFwdThreads, 0, s>>>(T, a);
-}
-
-template <int BX>
-static void bwd_one(const Table& T, const BlendBwdArgs& a, int num_sms, cudaStream_t s)
-{
-    if (a.dl_depth) bwd_launch<BX, true>(T, a, num_sms, s);
-    else bwd_launch<BX, false>(T, a, num_sms, s);
+    kern<<<(unsigned)grid, kBlendThreads, smem, s>>>(T, a);
 }
 
 bool blend_supported(int tw, int th, int batch)
@@ -911,7 +929,25 @@ bool blend_supported(int tw, int th, int batch)
     return shape && b;
 }
 
-// (both directions stage chunks of 32 entries per warp whatever the configured batch)
+#define GSR_DISPATCH(FN, T, batch, ...)                                                          \
+    do {                                                                                         \
+        const int tw_ = (T).tile_w, th_ = (T).tile_h;                                            \
+        if (tw_ == 16 && th_ == 16) {                                                            \
+            if (batch == 128) FN<16, 16, 128>(T, __VA_ARGS__);                                   \
+            else if (batch == 256) FN<16, 16, 256>(T, __VA_ARGS__);                              \
+            else FN<16, 16, 512>(T, __VA_ARGS__);                                                \
+        } else if (tw_ == 32 && th_ == 8) {                                                      \
+            if (batch == 128) FN<32, 8, 128>(T, __VA_ARGS__);                                    \
+            else if (batch == 256) FN<32, 8, 256>(T, __VA_ARGS__);                               \
+            else FN<32, 8, 512>(T, __VA_ARGS__);                                                 \
+        } else {                                                                                 \
+            if (batch == 128) FN<8, 32, 128>(T, __VA_ARGS__);                                    \
+            else if (batch == 256) FN<8, 32, 256>(T, __VA_ARGS__);                               \
+            else FN<8, 32, 512>(T, __VA_ARGS__);                                                 \
+        }                                                                                        \
+    } while (0)
+
+// (the forward stages chunks of 32 entries per warp whatever the staging batch)
 void launch_blend_fwd(const Table& T, const BlendFwdArgs& a, int num_sms, cudaStream_t s)
 {
     if (T.tile_w == 16) fwd_one<16>(T, a, num_sms, s);
@@ -924,11 +960,9 @@ size_t blend_mask_bytes(int64_t list_span, int64_t n_tiles)
     return ((size_t)(list_span / kChunk) + 2 * (size_t)n_tiles + 1) * kMaskWords * sizeof(uint32_t);
 }
 
-void launch_blend_bwd(const Table& T, const BlendBwdArgs& a, int num_sms, cudaStream_t s)
+void launch_blend_bwd(const Table& T, int batch, const BlendBwdArgs& a, int num_sms, cudaStream_t s)
 {
-    if (T.tile_w == 16) bwd_one<16>(T, a, num_sms, s);
-    else if (T.tile_w == 32) bwd_one<32>(T, a, num_sms, s);
-    else bwd_one<8>(T, a, num_sms, s);
+    GSR_DISPATCH(bwd_one, T, batch, a, num_sms, s);
 }
 
 }  // namespace gsr

@@ -22,7 +22,7 @@ namespace gsr {
 
 constexpr int kMaxViews = 64;
 constexpr int kRecordBytes = 64;        // projected record: 4 x float4
-constexpr int kGradBytes = 80;          // per-record 2D gradient: ten binary64 sums (see GradRec)
+constexpr int kGradFloats = 12;         // per-record 2D gradient: 3 x float4
 
 // status word bits (device)
 constexpr uint32_t kErrRecCapacity = 1u;
@@ -561,27 +561,6 @@ __device__ __forceinline__ bool earlier_wait_timed_out(const uint32_t* status)
     if (threadIdx.x == 0) s_timed_out = (*reinterpret_cast<const volatile uint32_t*>(status) & kErrTimeout) != 0;
     __syncthreads();
     return s_timed_out != 0;
-}
-
-// ---------------------------------------------------------------------------
-// per-record 2D gradient
-// ---------------------------------------------------------------------------
-// Ten binary64 sums per compact record, {u, qa, qc, r, v, qb, sigma, g} at
-// base + 8 k and {z, b} at base + 8 cap + 2 k: the four values that four lanes
-// of the backward blend add at a time share a 32-byte sector.
-struct GradRec {
-    float u, v, qa, qb, qc, sig, z, r, g, b;
-};
-__device__ __forceinline__ GradRec load_grad_rec(const double* base, int64_t cap, int64_t k)
-{
-    const double2* p = reinterpret_cast<const double2*>(base + 8 * k);
-    const double2 a0 = p[0], a1 = p[1], a2 = p[2], a3 = p[3];
-    const double2 c = *reinterpret_cast<const double2*>(base + 8 * cap + 2 * k);
-    GradRec o;
-    o.u = (float)a0.x; o.qa = (float)a0.y; o.qc = (float)a1.x; o.r = (float)a1.y;
-    o.v = (float)a2.x; o.qb = (float)a2.y; o.sig = (float)a3.x; o.g = (float)a3.y;
-    o.z = (float)c.x; o.b = (float)c.y;
-    return o;
 }
 
 // ---------------------------------------------------------------------------

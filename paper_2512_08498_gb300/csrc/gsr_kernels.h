@@ -118,8 +118,7 @@ struct PreprocessBwdArgs {
     const float* sh;
     const uint4* vis_aux;
     const uint32_t* kstart;
-    const double* grad_rec;        // see GradRec
-    int64_t rec_cap;
+    const float4* grad_rec;        // [n_vis][3]
     float* grad_means;
     float* grad_log_scales;
     float* grad_quats;
@@ -253,7 +252,7 @@ struct BlendFwdArgs {
     uint32_t* ncontrib;
     uint32_t* wmask;               // blend_mask_bytes: which 8x4 blocks composited each list entry (may be nullptr)
     uint32_t region2 = 0xffffffffu;    // first list position of the second region (0xffffffff: one region)
-    unsigned int* work;            // zeroed tile counter
+    unsigned int* work;            // zeroed block counter
     uint32_t* status;
     unsigned long long* counters;
     bool count_pairs = true;       // examined and composited pair counters
@@ -284,17 +283,17 @@ struct BlendBwdArgs {
     const float* dl_alpha;         // may be nullptr
     const uint32_t* wmask;         // written by the forward that filled the saved state
     uint32_t region2 = 0xffffffffu;    // as in that forward
-    double* grad_rec;              // see GradRec, zeroed
-    int64_t rec_cap;
+    float4* grad_rec;              // [n_vis][3], zeroed
     unsigned int* work;            // zeroed tile counter
     uint32_t* status;
     unsigned long long* counters;
+    uint64_t wait_ns = kWaitLimitNs;   // limit of each mbarrier wait
 };
 
 bool blend_supported(int tile_w, int tile_h, int batch);
 void launch_blend_fwd(const Table& T, const BlendFwdArgs& a, int num_sms, cudaStream_t s);
 size_t blend_mask_bytes(int64_t list_span, int64_t n_tiles);   // composited-entry masks of a forward's lists
-void launch_blend_bwd(const Table& T, const BlendBwdArgs& a, int num_sms, cudaStream_t s);
+void launch_blend_bwd(const Table& T, int batch, const BlendBwdArgs& a, int num_sms, cudaStream_t s);
 
 // ---- insertion probability (Sec. 3.2, Eq. 4-6) -------------------------------
 constexpr int kInsMaxRadius = 7;
@@ -410,7 +409,7 @@ struct DebugArgs {
     const uint32_t* tile_val;
     const float4* rec;
     const uint4* vis_aux;
-    const double* grad_rec;
+    const float4* grad_rec;
     const unsigned long long* counters;
     int64_t rec_cap, inst_cap;
     int64_t first = 0, count = INT64_MAX;   // list positions exported by launch_debug_lists

@@ -911,10 +911,10 @@ preprocess_bwd_kernel(const __grid_constant__ Table Tb, int gi, PreprocessBwdArg
             const float* kk = a.sh + (size_t)gauss * K * 3;
             Chain f;
             chain_values(V, mu, ls, q, a.opacity[gauss], aux.w, f);
-            const GradRec gr = load_grad_rec(a.grad_rec, a.rec_cap, k);
-            gcol[0] = (f.cclamp & 1u) ? 0.0f : gr.r;
-            gcol[1] = (f.cclamp & 2u) ? 0.0f : gr.g;
-            gcol[2] = (f.cclamp & 4u) ? 0.0f : gr.b;
+            const float4 g0 = a.grad_rec[3 * k], g1 = a.grad_rec[3 * k + 1], g2 = a.grad_rec[3 * k + 2];
+            gcol[0] = (f.cclamp & 1u) ? 0.0f : g2.x;
+            gcol[1] = (f.cclamp & 2u) ? 0.0f : g2.y;
+            gcol[2] = (f.cclamp & 4u) ? 0.0f : g2.z;
 
             // Geometry adjoint.  Records of large angular size go to the
             // extended-precision queue (see needs_binary64); the rest are evaluated here
@@ -925,8 +925,8 @@ preprocess_bwd_kernel(const __grid_constant__ Table Tb, int gi, PreprocessBwdArg
                 else atomicOr(a.status, kErrInternal);
             } else {
                 float pose[8];
-                geom_adjoint<float>(f, V, gr.u, gr.v, gr.qa * GSR_NHALF_L2E, gr.qb * GSR_NL2E, gr.qc * GSR_NHALF_L2E,
-                                    gr.z, want_cam, v, v + 3, v + 6, pose);
+                geom_adjoint<float>(f, V, g0.x, g0.y, g0.z * GSR_NHALF_L2E, g0.w * GSR_NL2E, g1.x * GSR_NHALF_L2E,
+                                    g1.z, want_cam, v, v + 3, v + 6, pose);
                 if (want_cam) {
                     float* sp = s_pose[wid][view - G.first_view];
 #pragma unroll
@@ -955,7 +955,7 @@ preprocess_bwd_kernel(const __grid_constant__ Table Tb, int gi, PreprocessBwdArg
 #pragma unroll
             for (int i = 0; i < 3; ++i) v[i] += (gdir[i] - f.dir[i] * dd) * f.idn;
             // opacity
-            v[10] = gr.sig * f.sig * (1.0f - f.sig);
+            v[10] = g1.y * f.sig * (1.0f - f.sig);
         }
 
         // segments of equal j (lanes without a record have unique sentinels)
@@ -1171,9 +1171,9 @@ preprocess_bwd64_kernel(const __grid_constant__ Table Tb, PreprocessBwdArgs a)
         qq[0] = q4.x; qq[1] = q4.y; qq[2] = q4.z; qq[3] = q4.w;
         Chain f;
         chain_values(V, mu, ls, qq, a.opacity[gauss], aux.w, f);
-        const GradRec gr = load_grad_rec(a.grad_rec, a.rec_cap, k);
+        const float4 g0 = a.grad_rec[3 * (size_t)k], g1 = a.grad_rec[3 * (size_t)k + 1];
         df64 gmu[3] = {0, 0, 0}, gls[3] = {0, 0, 0}, gq[4] = {0, 0, 0, 0}, pose[8];
-        geom_adjoint<df64>(f, V, gr.u, gr.v, gr.qa * GSR_NHALF_L2E, gr.qb * GSR_NL2E, gr.qc * GSR_NHALF_L2E, gr.z,
+        geom_adjoint<df64>(f, V, g0.x, g0.y, g0.z * GSR_NHALF_L2E, g0.w * GSR_NL2E, g1.x * GSR_NHALF_L2E, g1.z,
                            want_cam, gmu, gls, gq, pose);
 #pragma unroll
         for (int i = 0; i < 3; ++i) {

@@ -1053,10 +1053,10 @@ __global__ void debug_records_kernel(const __grid_constant__ Table Tb, DebugArgs
         if (a.flags_out) a.flags_out[r] = 0u;
         if (a.grec_out && a.grad_rec) {
             float* o = a.grec_out + 12 * r;
-            const GradRec q = load_grad_rec(a.grad_rec, a.rec_cap, k);
-            o[0] = q.u; o[1] = q.v; o[2] = q.qa; o[3] = q.qb;
-            o[4] = q.qc; o[5] = q.sig; o[6] = q.z; o[7] = 0.0f;
-            o[8] = q.r; o[9] = q.g; o[10] = q.b; o[11] = 0.0f;
+            const float4 g0 = a.grad_rec[3 * k], g1 = a.grad_rec[3 * k + 1], g2 = a.grad_rec[3 * k + 2];
+            o[0] = g0.x; o[1] = g0.y; o[2] = g0.z; o[3] = g0.w;
+            o[4] = g1.x; o[5] = g1.y; o[6] = g1.z; o[7] = g1.w;
+            o[8] = g2.x; o[9] = g2.y; o[10] = g2.z; o[11] = g2.w;
         }
     }
 }
