@@ -101,9 +101,10 @@ typedef struct gsr_saved gsr_saved;
 
 typedef struct {
     int tile_w, tile_h;   /* screen tile: 16x16, 32x8 or 8x32                 */
-    int blend_batch;      /* Gaussians staged in shared memory per batch by
-                             the backward blend when blend_batch_bwd is 0:
-                             128, 256 or 512 (the forward stages 32 per warp) */
+    int blend_batch;      /* Gaussians staged in shared memory per batch: 128,
+                             256 or 512 (by the backward blend only where
+                             blend_batch_bwd is 0; a forward over long even
+                             lists stages 32 per warp whatever the value)     */
     int sh_degree;        /* 0 .. 3                                           */
     float near_plane;     /* records with camera z <= near are culled (0.2)   */
     float bg[3];          /* background colour                                */

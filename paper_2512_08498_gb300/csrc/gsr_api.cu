@@ -745,7 +745,14 @@ static void enqueue_forward(gsr_ctx* ctx, gsr_saved* s, const gsr_gaussians* g, 
     ba.region2 = two ? (uint32_t)s->region2 : 0xffffffffu;
     ba.status = status;
     ba.counters = counters;
+    ba.wait_ns = ctx->wait_ns;
     ba.count_pairs = !(ctx->cfg.flags & GSR_FLAG_NO_PAIR_COUNTS);
+    LongList long_list;
+    if (const int parts = blend_fwd_list_parts(T, ba.count_pairs, ctx->num_sms)) {
+        long_list.flag = counters + kCntLongList;
+        long_list.parts = parts;
+        ba.long_list = long_list.flag;
+    }
     ba.prefix = prefix;
     ba.open_tiles = two ? s->open_tiles.as<uint32_t>() : nullptr;
     ba.open_blocks = two ? ba.open_tiles + open_words(T.n_tiles) : nullptr;
@@ -810,6 +817,8 @@ static void enqueue_forward(gsr_ctx* ctx, gsr_saved* s, const gsr_gaussians* g, 
             RowListArgs ra{};
             row_lists_layout(T, s->row_cap, ctx->row_work.as<unsigned char>(), &ra);
             ra.n_rows = da.n_rows;
+            ra.inst_count = inst_count;
+            ra.lists = second ? LongList{} : long_list;
             ra.order = tv;
             ra.runs = da.runs;
             ra.sorted = ctx->dup_rows.as<uint2>() + s->row_cap;
@@ -823,19 +832,20 @@ static void enqueue_forward(gsr_ctx* ctx, gsr_saved* s, const gsr_gaussians* g, 
             ra.base = (uint32_t)base;
             cudaMemsetAsync(ra.row_range, 0, (size_t)ra.n_trows * 8, st);
             launch_ranges((passes & 1) ? tk : rk, da.n_rows, s->row_cap, ra.row_range, ra.n_trows, 0, status,
-                          ctx->num_sms, st);
+                          LongList{}, ctx->num_sms, st);
             launch_row_lists(T, ra, ctx->num_sms, st);
         } else {
             launch_duplicate(T, da, ctx->num_sms, st);
             prof_mark(pr, m0 + 1, st);
             radix_sort_pairs(xk, xv, yk, yv, false, inst_count, s->inst_cap, bits, rs, st);
             prof_mark(pr, m0 + 2, st);
-            launch_ranges(rk, inst_count, s->inst_cap, s->ranges.as<uint2>(), T.n_tiles, base, status, ctx->num_sms, st);
+            launch_ranges(rk, inst_count, s->inst_cap, s->ranges.as<uint2>(), T.n_tiles, base, status,
+                          second ? LongList{} : long_list, ctx->num_sms, st);
         }
         ba.round = r;
         ba.work = reinterpret_cast<unsigned int*>(ctrl + (second ? kCtrlWorkFwd2 : kCtrlWorkFwd));
         prof_mark(pr, m0 + 3, st);
-        launch_blend_fwd(T, ba, ctx->num_sms, st);
+        launch_blend_fwd(T, s->batch, ba, ctx->num_sms, st);
         prof_mark(pr, m0 + 4, st);
     }
 }
@@ -1838,7 +1848,7 @@ gsr_status gsr_forward_noalloc(const gsr_config* cfg, const gsr_gaussians* g, co
     da.full_count = counters + kCntFullInst;
     launch_duplicate(T, da, num_sms, st);
     radix_sort_pairs(xk, xv, yk, yv, false, counters + kCntInstances, kNaInstances, bits, rs, st);
-    launch_ranges(tile_key, counters + kCntInstances, kNaInstances, ranges, T.n_tiles, 0, status, num_sms, st);
+    launch_ranges(tile_key, counters + kCntInstances, kNaInstances, ranges, T.n_tiles, 0, status, LongList{}, num_sms, st);
 
     BlendFwdArgs ba;
     ba.rec = d_rec;
@@ -1854,7 +1864,7 @@ gsr_status gsr_forward_noalloc(const gsr_config* cfg, const gsr_gaussians* g, co
     ba.status = status;
     ba.counters = counters;
     ba.count_pairs = !(cfg->flags & GSR_FLAG_NO_PAIR_COUNTS);
-    launch_blend_fwd(T, ba, num_sms, st);
+    launch_blend_fwd(T, cfg->blend_batch, ba, num_sms, st);
     if (cudaGetLastError() != cudaSuccess) return GSR_ERR_CUDA;
 
     // the instance count is only known on the device: read the status word

@@ -3,18 +3,19 @@
 // One persistent launch per direction covers every (view, tile) of the batch:
 // work comes from an atomic tile counter, so views of uneven size and tiles of
 // uneven list length share one grid of (SMs x resident blocks).  A tile has
-// 256 pixels.  The forward gives an 8x8 pixel block to a warp that waits for
-// no other (see below); the backward gives the tile to a block of eight warps
-// over 8x4 pixels each and walks the list in batches of BATCH records, each
-// gathered into shared memory with one bulk async copy (cp.async.bulk, the TMA
-// engine) per record (the 48 bytes it reads), completing on an mbarrier,
-// double-buffered so the gather of batch b+1 overlaps the arithmetic of batch b.
+// 256 pixels.  The backward, and the forward's tile form, give the tile to a block
+// of eight warps over 8x4 pixels each and walk the list in batches of BATCH
+// records, each gathered into shared memory with one bulk async copy
+// (cp.async.bulk, the TMA engine) per record (64 bytes; the backward stages only
+// the 48 it reads), completing on an mbarrier, double-buffered so the gather of
+// batch b+1 overlaps the arithmetic of batch b.  The forward's warp form gives an
+// 8x8 pixel block to a warp that waits for no other (see below).
 //
 // Culling: every record carries a conservative box outside which its
 // binary32 alpha is certainly below 1/255 (see alpha_box in
 // gsr_preprocess.cu) and a threshold of its exponent.  A forward warp walks only
-// the entries that can touch its block, in list order, and records which 8x4
-// halves composited each entry; the backward walks exactly those.  Skipped
+// the entries that can touch its pixels, in list order, and records which 8x4
+// blocks composited each entry; the backward walks exactly those.  Skipped
 // pairs would have been skipped by the 1/255 rule anyway, so every decision
 // (blend, skip, stop, contributor count) is unchanged.
 //
@@ -33,6 +34,7 @@
 //   warp through per-warp slot buffers (one entry per lane pair, see
 //   slots_reduce), over the CTA in shared memory, and added to the
 //   per-record gradient with one vector atomic per 16 bytes.
+#include <algorithm>
 #include <type_traits>
 
 #include "gsr_common.cuh"
@@ -86,8 +88,381 @@ __device__ __forceinline__ float rect_max_form(float x0, float x1, float y0, flo
 }
 
 // ---------------------------------------------------------------------------
+// composited-entry masks
+// ---------------------------------------------------------------------------
+constexpr int kChunk = 32;              // list entries per mask word
+constexpr int kBlk = 8;                 // a pixel block's side
+constexpr int kBlocksPerTile = kBlendThreads / (kBlk * kBlk);
+
+// First 32-bit word of a tile's composited-entry masks: kMaskWords words per
+// chunk of 32 list positions, word 2 blk + h the entries that some pixel of
+// the upper (h = 0) or lower 8x4 half of block blk composited.  A tile's
+// chunks start at its range's first position / 32 plus the tile id (plus the
+// tile count in the second list region), so no two tiles' words overlap:
+// floor((x + n) / 32) - floor(x / 32) + 1 >= ceil(n / 32).
+constexpr int kMaskWords = 2 * kBlocksPerTile;
+__device__ __forceinline__ size_t mask_base(uint32_t first, uint32_t tile, uint32_t region2, int64_t n_tiles)
+{
+    return (size_t)kMaskWords * ((size_t)(first / kChunk) + tile + (first >= region2 ? (size_t)n_tiles : (size_t)0));
+}
+// The word of the 8x4 pixels of warp w of a tile-wide block, WPR warps per tile row.
+template <int WPR>
+__device__ __forceinline__ int mask_word(int w) { return 2 * ((w / WPR / 2) * WPR + w % WPR) + ((w / WPR) & 1); }
+
+// ---------------------------------------------------------------------------
 // forward
 // ---------------------------------------------------------------------------
+// Two forms, the same results bit for bit.
+//   warp form  one warp per 8x8 pixel block, two pixels per lane, no waits
+//              between warps (below): fewer instructions per pair.
+//   tile form  the tile's eight 8x4 warps in step, a pixel per lane: twice the
+//              warps on a tile and the shorter chain per list entry.
+// The sum of the work decides for the warp form, the longest lists' chains for the
+// tile form.  So the lists choose, on the device: the warp form if the longest one has at
+// most 1 / kWarpFormShare of the instances per resident block (the kernels that
+// make the lists see it as they go).  Times of
+// the two (tile, warp form; ms) around that line, from 4096 tiles on:
+//   share 3.9  six 1600x900 views, 1M Gaussians      2.10  1.63
+//   share 1.9  1237x701 and smaller, 32x8 tiles      0.263 0.229
+//   share 1.9  24 views of 606x348                   0.351 0.353
+//   share 1.5  18 1080p views of the road, 300k      3.20  2.90
+//   share 1.0  one view of 1242x995                  0.090 0.123
+//   share 0.8  24 views of 400x225, 300k             1.08  1.38
+//   share 0.2  24 views up to 994x845 of the road    1.40  2.97
+// Fewer tiles never fill the chip at that share (3840 tiles at share 2.6: 0.193
+// and 0.175; 2300 at 2.0: 0.107 and 0.114), and small images would feel the
+// second launch (the form not taken returns after 4 us).
+constexpr int64_t kWarpFormMinTiles = 4096;
+constexpr double kWarpFormShare = 1.5;
+__device__ __forceinline__ bool warp_form(const BlendFwdArgs& a) { return a.long_list && *a.long_list == 0ull; }
+
+// ---- tile form
+// A block has one thread per pixel and takes the next tile from the counter.  The
+// list is walked in batches of BATCH records, each gathered into shared memory with
+// one bulk async copy per record, completing on an mbarrier, double-buffered so
+// that the gather of batch b+1 overlaps the arithmetic of batch b.  After a batch
+// lands, each record's box is tested against the eight warps' 8x4 pixel blocks, and
+// each warp walks only the entries that can touch its pixels.
+
+// Bit w of mask[t]: record t can reach alpha >= 1/255 at a pixel centre of
+// warp w.  Two conservative tests: the record's alpha box against the warp's
+// block, then the maximum of the record's exponent over the block against
+// its culling threshold (record slot 11).  The corner offsets are rounded
+// exactly as the blend rounds each pixel's offset, so every pixel's rounded
+// offset lies in the tested rectangle.
+template <int BX, int BY>
+__device__ __forceinline__ void warp_masks(const float4* B, int cnt, int tx0, int ty0, uint8_t* s_mask)
+{
+    using TS = TileShape<BX, BY>;
+    for (int t = threadIdx.x; t < cnt; t += kBlendThreads) {
+        const float4 r0 = B[4 * t];
+        const float qc = B[4 * t + 1].x;
+        const float thr_cull = B[4 * t + 2].w;
+        const float4 bb = B[4 * t + 3];
+        const float kx = -r0.w / (2.0f * r0.z), ky = -r0.w / (2.0f * qc);
+        uint32_t m = 0;
+#pragma unroll 1
+        for (int w = 0; w < kWarps; ++w) {
+            const float X0 = (float)(tx0 + (w % TS::WPR) * TS::WX);
+            const float Y0 = (float)(ty0 + (w / TS::WPR) * TS::WY);
+            bool hit = bb.x <= X0 + (TS::WX - 0.5f) && bb.y >= X0 + 0.5f && bb.z <= Y0 + (TS::WY - 0.5f) &&
+                       bb.w >= Y0 + 0.5f;
+            if (hit && thr_cull > -3.0e38f) {
+                const float x0 = __fsub_rn(__fadd_rn(X0, 0.5f), r0.x);
+                const float x1 = __fsub_rn(__fadd_rn(X0, TS::WX - 0.5f), r0.x);
+                const float y0 = __fsub_rn(__fadd_rn(Y0, 0.5f), r0.y);
+                const float y1 = __fsub_rn(__fadd_rn(Y0, TS::WY - 0.5f), r0.y);
+                hit = rect_max_form(x0, x1, y0, y1, r0.z, r0.w, qc, kx, ky) >= thr_cull;
+            }
+            m |= (uint32_t)hit << w;
+        }
+        s_mask[t] = (uint8_t)m;
+    }
+}
+
+// This warp's entries of the batch, in list order; returns their number.
+__device__ __forceinline__ int warp_list(const uint8_t* s_mask, int cnt, int w, int lane, uint16_t* list)
+{
+    int nl = 0;
+    const uint32_t lt = (1u << lane) - 1u;
+    for (int base = 0; base < cnt; base += 32) {
+        const int t = base + lane;
+        const bool bit = t < cnt && ((s_mask[t] >> w) & 1u);
+        const uint32_t bal = __ballot_sync(0xffffffffu, bit);
+        if (bit) list[nl + __popc(bal & lt)] = (uint16_t)t;
+        nl += __popc(bal);
+    }
+    __syncwarp();
+    return nl;
+}
+
+// One (pixel, entry) pair of the forward up to alpha (independent of T).
+struct TilePair {
+    int k;
+    float P2, al;
+    float4 c;      // colour, depth
+};
+
+__device__ __forceinline__ TilePair tile_pair(const float4* B, int k, float pxf, float pyf)
+{
+    TilePair e;
+    e.k = k;
+    const float4 r0 = B[4 * k];
+    const float4 r1 = B[4 * k + 1];
+    const float4 r2 = B[4 * k + 2];
+    const float dx = __fsub_rn(pxf, r0.x), dy = __fsub_rn(pyf, r0.y);
+    e.P2 = __fmaf_rn(dx, __fmaf_rn(r0.z, dx, __fmul_rn(r0.w, dy)), __fmul_rn(__fmul_rn(r1.x, dy), dy));
+    e.al = fminf(GSR_ALPHA_MAX, __fmul_rn(r1.y, exp2_nonpos(fminf(e.P2, 0.0f))));
+    e.c = make_float4(r2.x, r2.y, r2.z, r1.z);
+    return e;
+}
+
+// Four blocks per SM: 64 registers (the two-entry walk would otherwise take
+// 72 and leave room for three).  COUNT: keep the per-pixel examined and
+// composited counts (statistics only; a separate instantiation because the
+// two running counts cost about 6 % of the walk).
+template <int BX, int BY, int BATCH, bool COUNT>
+__global__ void __launch_bounds__(kBlendThreads, 4)
+blend_fwd_tile_kernel(const __grid_constant__ Table Tb, BlendFwdArgs a)
+{
+    if (earlier_wait_timed_out(a.status) || warp_form(a)) return;
+    using TS = TileShape<BX, BY>;
+    extern __shared__ __align__(128) float4 s_buf[];     // [2][BATCH][4]
+    __shared__ __align__(8) uint64_t s_bar[2];
+    __shared__ unsigned int s_item;
+    __shared__ uint8_t s_mask[BATCH];
+    __shared__ uint16_t s_list[kWarps][BATCH];
+    __shared__ __align__(16) uint8_t s_wb[kWarps][BATCH]; // per warp: composited each entry of the batch
+    // per tile (kept in shared memory, off the walk's registers): the warps'
+    // walked entries, and the list entries up to the end of the batch in
+    // which every pixel had stopped (0: they did not)
+    __shared__ unsigned int s_witer[kWarps];
+    __shared__ int s_satpos;
+    __shared__ int s_prefix_all;   // the first round's lists are the full ones
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    if (tid == 0) {
+        mbar_init(&s_bar[0], 1);
+        mbar_init(&s_bar[1], 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        const int64_t n_vis = (int64_t)a.counters[kCntVisible];
+        s_prefix_all = prefix_records(n_vis, a.prefix) == n_vis;
+    }
+    for (int t = tid; t < kWarps * BATCH / 4; t += kBlendThreads) reinterpret_cast<uint32_t*>(&s_wb[0][0])[t] = 0u;
+    __syncthreads();
+    uint32_t par0 = 0u, par1 = 0u;
+    const int lx = TS::lx(tid), ly = TS::ly(tid);
+    unsigned long long exam_total = 0, blended_total = 0;
+    unsigned int witer = 0;
+    bool failed = false;
+    uint16_t* L = s_list[w];
+    if (a.round == 2 && a.counters[kCntOpenTiles] == 0ull) return;
+
+    for (;;) {
+        if (tid == 0) s_item = atomicAdd(a.work, 1u);
+        __syncthreads();
+        const unsigned int item = s_item;
+        __syncthreads();
+        if ((int64_t)item >= Tb.n_tiles || failed) break;
+        if (a.round == 2 && !((a.open_tiles[item >> 5] >> (item & 31u)) & 1u)) continue;
+        if (lane == 0) s_witer[w] = 0u;
+        if (tid == 0) s_satpos = 0;
+        const int view = find_view_of_tile(Tb, item);
+        const DevView& V = Tb.v[view];
+        const int lt = (int)(item - V.tile_base);
+        const int tx0 = (lt % V.TX) * BX, ty0 = (lt / V.TX) * BY;
+        const int px = tx0 + lx, py = ty0 + ly;
+        const bool inside = px < V.W && py < V.H;
+        const uint2 rg = a.ranges[item];
+        const int n = (int)(rg.y - rg.x);
+        const int nb = (n + BATCH - 1) / BATCH;
+        const float pxf = __fadd_rn((float)px, 0.5f), pyf = __fadd_rn((float)py, 0.5f);
+        float T = 1.0f, C0 = 0.0f, C1 = 0.0f, C2 = 0.0f, D = 0.0f;
+        uint32_t last = 0, exam = (uint32_t)n, nblend = 0;
+        bool done = !inside;
+
+        if (nb > 0) issue_batch<4>(a.vals, a.rec, rg.x, min(BATCH, n), s_buf, &s_bar[0], nullptr);
+        for (int b = 0; b < nb; ++b) {
+            const int s = b & 1;
+            if (b + 1 < nb)
+                issue_batch<4>(a.vals, a.rec, rg.x + (b + 1) * BATCH, min(BATCH, n - (b + 1) * BATCH),
+                            s_buf + (size_t)(s ^ 1) * BATCH * 4, &s_bar[s ^ 1], nullptr);
+            const bool ok = mbar_wait_bounded(&s_bar[s], s ? par1 : par0, a.status, a.wait_ns);
+            if (s) par1 ^= 1u; else par0 ^= 1u;
+            if (__syncthreads_or(!ok)) {
+                failed = true;
+                if (b + 1 < nb) mbar_wait_bounded(&s_bar[s ^ 1], s ? par0 : par1, a.status, a.wait_ns);
+                break;
+            }
+            const int cnt = min(BATCH, n - b * BATCH);
+            const float4* B = s_buf + (size_t)s * BATCH * 4;
+            warp_masks<BX, BY>(B, cnt, tx0, ty0, s_mask);
+            __syncthreads();
+            const int nl = warp_list(s_mask, cnt, w, lane, L);
+            // Structured body and a warp vote per entry: the vote reconverges
+            // the warp every iteration (lanes would otherwise drift apart under
+            // independent thread scheduling) and ends the batch for the warp
+            // once all of its pixels are done.
+            if (!__all_sync(0xffffffffu, done)) {
+                // Branch-free: after exact culling nearly every walked entry
+                // composites somewhere in the warp, so every lane evaluates it
+                // and the decisions select the updates (a zero weight leaves C
+                // and D bit-identical).  Entries are taken two at a time: the
+                // second's alpha does not depend on T, so it overlaps the
+                // first's update; the warp vote that ends the walk once every
+                // pixel has stopped is taken after every second pair (a done
+                // pixel passes nothing, so the extra entries change no result).
+                // Returns whether this pixel composited the entry.
+                auto step = [&](const TilePair& e) {
+                    const float Tn = __fmul_rn(T, __fsub_rn(1.0f, e.al));
+                    const bool pass = !done && e.P2 <= 0.0f && e.al >= GSR_ALPHA_MIN;
+                    const bool stop = pass && Tn < GSR_T_STOP;
+                    const bool blended_now = pass && !stop;
+                    const float wgt = blended_now ? e.al * T : 0.0f;
+                    C0 = fmaf(e.c.x, wgt, C0);
+                    C1 = fmaf(e.c.y, wgt, C1);
+                    C2 = fmaf(e.c.z, wgt, C2);
+                    D = fmaf(e.c.w, wgt, D);
+                    T = blended_now ? Tn : T;
+                    if constexpr (COUNT) {
+                        exam = stop ? (uint32_t)(b * BATCH + e.k + 1) : exam;
+                        nblend += blended_now ? 1u : 0u;
+                    }
+                    done = done || stop;
+                    return blended_now;
+                };
+                // Bit p of a lane's wb is its own decision for the p-th entry of
+                // a group of 32.  Per group: the pixel's last composited entry
+                // is the highest set bit, and one OR over the warp publishes
+                // which entries some pixel of the warp composited (entry
+                // L[i0 + l] by lane l).
+                auto publish = [&](uint32_t wb, int i0, int cnt) {
+                    if (wb) last = (uint32_t)(b * BATCH + L[i0 + 31 - __clz(wb)] + 1);
+                    const uint32_t any = __reduce_or_sync(0xffffffffu, wb);
+                    if (lane < cnt && ((any >> lane) & 1u)) s_wb[w][L[i0 + lane]] = 1;
+                };
+                int i = 0;
+                bool all = false;
+                // whole groups of 32 entries, bit positions fixed at compile time
+                for (; i + 32 <= nl; i += 32) {
+                    uint32_t wb = 0;
+                    int p = 0;
+#pragma unroll
+                    for (; p < 32; p += 2) {
+                        const TilePair e0 = tile_pair(B, L[i + p], pxf, pyf);
+                        const TilePair e1 = tile_pair(B, L[i + p + 1], pxf, pyf);
+                        if (step(e0)) wb |= 1u << p;
+                        if (step(e1)) wb |= 2u << p;
+                        if ((p & 2) && __all_sync(0xffffffffu, done)) { p += 2; all = true; break; }
+                    }
+                    publish(wb, i, p);
+                    if (all) { i += p; break; }
+                }
+                if (!all) {
+                    // the last (fewer than 32) entries
+                    uint32_t wb = 0;
+                    int p = 0;
+                    for (; i + p + 1 < nl; p += 2) {
+                        const TilePair e0 = tile_pair(B, L[i + p], pxf, pyf);
+                        const TilePair e1 = tile_pair(B, L[i + p + 1], pxf, pyf);
+                        if (step(e0)) wb |= 1u << p;
+                        if (step(e1)) wb |= 2u << p;
+                        if (__all_sync(0xffffffffu, done)) { p += 2; all = true; break; }
+                    }
+                    if (!all && i + p < nl) {
+                        if (step(tile_pair(B, L[i + p], pxf, pyf))) wb |= 1u << p;
+                        ++p;
+                    }
+                    publish(wb, i, p);
+                    i += p;
+                }
+                if (lane == 0) s_witer[w] += (unsigned)i;
+            }
+            const bool all_done = __syncthreads_and(done);
+            // publish which warps composited each entry (the backward walks only
+            // those): a warp writes the eight mask words of 32 entries
+            for (int c = w; c * kChunk < cnt; c += kWarps) {
+                const int t = c * kChunk + lane;
+                uint32_t mine = 0u;
+#pragma unroll
+                for (int ww = 0; ww < kWarps; ++ww) {
+                    const uint32_t any = __ballot_sync(0xffffffffu, s_wb[ww][t] != 0);
+                    if (lane == mask_word<TS::WPR>(ww)) mine = any;
+                    s_wb[ww][t] = 0;
+                }
+                if (a.wmask && lane < kMaskWords)
+                    a.wmask[mask_base(rg.x, s_item, a.region2, Tb.n_tiles) +
+                            (size_t)(b * (BATCH / kChunk) + c) * kMaskWords + lane] = mine;
+            }
+            if (all_done) {
+                if (tid == 0) s_satpos = b * BATCH + cnt;
+                // drain the prefetched batch before leaving the tile
+                if (b + 1 < nb) {
+                    const bool ok2 = mbar_wait_bounded(&s_bar[s ^ 1], s ? par0 : par1, a.status, a.wait_ns);
+                    if (s) par0 ^= 1u; else par1 ^= 1u;
+                    if (__syncthreads_or(!ok2)) failed = true;
+                }
+                break;
+            }
+        }
+        // A first round's tile is final when its pixels all stopped within
+        // the prefix lists (or those were the full lists); otherwise the
+        // second round renders it again over its full list.
+        const bool saturated = __syncthreads_and(done);   // (also publishes s_witer and s_satpos)
+        const bool final_tile = a.round != 1 || saturated || s_prefix_all;
+        // (thread 0 re-reads the tile and its range: nothing of them stays
+        // live in registers across the walk)
+        if (!final_tile) {
+            if (tid == 0 && !failed) {
+                const unsigned int it = s_item;
+                atomicOr(a.open_tiles + (it >> 5), 1u << (it & 31u));
+                atomicAdd(a.counters + kCntOpenTiles, 1ull);
+            }
+            continue;
+        }
+        if (lane == 0) witer += s_witer[w];
+        if (tid == 0 && a.hist && !failed) {
+            // the share of the depth-ordered records the tile needed before
+            // every pixel stopped, weighted by its (estimated full) list length
+            const uint2 r = a.ranges[s_item];
+            const unsigned long long n_vis = a.counters[kCntVisible];
+            int bucket = kSatBuckets;
+            if (saturated && s_satpos > 0 && n_vis > 0ull) {
+                const uint32_t k = a.vals[r.x + s_satpos - 1];
+                bucket = sat_bucket((float)(a.depthpos[k] + 1u) / (float)n_vis);
+            }
+            unsigned long long len = r.y - r.x;
+            if (a.round == 1) {
+                const unsigned long long n_pre = (unsigned long long)prefix_records((int64_t)n_vis, a.prefix);
+                if (n_pre > 0ull) len = len * n_vis / n_pre;
+            }
+            if (len) atomicAdd(a.hist + bucket, len);
+        }
+        if (inside) {
+            const int64_t hw = (int64_t)V.W * V.H;
+            const int64_t off = (int64_t)py * V.W + px;
+            const int64_t pix = V.pix_base + off;
+            float* rgb = a.rgb + 3 * V.pix_base;
+            rgb[off] = C0 + T * Tb.bg[0];
+            rgb[hw + off] = C1 + T * Tb.bg[1];
+            rgb[2 * hw + off] = C2 + T * Tb.bg[2];
+            a.depth[pix] = D;
+            a.alpha[pix] = 1.0f - T;
+            a.tfinal[pix] = T;
+            a.ncontrib[pix] = last;
+            if constexpr (COUNT) {
+                exam_total += exam;
+                blended_total += nblend;
+            }
+        }
+    }
+    exam_total = warp_sum(exam_total);
+    blended_total = warp_sum(blended_total);
+    if (lane == 0 && exam_total) atomicAdd(a.counters + kCntFwdPairs, exam_total);
+    if (lane == 0 && blended_total) atomicAdd(a.counters + kCntBlended, blended_total);
+    if (lane == 0 && witer) atomicAdd(a.counters + kCntWarpFwd, (unsigned long long)witer);
+}
+
+// ---- warp form
 // One warp renders one 8x8 pixel block of a tile, two horizontally adjacent
 // pixels per lane, and nothing in it waits for another warp.  The tile's list
 // is walked in chunks of 32 entries.  Per chunk: the records (64 bytes each)
@@ -106,11 +481,8 @@ __device__ __forceinline__ float rect_max_form(float x0, float x1, float y0, flo
 // pair counters) 9.8 -> 7.35 ms, 60-view road 29.1 -> 21.6 ms.  Packed pairs
 // (fma.rn.f32x2 over the two pixels) take the issue slots of the two scalar
 // operations on this part and need their operands twice: 1.69 ms on the rig.
-constexpr int kFwdWarps = 4;            // warps per block (they share nothing)
+constexpr int kFwdWarps = 4;            // warps per block (they share a tile, see next_block)
 constexpr int kFwdThreads = 32 * kFwdWarps;
-constexpr int kChunk = 32;              // list entries per step: one per lane
-constexpr int kBlk = 8;                 // the pixel block's side
-constexpr int kBlocksPerTile = kBlendThreads / (kBlk * kBlk);
 
 // A surviving record as the walk reads it.
 struct DenseRec {
@@ -220,26 +592,14 @@ __device__ __forceinline__ uint2 next_block(unsigned long long* shared, uint2* o
     }
 }
 
-// First 32-bit word of a tile's composited-entry masks: kMaskWords words per
-// chunk of 32 list positions, word 2 blk + h the entries that some pixel of
-// the upper (h = 0) or lower 8x4 half of block blk composited.  A tile's
-// chunks start at its range's first position / 32 plus the tile id (plus the
-// tile count in the second list region), so no two tiles' words overlap:
-// floor((x + n) / 32) - floor(x / 32) + 1 >= ceil(n / 32).
-constexpr int kMaskWords = 2 * kBlocksPerTile;
-__device__ __forceinline__ size_t mask_base(uint32_t first, uint32_t tile, uint32_t region2, int64_t n_tiles)
-{
-    return (size_t)kMaskWords * ((size_t)(first / kChunk) + tile + (first >= region2 ? (size_t)n_tiles : (size_t)0));
-}
-
 // COUNT: keep the per-pixel examined and composited counts (statistics only;
 // a separate instantiation because the running counts lengthen the walk).
 // 80 registers, six blocks per SM (at 72 the walk spills: 6 % slower).
 template <int BX, bool COUNT>
 __global__ void __launch_bounds__(kFwdThreads, 6)
-blend_fwd_kernel(const __grid_constant__ Table Tb, BlendFwdArgs a)
+blend_fwd_warp_kernel(const __grid_constant__ Table Tb, BlendFwdArgs a)
 {
-    if (earlier_wait_timed_out(a.status)) return;
+    if (earlier_wait_timed_out(a.status) || !warp_form(a)) return;
     constexpr int BY = kBlendThreads / BX, BPR = BX / kBlk;   // blocks per tile row
     __shared__ __align__(128) FwdSmem s_warp[kFwdWarps];
     __shared__ unsigned long long s_queue;
@@ -729,7 +1089,7 @@ blend_bwd_kernel(const __grid_constant__ Table Tb, BlendBwdArgs a)
         if (lane == 0 && warp_last) atomicMax(&s_maxlast, (uint32_t)warp_last);
         // this warp's 8x4 block: half (w / WPR) & 1 of the forward's 8x8 block
         const uint32_t* words = a.wmask + mask_base(rg.x, item, a.region2, Tb.n_tiles) +
-                                2 * ((w / TS::WPR / 2) * TS::WPR + w % TS::WPR) + ((w / TS::WPR) & 1);
+                                mask_word<TS::WPR>(w);
         __syncthreads();
         const int maxlast = (int)s_maxlast;
         const int nb = (maxlast + BATCH - 1) / BATCH;
@@ -872,30 +1232,58 @@ blend_bwd_kernel(const __grid_constant__ Table Tb, BlendBwdArgs a)
 // ---------------------------------------------------------------------------
 // dispatch
 // ---------------------------------------------------------------------------
-template <int BX, bool COUNT>
-static void fwd_launch(const Table& T, const BlendFwdArgs& a, int num_sms, cudaStream_t s)
+template <int BX, int BY, int BATCH, bool COUNT>
+static void fwd_tile_launch(const Table& T, const BlendFwdArgs& a, int num_sms, cudaStream_t s)
 {
-    auto kern = blend_fwd_kernel<BX, COUNT>;
+    auto kern = blend_fwd_tile_kernel<BX, BY, BATCH, COUNT>;
+    const size_t smem = (size_t)2 * BATCH * kRecordBytes;
     // function attributes and occupancy are per device
     static std::atomic<int> per_sm_dev[kMaxDevices];
     const int per_sm = per_device_once(per_sm_dev, [&] {
         int n = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kFwdThreads, 0);
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kBlendThreads, smem);
         return n < 1 ? 1 : n;
     });
     int64_t grid = (int64_t)num_sms * per_sm;
-    const int64_t want = (T.n_tiles * kBlocksPerTile + kFwdWarps - 1) / kFwdWarps;
-    if (grid > want) grid = want;
+    if (grid > T.n_tiles) grid = T.n_tiles;
     if (grid < 1) return;
     GSR_COUNT_LAUNCH();
-    kern<<<(unsigned)grid, kFwdThreads, 0, s>>>(T, a);
+    kern<<<(unsigned)grid, kBlendThreads, smem, s>>>(T, a);
+}
+
+template <int BX, int BY, int BATCH>
+static void fwd_tile_one(const Table& T, const BlendFwdArgs& a, int num_sms, cudaStream_t s)
+{
+    if (a.count_pairs) fwd_tile_launch<BX, BY, BATCH, true>(T, a, num_sms, s);
+    else fwd_tile_launch<BX, BY, BATCH, false>(T, a, num_sms, s);
+}
+
+// Blocks of the warp form resident on the device.
+template <int BX, bool COUNT>
+static int fwd_warp_resident(int num_sms)
+{
+    static std::atomic<int> per_sm_dev[kMaxDevices];
+    return num_sms * per_device_once(per_sm_dev, [&] {
+        int n = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, blend_fwd_warp_kernel<BX, COUNT>, kFwdThreads, 0);
+        return n < 1 ? 1 : n;
+    });
+}
+
+template <int BX, bool COUNT>
+static void fwd_warp_launch(const Table& T, const BlendFwdArgs& a, int num_sms, cudaStream_t s)
+{
+    const int64_t grid = std::min<int64_t>(fwd_warp_resident<BX, COUNT>(num_sms), T.n_tiles);
+    GSR_COUNT_LAUNCH();
+    blend_fwd_warp_kernel<BX, COUNT><<<(unsigned)grid, kFwdThreads, 0, s>>>(T, a);
 }
 
 template <int BX>
-static void fwd_one(const Table& T, const BlendFwdArgs& a, int num_sms, cudaStream_t s)
+static void fwd_warp_one(const Table& T, const BlendFwdArgs& a, int num_sms, cudaStream_t s)
 {
-    if (a.count_pairs) fwd_launch<BX, true>(T, a, num_sms, s);
-    else fwd_launch<BX, false>(T, a, num_sms, s);
+    if (a.count_pairs) fwd_warp_launch<BX, true>(T, a, num_sms, s);
+    else fwd_warp_launch<BX, false>(T, a, num_sms, s);
 }
 
 template <int BX, int BY, int BATCH>
@@ -947,12 +1335,26 @@ bool blend_supported(int tw, int th, int batch)
         }                                                                                        \
     } while (0)
 
-// (the forward stages chunks of 32 entries per warp whatever the staging batch)
-void launch_blend_fwd(const Table& T, const BlendFwdArgs& a, int num_sms, cudaStream_t s)
+int blend_fwd_list_parts(const Table& T, bool count_pairs, int num_sms)
 {
-    if (T.tile_w == 16) fwd_one<16>(T, a, num_sms, s);
-    else if (T.tile_w == 32) fwd_one<32>(T, a, num_sms, s);
-    else fwd_one<8>(T, a, num_sms, s);
+    if (T.n_tiles < kWarpFormMinTiles) return 0;
+    const int resident = T.tile_w == 16 ? (count_pairs ? fwd_warp_resident<16, true>(num_sms) : fwd_warp_resident<16, false>(num_sms))
+                       : T.tile_w == 32 ? (count_pairs ? fwd_warp_resident<32, true>(num_sms) : fwd_warp_resident<32, false>(num_sms))
+                                        : (count_pairs ? fwd_warp_resident<8, true>(num_sms) : fwd_warp_resident<8, false>(num_sms));
+    return (int)(kWarpFormShare * resident);
+}
+
+// Both forms are launched where the warp form may be taken; the lists decide on
+// the device which of the two returns at once (a second round of two takes the
+// first one's form).
+void launch_blend_fwd(const Table& T, int batch, const BlendFwdArgs& a, int num_sms, cudaStream_t s)
+{
+    if (a.long_list) {
+        if (T.tile_w == 16) fwd_warp_one<16>(T, a, num_sms, s);
+        else if (T.tile_w == 32) fwd_warp_one<32>(T, a, num_sms, s);
+        else fwd_warp_one<8>(T, a, num_sms, s);
+    }
+    GSR_DISPATCH(fwd_tile_one, T, batch, a, num_sms, s);
 }
 
 size_t blend_mask_bytes(int64_t list_span, int64_t n_tiles)

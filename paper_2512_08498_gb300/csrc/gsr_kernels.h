@@ -47,6 +47,7 @@ enum : int {
     kCntRuns = 10,       // runs of the list round by tile rows (0 after an overflow)
     kCntRuns2 = 11,      // the same for the second round
     kCntChunks = 12,     // their chunks (u32) and the placement's ticket (u32)
+    kCntLongList = 13,   // the forward's first (or only) round has a list too long for the warp form
     kCntSlots = 16,
 };
 
@@ -202,11 +203,20 @@ struct DuplicateArgs {
     unsigned long long* n_rows = nullptr;   // runs written (0 after an overflow)
 };
 
+// Whether one of a round's lists has more than 1 / parts of its instances.
+struct LongList {
+    unsigned long long* flag = nullptr;   // zeroed; set to one if so (nullptr: not asked)
+    int parts = 1;
+    __host__ __device__ int64_t far(int64_t instances) const { return instances / parts + 1; }
+};
+
 // Tile lists from depth-ordered runs sorted by tile row (see gsr_sort.cu).
 constexpr int kRowListMaxTiles = 1024;      // tile columns of a view (4 bytes of row_count's shared memory per warp)
 constexpr int64_t kRowChunksMin = 8192;     // chunks wanted of small run counts
 struct RowListArgs {
     const unsigned long long* n_rows;
+    const unsigned long long* inst_count;
+    LongList lists;
     const uint32_t* order;         // [n_rows] run index in sorted order
     const uint2* runs;             // [row_cap] by run index
     uint2* sorted;                 // [row_cap] scratch: the runs in sorted order
@@ -238,7 +248,7 @@ int64_t duplicate_windows(int64_t inst_cap);   // win_cap for inst_cap kept inst
 // A key outside [0, n_tiles) sets kErrInternal and is skipped.  Positions
 // are written as offset + index (the list region's start).
 void launch_ranges(const uint32_t* sorted_tile_keys, const unsigned long long* m_dev, int64_t cap, uint2* ranges,
-                   int64_t n_tiles, int64_t offset, uint32_t* status, int num_sms, cudaStream_t s);
+                   int64_t n_tiles, int64_t offset, uint32_t* status, LongList L, int num_sms, cudaStream_t s);
 
 // ---- blend ----------------------------------------------------------------
 struct BlendFwdArgs {
@@ -252,10 +262,12 @@ struct BlendFwdArgs {
     uint32_t* ncontrib;
     uint32_t* wmask;               // blend_mask_bytes: which 8x4 blocks composited each list entry (may be nullptr)
     uint32_t region2 = 0xffffffffu;    // first list position of the second region (0xffffffff: one region)
-    unsigned int* work;            // zeroed block counter
+    unsigned int* work;            // zeroed tile counter
     uint32_t* status;
     unsigned long long* counters;
+    uint64_t wait_ns = kWaitLimitNs;   // limit of each mbarrier wait
     bool count_pairs = true;       // examined and composited pair counters
+    const unsigned long long* long_list = nullptr;   // LongList::flag of the lists: the warp form may be taken
     // Two-round lists.  round: 0 for a forward of one round; 1 for the
     // first of two, which renders the prefix lists (the first
     // prefix_records(n, prefix) records), finishes the tiles whose pixels
@@ -291,7 +303,8 @@ struct BlendBwdArgs {
 };
 
 bool blend_supported(int tile_w, int tile_h, int batch);
-void launch_blend_fwd(const Table& T, const BlendFwdArgs& a, int num_sms, cudaStream_t s);
+void launch_blend_fwd(const Table& T, int batch, const BlendFwdArgs& a, int num_sms, cudaStream_t s);
+int blend_fwd_list_parts(const Table& T, bool count_pairs, int num_sms);   // LongList::parts (0: no warp form)
 size_t blend_mask_bytes(int64_t list_span, int64_t n_tiles);   // composited-entry masks of a forward's lists
 void launch_blend_bwd(const Table& T, int batch, const BlendBwdArgs& a, int num_sms, cudaStream_t s);
 

@@ -712,6 +712,7 @@ row_scan_kernel(const __grid_constant__ Table Tb, RowListArgs a)
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t nc = *a.n_chunks;
     const int ch = row_chunk((int64_t)*a.n_rows);
+    const int64_t far = a.lists.flag ? a.lists.far((int64_t)*a.inst_count) : 0;
     for (int64_t r = blockIdx.x; r < a.n_trows; r += gridDim.x) {
         const TileRow tr = tile_row(s_vt, Tb, (uint32_t)r);
         const uint2 g = a.row_range[r];
@@ -755,7 +756,10 @@ row_scan_kernel(const __grid_constant__ Table Tb, RowListArgs a)
                 const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
                 if (lane >= o) incl += t;
             }
-            if (w == 0 && in) a.tile_first[tr.first_tile + x] = make_uint2(carry + incl - total, total);
+            if (w == 0 && in) {
+                a.tile_first[tr.first_tile + x] = make_uint2(carry + incl - total, total);
+                if (a.lists.flag && (int64_t)total > far) *a.lists.flag = 1ull;
+            }
             carry += __shfl_sync(0xffffffffu, incl, 31);
             __syncthreads();   // the sums are rewritten by the next columns
         }
@@ -959,12 +963,17 @@ void launch_row_lists(const Table& T, const RowListArgs& a, int num_sms, cudaStr
 }
 
 // Four keys per thread (one 16-byte load, the keys array starts 16-byte
-// aligned) plus the neighbour on each side.
+// aligned) plus the neighbour on each side.  With L.flag, also whether some list
+// is longer than `far` entries: then equal keys lie that far apart.  (Every 32nd
+// key is compared where that is near enough: the lists are flagged from far + 32
+// entries on at the latest.)
 __global__ void ranges_kernel(const uint32_t* __restrict__ keys, const unsigned long long* m_dev, int64_t cap,
-                              uint2* __restrict__ ranges, int64_t n_tiles, int64_t offset, uint32_t* status)
+                              uint2* __restrict__ ranges, int64_t n_tiles, int64_t offset, uint32_t* status, LongList L)
 {
     const int64_t m = clamped_count(m_dev, cap);
     const int64_t nq = (m + 3) / 4;
+    const int64_t far = L.far(m);
+    const int64_t every = far < 256 ? 1 : 8;
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nq; q += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i0 = 4 * q;
         uint32_t k[6];
@@ -977,6 +986,7 @@ __global__ void ranges_kernel(const uint32_t* __restrict__ keys, const unsigned 
         }
         k[0] = i0 > 0 ? keys[i0 - 1] : 0u;
         k[5] = i0 + 4 < m ? keys[i0 + 4] : 0u;
+        if (L.flag && q % every == 0 && i0 + far < m && keys[i0 + far] == k[1]) *L.flag = 1ull;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int64_t i = i0 + u;
@@ -996,13 +1006,13 @@ __global__ void ranges_kernel(const uint32_t* __restrict__ keys, const unsigned 
 }
 
 void launch_ranges(const uint32_t* sorted_tile_keys, const unsigned long long* m_dev, int64_t cap, uint2* ranges,
-                   int64_t n_tiles, int64_t offset, uint32_t* status, int num_sms, cudaStream_t s)
+                   int64_t n_tiles, int64_t offset, uint32_t* status, LongList L, int num_sms, cudaStream_t s)
 {
     if (cap <= 0) return;
     int64_t blocks = (cap / 4 + 255) / 256 + 1;
     if (blocks > (int64_t)num_sms * 8) blocks = (int64_t)num_sms * 8;
     GSR_COUNT_LAUNCH();
-    ranges_kernel<<<(unsigned)blocks, 256, 0, s>>>(sorted_tile_keys, m_dev, cap, ranges, n_tiles, offset, status);
+    ranges_kernel<<<(unsigned)blocks, 256, 0, s>>>(sorted_tile_keys, m_dev, cap, ranges, n_tiles, offset, status, L);
 }
 
 // ---------------------------------------------------------------------------
