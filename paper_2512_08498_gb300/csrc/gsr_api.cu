@@ -567,19 +567,42 @@ static float choose_prefix(const unsigned long long* H, const unsigned long long
     return best_b < kSatBuckets && best <= kTake * one ? (float)sat_edge(best_b) : 1.0f;
 }
 
+// Instances that a state starts with room for.
+static int64_t first_inst_cap(int64_t rec_cap) { return std::max<int64_t>(4 * rec_cap, 1 << 20); }
+
 // Lists by tile rows: the runs of the records' tiles are sorted by tile row and
-// expanded into the lists, instead of expanding and sorting the instances.  It
-// takes the batches of 65536 records and 4096 tiles and more whose views are at
-// most kRowListMaxTiles tiles wide; and not the allocation-free forward.  Fewer
-// records are bound by launches (four more here: 10 us of a 240 us step on 10k
-// records).  Fewer tiles have few instances, and few tile rows that hold all the
-// runs: emission, sort and ranges together, sorted instances against rows, took
-// 0.125 / 0.136 ms at 960 tiles (100k records), 0.185 / 0.238 at 2000 (18 small
-// views), 0.165 / 0.151 at 4600 (210k records).
+// expanded into the lists, instead of expanding and sorting the instances.  That
+// costs five kernels more (40-60 us) and saves about a third of the emission and
+// most of the sort, in proportion to the instances; so it is worth it from some
+// five million instances on.  How many there are is known on the device only.
+// The host takes it where they must be many:
+//   * batches of kRowListRecords records and more in large views (a record's
+//     instances grow with the view's width in tiles);
+//   * states whose lists have outgrown the four instances per record that they
+//     started with room for, to kRowListInstances and more (near Gaussians with
+//     footprints of tens of tiles).
+// Emission, sort and ranges together, sorted instances against rows, ms:
+//   1080p view, 500k near Gaussians, 74 M instances    1.40  0.49
+//   box of 100k, 1600 x 960, 13.6 M                    0.33  0.20
+//   three views of 60k, 32x8 tiles, 7.3 M              0.25  0.21
+//   30-view window, 35 M records, 167 M instances      4.86  3.17
+//   six 1600x900 views, 6 M records, 19 M              0.63  0.57
+//   18 1080p views, 5.4 M records, 8.2 M               0.36  0.36
+//   six 1600x900 views, 1.5 M records, 4.9 M           0.22  0.24   sorted
+//   12 views of 1104x814, 0.1 M records, 0.25 M        0.09  0.14   sorted
+//   24 views of 400x225, 24 M records, 16 M            0.84  1.09   sorted
+//   one 1600x900 view of the road, 260k, 0.6 M         0.10  0.16   sorted
+// Under 65536 records or 4096 tiles a batch is bound by launches, views wider than
+// kRowListMaxTiles do not fit row_count's shared memory, and the allocation-free
+// forward always sorts.
 constexpr int64_t kRowListMinRecords = 65536, kRowListMinTiles = 4096;
-static bool use_row_lists(const Table& T)
+constexpr int64_t kRowListRecords = 5000000, kRowListViewTiles = 4096, kRowListInstances = 5000000;
+static bool use_row_lists(const Table& T, const gsr_saved* s)
 {
-    return T.n_records >= kRowListMinRecords && T.n_tiles >= kRowListMinTiles && row_list_stride(T) <= kRowListMaxTiles;
+    if (T.n_records < kRowListMinRecords || T.n_tiles < kRowListMinTiles || row_list_stride(T) > kRowListMaxTiles)
+        return false;
+    if (T.n_records >= kRowListRecords && T.n_tiles >= kRowListViewTiles * T.n_views) return true;
+    return s->inst_cap >= kRowListInstances && s->inst_cap > first_inst_cap(s->rec_cap);
 }
 
 // Its scratch in gsr_ctx::row_work; returns the bytes.
@@ -623,7 +646,7 @@ static gsr_status size_saved(gsr_ctx* ctx, gsr_saved* s, const Table& T)
         if (cap > (64ll << 20)) cap = std::max<int64_t>(64ll << 20, cap / 3);
         s->rec_cap = std::max<int64_t>(s->rec_cap, std::max<int64_t>(cap, 1));
     }
-    if (s->inst_cap == 0 || grown) s->inst_cap = std::max<int64_t>(s->inst_cap, std::max<int64_t>(4 * s->rec_cap, 1 << 20));
+    if (s->inst_cap == 0 || grown) s->inst_cap = std::max<int64_t>(s->inst_cap, first_inst_cap(s->rec_cap));
     // the emission keeps two counts per record in the tile-sort destination
     // keys while they are free
     s->inst_cap = std::max<int64_t>(s->inst_cap, 2 * s->rec_cap);
@@ -665,7 +688,7 @@ static gsr_status size_saved(gsr_ctx* ctx, gsr_saved* s, const Table& T)
     if ((e = ctx->tmp_vals.ensure((size_t)tmp * 4)) != cudaSuccess) return cuda_fail(ctx, e, "alloc sort scratch");
     if ((e = ctx->hist.ensure((size_t)256 * (ctx->hist_blocks + 1) * 4)) != cudaSuccess) return cuda_fail(ctx, e, "alloc histogram");
     if ((e = ctx->dup_rows.ensure((size_t)s->row_cap * 16)) != cudaSuccess) return cuda_fail(ctx, e, "alloc tile rows");
-    if (use_row_lists(T) &&
+    if (use_row_lists(T, s) &&
         (e = ctx->row_work.ensure(row_lists_layout(T, s->row_cap, nullptr, nullptr))) != cudaSuccess)
         return cuda_fail(ctx, e, "alloc row lists");
     return GSR_OK;
@@ -728,7 +751,7 @@ static void enqueue_forward(gsr_ctx* ctx, gsr_saved* s, const gsr_gaussians* g, 
     // histograms): taken by forwards that synchronise, the only ones whose
     // statistics are read back
     const bool hist = ctx->cfg.list_prefix == 0.0f && !(ctx->cfg.flags & GSR_FLAG_NO_SYNC);
-    const bool by_rows = use_row_lists(T);
+    const bool by_rows = use_row_lists(T, s);
     s->row_lists = by_rows;
     const int bits = tile_bits(by_rows ? row_list_rows(T) : T.n_tiles);
     const int passes = (bits + 7) / 8;
