@@ -203,7 +203,8 @@ struct gsr_saved {
     int64_t lb_pre_words = 0, lb_dup_words = 0;
     DevMem rec, vis_key, sorted_k, vis_aux, kstart, tile_key, tile_val, ranges, tfinal, ncontrib, wmask, ctrl;
     // two-round lists: open-tile bits with the open blocks' behind them, record
-    // depth positions, per-tile statistics scratch
+    // depth positions, per-tile statistics scratch with the first round's ranges
+    // of the open tiles behind it (lists by tile rows only)
     DevMem open_tiles, depthpos, tile_need;
     // Two-round lists.  prefix: the first round's record fraction of the
     // last forward (1: one round); region2: where its second list region
@@ -671,7 +672,7 @@ static gsr_status size_saved(gsr_ctx* ctx, gsr_saved* s, const Table& T)
     if (two) {
         if ((e = s->open_tiles.ensure(4 * (open_words(T.n_tiles) + open_words(4 * T.n_tiles)))) != cudaSuccess)
             return cuda_fail(ctx, e, "alloc open tiles");
-        if ((e = s->tile_need.ensure((size_t)std::max<int64_t>(T.n_tiles, 1) * 8)) != cudaSuccess)
+        if ((e = s->tile_need.ensure((size_t)std::max<int64_t>(T.n_tiles, 1) * 16)) != cudaSuccess)
             return cuda_fail(ctx, e, "alloc tile statistics");
         if ((e = s->depthpos.ensure((size_t)rc * 4)) != cudaSuccess) return cuda_fail(ctx, e, "alloc depth positions");
     }
@@ -849,6 +850,7 @@ static void enqueue_forward(gsr_ctx* ctx, gsr_saved* s, const gsr_gaussians* g, 
             ra.ticket = ra.n_chunks + 1;
             ra.vals = s->tile_val.as<uint32_t>();
             ra.ranges = s->ranges.as<uint2>();
+            ra.first_ranges = second ? s->tile_need.as<uint2>() + T.n_tiles : nullptr;
             ra.open_tiles = da.open_tiles;
             ra.status = status;
             ra.inst_cap = s->inst_cap;
@@ -1522,16 +1524,22 @@ gsr_status gsr_frequency_schedule(gsr_ctx* ctx, int n_frames, const float* x_gt,
     return GSR_OK;
 }
 
+// Lists by tile rows keep no tile keys: written here from the ranges.
+static void export_tile_keys(gsr_saved* s, cudaStream_t cs)
+{
+    if (!s->row_lists) return;
+    const int64_t nt = s->table.n_tiles;
+    const bool two = s->region2 >= 0;
+    cudaMemsetAsync(s->tile_key.p, 0, s->tile_key.bytes, cs);
+    launch_tile_keys(s->ranges.as<uint2>(), two ? s->tile_need.as<uint2>() + nt : nullptr,
+                     two ? s->open_tiles.as<uint32_t>() : nullptr, nt, s->tile_key.as<uint32_t>(), cs);
+}
+
 gsr_status gsr_debug_lists(gsr_saved* s, uint64_t* keys, uint32_t* vals, uint32_t* ranges, void* stream)
 {
     if (!s || !s->filled) return GSR_ERR_INVALID_ARG;
     s->reusable = false;   // its buffers are read on any stream
-    if (s->row_lists && keys) {
-        // lists by tile rows keep no tile keys: written here from the ranges
-        cudaMemsetAsync(s->tile_key.p, 0, s->tile_key.bytes, static_cast<cudaStream_t>(stream));
-        launch_tile_keys(s->ranges.as<uint2>(), s->table.n_tiles, s->tile_key.as<uint32_t>(),
-                         static_cast<cudaStream_t>(stream));
-    }
+    if (keys) export_tile_keys(s, static_cast<cudaStream_t>(stream));
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     DebugArgs a{};
     a.tile_key = s->tile_key.as<uint32_t>();
@@ -1555,12 +1563,7 @@ gsr_status gsr_debug_list_slice(gsr_saved* s, int64_t first, int64_t count, uint
 {
     if (!s || !s->filled || first < 0 || count < 0) return GSR_ERR_INVALID_ARG;
     s->reusable = false;   // its buffers are read on any stream
-    if (s->row_lists && keys) {
-        // lists by tile rows keep no tile keys: written here from the ranges
-        cudaMemsetAsync(s->tile_key.p, 0, s->tile_key.bytes, static_cast<cudaStream_t>(stream));
-        launch_tile_keys(s->ranges.as<uint2>(), s->table.n_tiles, s->tile_key.as<uint32_t>(),
-                         static_cast<cudaStream_t>(stream));
-    }
+    if (keys) export_tile_keys(s, static_cast<cudaStream_t>(stream));
     DebugArgs a{};
     a.tile_key = s->tile_key.as<uint32_t>();
     a.tile_val = s->tile_val.as<uint32_t>();

@@ -230,6 +230,7 @@ struct RowListArgs {
     uint32_t* ticket;              // set to zero by the plan
     uint32_t* vals;                // list positions from 0: the region's start is in base
     uint2* ranges;
+    uint2* first_ranges;           // a second round keeps the ranges it replaces here (nullptr: not)
     const uint32_t* open_tiles;    // a second round lists these only
     uint32_t* status;
     int64_t n_trows, chunk_cap, inst_cap;
@@ -240,7 +241,8 @@ int row_list_stride(const Table& T);
 int64_t row_list_rows(const Table& T);
 int64_t row_list_chunks(const Table& T, int64_t row_cap);
 void launch_row_lists(const Table& T, const RowListArgs& a, int num_sms, cudaStream_t s);
-void launch_tile_keys(const uint2* ranges, int64_t n_tiles, uint32_t* keys, cudaStream_t s);
+void launch_tile_keys(const uint2* ranges, const uint2* first_ranges, const uint32_t* open_tiles, int64_t n_tiles,
+                      uint32_t* keys, cudaStream_t s);
 void launch_duplicate(const Table& T, const DuplicateArgs& a, int num_sms, cudaStream_t s);
 int64_t duplicate_blocks(int64_t rec_cap);     // look-back words of the scan
 int64_t duplicate_windows(int64_t inst_cap);   // win_cap for inst_cap kept instances

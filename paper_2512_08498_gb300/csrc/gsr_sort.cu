@@ -863,7 +863,11 @@ row_place_kernel(const __grid_constant__ Table Tb, RowListArgs a)
             const uint2 t = a.tile_first[tr.first_tile + x];
             const uint32_t at = a.row_first[r] + t.x;
             first = at + a.chunk_count[(size_t)c * a.stride + x];
-            if (c == a.chunk_first[r] && t.y) a.ranges[tr.first_tile + x] = make_uint2(at, at + t.y);
+            if (c == a.chunk_first[r] && t.y) {
+                uint2* range = a.ranges + tr.first_tile + x;
+                if (a.first_ranges) a.first_ranges[tr.first_tile + x] = *range;
+                *range = make_uint2(at, at + t.y);
+            }
             listed = tile_open(a.open_tiles, tr.first_tile + (uint32_t)x);
         }
         uint32_t p = first, done = first;   // entries appended and written up to here
@@ -912,19 +916,27 @@ row_place_kernel(const __grid_constant__ Table Tb, RowListArgs a)
     }
 }
 
-// Positions of each tile's range get the tile's id (for the parity exports).
-__global__ void tile_keys_kernel(const uint2* __restrict__ ranges, int64_t n_tiles, uint32_t* __restrict__ keys)
+// Positions of each tile's range get the tile's id (for the parity exports); with
+// first_ranges (a forward of two rounds) also those of an open tile's first range,
+// which the second round's has replaced unless the tile's lists are empty.
+__global__ void tile_keys_kernel(const uint2* __restrict__ ranges, const uint2* __restrict__ first_ranges,
+                                 const uint32_t* __restrict__ open_tiles, int64_t n_tiles, uint32_t* __restrict__ keys)
 {
     for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
         const uint2 g = ranges[t];
         for (uint32_t i = g.x + threadIdx.x; i < g.y; i += blockDim.x) keys[i] = (uint32_t)t;
+        if (!first_ranges || g.y <= g.x || !((open_tiles[t >> 5] >> (t & 31)) & 1u)) continue;
+        const uint2 f = first_ranges[t];
+        for (uint32_t i = f.x + threadIdx.x; i < f.y; i += blockDim.x) keys[i] = (uint32_t)t;
     }
 }
 
-void launch_tile_keys(const uint2* ranges, int64_t n_tiles, uint32_t* keys, cudaStream_t s)
+void launch_tile_keys(const uint2* ranges, const uint2* first_ranges, const uint32_t* open_tiles, int64_t n_tiles,
+                      uint32_t* keys, cudaStream_t s)
 {
     GSR_COUNT_LAUNCH();
-    tile_keys_kernel<<<(unsigned)std::min<int64_t>(std::max<int64_t>(n_tiles, 1), 65535), 128, 0, s>>>(ranges, n_tiles, keys);
+    tile_keys_kernel<<<(unsigned)std::min<int64_t>(std::max<int64_t>(n_tiles, 1), 65535), 128, 0, s>>>(
+        ranges, first_ranges, open_tiles, n_tiles, keys);
 }
 
 int row_list_stride(const Table& T)

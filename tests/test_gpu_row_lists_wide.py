@@ -90,3 +90,16 @@ def test_large_records_against_sorted_instances(tile, prefix):
         for a, b in zip(g["ranges"][:: max(1, len(g["ranges"]) // 400)], s["ranges"][:: max(1, len(g["ranges"]) // 400)]):
             assert np.array_equal(g[k][a[0]:a[1]], s[k][b[0]:b[1]]), k
     assert np.array_equal(g["ranges"][:, 1] - g["ranges"][:, 0], s["ranges"][:, 1] - s["ranges"][:, 0])
+
+
+@pytest.mark.parametrize("prefix", [0.05, 0.5])
+def test_first_region_of_two_rounds_is_exported_whole(prefix):
+    # the first round's lists of the tiles that the second one listed again
+    # keep their tile ids
+    sc = _scene((16, 16), (-4.5, -1.3))
+    g, _ = _run(sc, True, prefix)
+    s, _ = _run(sc, False, prefix)
+    assert s["info"]["open_tiles"] > 0
+    m = s["info"]["n_instances"] - s["info"]["n_instances_second"]
+    assert 0 < m and np.array_equal(g["vals"][:m], s["vals"][:m])
+    assert np.array_equal(g["keys"][:m], s["keys"][:m])
