@@ -975,12 +975,21 @@ gsr_status gsr_forward(gsr_ctx* ctx, const gsr_gaussians* g, const gsr_view* vie
     s->filled = false;
     s->have_grads = false;
     // a recycled state's earlier work comes first (a capture cannot wait for an
-    // event from outside it: the host waits)
+    // event from outside it: the host waits, which a capture in the global or the
+    // thread-local mode permits only to a thread that has set itself to relaxed)
     if (s->grown && s->pending) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         cudaError_t e = cudaStreamIsCapturing(cs, &cap);
-        if (e == cudaSuccess)
-            e = cap == cudaStreamCaptureStatusNone ? cudaStreamWaitEvent(cs, s->done, 0) : cudaEventSynchronize(s->done);
+        if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+            e = cudaStreamWaitEvent(cs, s->done, 0);
+        } else if (e == cudaSuccess) {
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            if ((e = cudaThreadExchangeStreamCaptureMode(&mode)) == cudaSuccess) {
+                e = cudaEventSynchronize(s->done);
+                const cudaError_t back = cudaThreadExchangeStreamCaptureMode(&mode);
+                if (e == cudaSuccess) e = back;
+            }
+        }
         if (e != cudaSuccess) return cuda_fail(ctx, e, "recycled state");
         s->pending = false;
     }
