@@ -639,22 +639,22 @@ static size_t open_words(int64_t n) { return (size_t)((std::max<int64_t>(n, 1) +
 static gsr_status size_saved(gsr_ctx* ctx, gsr_saved* s, const Table& T)
 {
     cudaError_t e;
-    // (a recycled state has at least the capacities a new one starts with)
+    // What a new state starts with; a recycled one has at least that, whatever it
+    // grew to for earlier batches.
+    int64_t rec0 = T.n_records;
+    if (rec0 > (64ll << 20)) rec0 = std::max<int64_t>(64ll << 20, rec0 / 3);
+    rec0 = std::max<int64_t>(rec0, 1);
     const bool grown = s->grown;
     s->grown = false;
-    if (s->rec_cap == 0 || grown) {
-        int64_t cap = T.n_records;
-        if (cap > (64ll << 20)) cap = std::max<int64_t>(64ll << 20, cap / 3);
-        s->rec_cap = std::max<int64_t>(s->rec_cap, std::max<int64_t>(cap, 1));
-    }
-    if (s->inst_cap == 0 || grown) s->inst_cap = std::max<int64_t>(s->inst_cap, first_inst_cap(s->rec_cap));
+    if (s->rec_cap == 0 || grown) s->rec_cap = std::max(s->rec_cap, rec0);
+    if (s->inst_cap == 0 || grown) s->inst_cap = std::max(s->inst_cap, first_inst_cap(grown ? rec0 : s->rec_cap));
     // the emission keeps two counts per record in the tile-sort destination
     // keys while they are free
     s->inst_cap = std::max<int64_t>(s->inst_cap, 2 * s->rec_cap);
     // a kept tile row holds >= 1 instance; rows are typically a third of them
     if (s->row_cap == 0 || grown)
-        s->row_cap = std::max<int64_t>(s->row_cap,
-                                       std::max<int64_t>(std::max<int64_t>(s->inst_cap / 2, 2 * s->rec_cap), 1 << 18));
+        s->row_cap = std::max<int64_t>(s->row_cap, std::max<int64_t>((grown ? first_inst_cap(rec0) : s->inst_cap) / 2,
+                                                                     std::max<int64_t>(2 * (grown ? rec0 : s->rec_cap), 1 << 18)));
     // (the runs' keys and order are sorted in list-sized buffers)
     s->inst_cap = std::max<int64_t>(s->inst_cap, s->row_cap);
     const int64_t rc = s->rec_cap, ic = s->inst_cap;
