@@ -224,7 +224,10 @@ GSR_API gsr_status gsr_get_config(const gsr_ctx* ctx, gsr_config* cfg);
 
 /* A saved state holds what one forward leaves for its backward: projected
  * records, the sorted tile lists and ranges, per-pixel final transmittance
- * and contributor counts.  Owned by the caller, tied to its context. */
+ * and contributor counts.  Owned by the caller, tied to its context.  The
+ * context keeps at most two destroyed states, of 2 GB together, whose buffers the
+ * next gsr_saved_create takes over; it frees them when one of its own device
+ * allocations fails and in gsr_destroy. */
 GSR_API gsr_status gsr_saved_create(gsr_ctx* ctx, gsr_saved** out);
 GSR_API void gsr_saved_destroy(gsr_saved* saved);
 GSR_API gsr_status gsr_saved_get_info(const gsr_saved* saved, gsr_saved_info* info);

@@ -93,7 +93,7 @@ struct ProfRecord {
 // allocation and release cost a forward that makes its own state (one per call
 // of the autograd function) 0.9 ms of the 1.2 ms of a 256 x 256 step.  At most
 // kPoolStates states of kPoolBytes together are kept; they go when the context
-// is destroyed or a device allocation fails.  Shared by the context and its
+// is destroyed or one of its device allocations fails.  Shared by the context and its
 // states, with a lock: a state may be destroyed from another host thread
 // (the autograd engine's) or after its context.
 struct SavedPool {
@@ -259,6 +259,16 @@ void SavedPool::drain(bool close)
         closed = closed || close;
     }
     for (gsr_saved* s : v) delete s;
+}
+
+// Sizes one of the context's buffers; the kept states go first if it does not fit.
+static cudaError_t ensure(gsr_ctx* ctx, DevMem& m, size_t bytes)
+{
+    cudaError_t e = m.ensure(bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    (void)cudaGetLastError();
+    ctx->pool->drain(false);
+    return m.ensure(bytes);
 }
 
 static gsr_status fail(gsr_ctx* ctx, gsr_status code, const std::string& msg)
@@ -1095,18 +1105,9 @@ gsr_status gsr_backward(gsr_ctx* ctx, const gsr_gaussians* g, const gsr_view* vi
     if (((uintptr_t)grads->quats & 15u) != 0) return fail(ctx, GSR_ERR_INVALID_ARG, "grad quats must be 16-byte aligned");
     const Table& T = s->table;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
-    auto ensure = [&](DevMem& m, size_t bytes) {
-        cudaError_t e = m.ensure(bytes);
-        if (e == cudaErrorMemoryAllocation) {
-            (void)cudaGetLastError();
-            ctx->pool->drain(false);
-            e = m.ensure(bytes);
-        }
-        return e;
-    };
-    cudaError_t e = ensure(ctx->grad_rec, (size_t)s->rec_cap * kGradFloats * 4);
+    cudaError_t e = ensure(ctx, ctx->grad_rec, (size_t)s->rec_cap * kGradFloats * 4);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "alloc record gradients");
-    if ((e = ensure(ctx->bwd_queue, (size_t)s->rec_cap * 4)) != cudaSuccess)
+    if ((e = ensure(ctx, ctx->bwd_queue, (size_t)s->rec_cap * 4)) != cudaSuccess)
         return cuda_fail(ctx, e, "alloc extended-precision queue");
     const bool reusable = s->reusable;
     s->reusable = false;   // until this call has succeeded
@@ -1266,7 +1267,7 @@ gsr_status gsr_insertion(gsr_ctx* ctx, const gsr_insert_params* p, const gsr_vie
     insertion_taps((double)p->sigma, &T.r, T.taps);
     // scratch: status word, ticket, look-back words (all start at zero)
     const int64_t words = insertion_lb_words(pix);
-    cudaError_t e = ctx->ins_scratch.ensure(16 + 8 * (size_t)words);
+    cudaError_t e = ensure(ctx, ctx->ins_scratch, 16 + 8 * (size_t)words);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "alloc insertion scratch");
     unsigned char* sc = ctx->ins_scratch.as<unsigned char>();
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
@@ -1361,7 +1362,7 @@ gsr_status gsr_merge(gsr_ctx* ctx, const gsr_merge_params* p, const gsr_view* vi
     const size_t o_map = 0, o_best = o_map + up((size_t)npix * 4), o_cnt = o_best + up((size_t)n_samples * 8);
     const size_t o_sum = o_cnt + up((size_t)n_samples * 4), o_dc = o_sum + up((size_t)n_samples * 32);
     const size_t o_pair = o_dc + up((size_t)n_samples * 12), total = o_pair + up((size_t)n_existing * 4);
-    cudaError_t e = ctx->merge_scratch.ensure(total);
+    cudaError_t e = ensure(ctx, ctx->merge_scratch, total);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "alloc merge workspace");
     unsigned char* b = ctx->merge_scratch.as<unsigned char>();
     cudaMemsetAsync(b + o_map, 0xff, (size_t)npix * 4, cs);
@@ -1405,7 +1406,7 @@ static gsr_status fft_lookup(gsr_ctx* ctx, int n, FftPlan* out)
             const double ang = 2.0 * 3.14159265358979323846 * (double)t / (double)n;
             h[(size_t)t] = make_float2((float)std::cos(ang), (float)-std::sin(ang));
         }
-        cudaError_t e = f.twiddles.ensure((size_t)n * sizeof(float2));
+        cudaError_t e = ensure(ctx, f.twiddles, (size_t)n * sizeof(float2));
         if (e == cudaSuccess) e = cudaMemcpy(f.twiddles.p, h.data(), (size_t)n * sizeof(float2), cudaMemcpyHostToDevice);
         if (e != cudaSuccess) {
             ctx->fft.erase(n);
@@ -1438,7 +1439,7 @@ gsr_status gsr_dft_energy(gsr_ctx* ctx, const gsr_image* images, int n_images, f
     }
     const size_t cap = std::max(kInterCap, max_need);
     const size_t acc_bytes = ((size_t)n_images * sizeof(double) + 255) & ~(size_t)255;
-    cudaError_t e = ctx->freq_scratch.ensure(acc_bytes + std::min(cap, [&] {
+    cudaError_t e = ensure(ctx, ctx->freq_scratch, acc_bytes + std::min(cap, [&] {
         size_t t = 0;
         for (size_t v : need) t += v;
         return t;

@@ -1,5 +1,7 @@
 """Device memory of recycled states: a state that has grown does not make the
-context's buffers grow again."""
+context's buffers grow again, and the kept states are given back to every call whose
+own allocation fails."""
+import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -37,3 +39,31 @@ def test_reuse_allocates_nothing():
     assert free - torch.cuda.mem_get_info()[0] < 8 * MB
     for a, b in zip(out, want):
         assert torch.equal(a, b)
+
+
+def test_kept_states_are_given_back_to_other_calls():
+    dev = P.device()
+    n = 3_000_000
+    rng = np.random.default_rng(1)
+    sc = scenes.random_scene(6, 4, [scenes.pinhole(64, 64, f=60.0)], 0)
+    params = [torch.from_numpy(np.ascontiguousarray(a, np.float32)).to(dev) for a in (
+        np.stack([rng.uniform(-1, 1, n), rng.uniform(-1, 1, n), rng.uniform(2, 6, n)], 1), np.full((n, 3), -7.0),
+        np.tile([1.0, 0.0, 0.0, 0.0], (n, 1)), np.zeros(n), np.zeros((n, 1, 3)))]
+    r = Rasterizer(sh_degree=0, device=dev)
+    r.forward(params, to_camera_views(sc.views, dev))   # (its state, about 400 MB, is destroyed and kept)
+    images = [(torch.rand(3 * 1600 * 900, device=dev), 1600, 900, 1)] * 18
+    x = torch.empty(18, device=dev)
+    r.dft_energy(images[:1], out=x[:1])                 # plans and tables
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    room = torch.cuda.mem_get_info()[0] - 96 * MB
+    block = torch.empty(room, dtype=torch.uint8, device=dev)
+    try:
+        # 18 half spectra of 17 MB do not fit beside the block
+        assert torch.cuda.mem_get_info()[0] < 18 * 17 * MB
+        r.dft_energy(images, out=x)
+        torch.cuda.synchronize()
+    finally:
+        del block
+        torch.cuda.empty_cache()
+    assert torch.equal(x, x[:1].expand(18))
