@@ -108,7 +108,7 @@ bool fft_plan(int n, FftPlan* P)
     for (int i = 0; i < k; ++i) {
         FftStage& S = P->st[i];
         S.R = radix[i]; S.Ns = Ns; S.m = n / S.R; S.step = n / (Ns * S.R);
-        S.mag_m = recip32(S.m); S.mag_ns = recip32(Ns); S.mag_r = recip32(S.R); S.pad = 0;
+        S.mag_m = recip32(S.m); S.mag_ns = recip32(Ns);
         Ns *= S.R;
     }
     return true;

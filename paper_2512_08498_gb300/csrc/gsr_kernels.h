@@ -342,10 +342,10 @@ constexpr int kFreqMaxFrames = 4096;
 
 // One Stockham pass: radix R, Ns = product of the earlier radices, m = n / R
 // butterflies per sequence, twiddle stride n / (Ns R), and multiply-high
-// reciprocals ceil(2^32 / d) of m, Ns and R (exact quotients of x < 2^16).
+// reciprocals ceil(2^32 / d) of m and Ns (exact quotients of x < 2^16).
 struct FftStage {
     int R, Ns, m, step;
-    uint32_t mag_m, mag_ns, mag_r, pad;
+    uint32_t mag_m, mag_ns;
 };
 
 // Mixed-radix Stockham plan of one transform length: passes in order and the
