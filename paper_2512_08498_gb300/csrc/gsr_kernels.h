@@ -283,6 +283,7 @@ struct BlendFwdArgs {
     uint32_t* open_blocks = nullptr;        // the same per 8x8 pixel block (bit 4 tile + block)
     uint2* tile_need = nullptr;             // with hist: [n_tiles] zeroed {largest position needed, blocks done}
     const uint32_t* depthpos = nullptr;     // with hist: record -> depth position
+    uint32_t stat_batch = 1;                // with hist: the positions' granularity (set by the launch)
     unsigned long long* hist = nullptr;     // [kSatBuckets + 1] saturation histogram, or nullptr
 };
 
@@ -305,7 +306,7 @@ struct BlendBwdArgs {
 };
 
 bool blend_supported(int tile_w, int tile_h, int batch);
-void launch_blend_fwd(const Table& T, int batch, const BlendFwdArgs& a, int num_sms, cudaStream_t s);
+void launch_blend_fwd(const Table& T, int batch, BlendFwdArgs a, int num_sms, cudaStream_t s);
 int blend_fwd_list_parts(const Table& T, bool count_pairs, int num_sms);   // LongList::parts (0: no warp form)
 size_t blend_mask_bytes(int64_t list_span, int64_t n_tiles);   // composited-entry masks of a forward's lists
 void launch_blend_bwd(const Table& T, int batch, const BlendBwdArgs& a, int num_sms, cudaStream_t s);

@@ -73,3 +73,18 @@ def test_batch_equals_its_views(tile, hot, prefix, batch):
     if prefix == 1.0:
         # the hot spot's list is longer than a resident block's share of the work
         assert (info["warp_entries_fwd"] == walked) == (hot > 0)
+
+
+@pytest.mark.parametrize("n,batch", [(20_000, 128), (60_000, 128), (60_000, 256)])   # (two rounds pay)
+def test_both_forms_choose_the_same_first_round(n, batch):
+    # the automatic fraction follows from where the pixels of each tile had stopped,
+    # in steps of the staging batch; a view twice (the warp form) has the shares of
+    # the view once (the tile form)
+    sc = _scene(n, 0, (16, 16))
+    sc.opacity_logits[:] = 4.0
+    sc.log_scales[:] = np.random.default_rng(1).uniform(-3.0, -2.0, (n, 3))
+    one = _render(sc, sc.views[:1], 0.0, batch, grads=False)[1]
+    two = _render(sc, [sc.views[0]] * 2, 0.0, batch, grads=False)[1]
+    assert one["n_tiles"] < 4096 <= two["n_tiles"]
+    assert 0.0 < one["list_prefix"] < 1.0
+    assert two["list_prefix"] == one["list_prefix"]
