@@ -119,10 +119,11 @@ __device__ __forceinline__ int mask_word(int w) { return 2 * ((w / WPR / 2) * WP
 //   tile form  the tile's eight 8x4 warps in step, a pixel per lane: twice the
 //              warps on a tile and the shorter chain per list entry.
 // The sum of the work decides for the warp form, the longest lists' chains for the
-// tile form.  So the lists choose, on the device: the warp form if the longest one has at
-// most 1 / kWarpFormShare of the instances per resident block (the kernels that
-// make the lists see it as they go).  Times of
-// the two (tile, warp form; ms) around that line, from 4096 tiles on:
+// tile form.  So the lists choose, on the device: the warp form if the longest one
+// has at most 1 / kWarpFormShare of the instances per resident block (the kernels
+// that make the lists see it as they go).  Times of the two (tile, warp form; ms)
+// around that line, by instances per resident block over longest list, from 4096
+// tiles on:
 //   share 3.9  six 1600x900 views, 1M Gaussians      2.10  1.63
 //   share 1.9  1237x701 and smaller, 32x8 tiles      0.263 0.229
 //   share 1.9  24 views of 606x348                   0.351 0.353
@@ -130,9 +131,9 @@ __device__ __forceinline__ int mask_word(int w) { return 2 * ((w / WPR / 2) * WP
 //   share 1.0  one view of 1242x995                  0.090 0.123
 //   share 0.8  24 views of 400x225, 300k             1.08  1.38
 //   share 0.2  24 views up to 994x845 of the road    1.40  2.97
-// Fewer tiles never fill the chip at that share (3840 tiles at share 2.6: 0.193
-// and 0.175; 2300 at 2.0: 0.107 and 0.114), and small images would feel the
-// second launch (the form not taken returns after 4 us).
+// With fewer tiles there is little to gain (3840 tiles at share 2.6: 0.193 and
+// 0.175; 2300 at 2.0: 0.107 and 0.114), and small images would feel the second
+// launch (the form not taken returns after 4 us).
 constexpr int64_t kWarpFormMinTiles = 4096;
 constexpr double kWarpFormShare = 1.5;
 __device__ __forceinline__ bool warp_form(const BlendFwdArgs& a) { return a.long_list && *a.long_list == 0ull; }
@@ -484,9 +485,9 @@ blend_fwd_tile_kernel(const __grid_constant__ Table Tb, BlendFwdArgs a)
 // block); the survivors' walk values are written densely to shared memory; the
 // walk evaluates each survivor at the lane's two pixels.
 //
-// Bound by instruction issue (about 90 % of the slots; DRAM idle).  Against one
+// Bound by instruction issue (88 % of the slots; DRAM 3 %).  Against one
 // pixel per lane with the tile's eight 8x4 warps in step (a barrier per 256
-// staged entries, 82 % of the slots): a record's loads, dy and the row's products
+// staged entries, 85 % of the slots for 22 % more instructions): a record's loads, dy and the row's products
 // serve two pixels, the barriers and the batch bookkeeping are gone, and a block
 // stops fetching as soon as its own pixels have stopped; it walks more idle
 // lanes (8x8 blocks composite 69 % of the walked lanes on the 1M-Gaussian
