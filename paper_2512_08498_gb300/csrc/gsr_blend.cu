@@ -879,8 +879,10 @@ blend_fwd_warp_kernel(const __grid_constant__ Table Tb, BlendFwdArgs a)
 // weights) and shifts them once per entry:
 //   sum gP dx = Mx - ux M0, sum gP dx^2 = Mxx - 2 ux Mx + ux^2 M0,
 //   sum gP dx dy = Mxy - ux My - uy Mx + ux uy M0 (and y alike).
-// The shifted form has the rounding error of the direct sums (bounded by
-// the sums of |gP| dx^2 both ways).  Per-pixel dC, dD come from s_dcd.
+// The shifts cancel: the rounding error is bounded by a few 2^-24 of the sums of
+// |gP| (|xo| + |ux|)^2 (|yo| <= 1.5 in the 8x4 block), not of |gP| dx^2; a record on
+// one corner pixel shows it (tests/test_gpu_record_sums.py).  Per-pixel dC, dD come
+// from s_dcd.
 constexpr int kSlots = 16;
 // Shared record sums: 10 floats per record at an odd stride, so lanes
 // adding to (or flushing) different records hit different banks.
