@@ -88,3 +88,38 @@ def test_both_forms_choose_the_same_first_round(n, batch):
     assert one["n_tiles"] < 4096 <= two["n_tiles"]
     assert 0.0 < one["list_prefix"] < 1.0
     assert two["list_prefix"] == one["list_prefix"]
+
+
+def test_a_replayed_graph_chooses_the_form_again():
+    # the same captured forward over even lists, over lists with a hot spot, and over
+    # even ones again, its buffers large enough for all
+    dev = P.device()
+    even, hot = _scene(9000, 6000, (16, 16)), _scene(9000, 6000, (16, 16))
+    even.means[9000:] = even.means[:6000]
+    even.log_scales[9000:] = even.log_scales[:6000]
+    r = Rasterizer(sh_degree=0, bg=even.bg, device=dev)
+    cams = to_camera_views(even.views, dev)
+    want = []
+    for sc in (even, hot):
+        params = P.params_of(sc, dev)
+        saved = r.new_saved()
+        want.append([t.clone() for t in r.forward(params, cams, saved=saved)[:3]] + [saved.info()["warp_entries_fwd"]])
+        assert saved.info()["n_tiles"] >= 4096
+    held = [t.clone() for t in P.params_of(even, dev)]
+    saved = r.new_saved()
+    assert r.lib.gsr_reserve(r.ctx, saved.h, 0, 2_000_000) == 0
+    out = r.forward(held, cams, saved=saved)[:3]
+    r.set_config(no_sync=True)
+    r.forward(held, cams, saved=saved, out=out)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        r.forward(held, cams, saved=saved, out=out)
+    for k in (0, 1, 0):
+        for h, p in zip(held, P.params_of((even, hot)[k], dev)):
+            h.copy_(p)
+        graph.replay()
+        torch.cuda.synchronize()
+        r.check(saved)
+        assert saved.info()["warp_entries_fwd"] == want[k][3]
+        for a, b in zip(out, want[k]):
+            assert torch.equal(a, b)
